@@ -333,6 +333,7 @@ __global__ void __launch_bounds__(kBatch)
     __shared__ int red[32];
     __shared__ int cut_sh, flag_sh;
     const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5, nw = blockDim.x >> 5;
+    sb.clear();
     for (int64_t t = cta_claim(head, &claim); t < nh; t = cta_claim(head, &claim)) {
         const BatchHeavy hv = htasks[t];
         const BatchInst in = insts[hv.inst];
@@ -353,10 +354,10 @@ __global__ void __launch_bounds__(kBatch)
             for (int w = tid; w < nwords; w += blockDim.x) bits[w] = 0;
             // (the first barrier of cta_products orders the clearing before every product)
             cta_products<false, SPG_SYM_UNROLL, Acc>(p0, p1, sb, in.Arow, (const Acc *)nullptr, first, seg,
-                                                     [&](int r, Acc) {
+                                                     each_product([&](int r, Acc) {
                                                          if ((uint64_t)r < (uint64_t)in.m)
                                                              set_bit_shared(bits + (r >> 5), 1u << (r & 31));
-                                                     });
+                                                     }));
             int c = 0;
             uint32_t *dst = scratch + hv.bits_off;
             for (int w = tid; w < nwords; w += blockDim.x) {
@@ -388,7 +389,7 @@ __global__ void __launch_bounds__(kBatch)
             int64_t done = 0;
             for (int w0 = 0; w0 < nwords;) {
                 const int nwin = min(kHeavyWinWords, nwords - w0);
-                const int total = cta_load_scan_bitmap(src + w0, bp, nwin, ctot);
+                const int total = cta_load_scan_words(src + w0, bp, nwin, ctot);
                 if (tid == 0) cut_sh = nwin;
                 __syncthreads();
                 if (total > kHeavyCap) {
@@ -404,14 +405,14 @@ __global__ void __launch_bounds__(kBatch)
                 const SegReg<Acc> first = cta_first_seg<Acc>(p0, p1, seg);
                 // (the first barrier of cta_products orders the zeroing before every product)
                 cta_products<true, SPG_NUM_UNROLL, Acc>(
-                    p0, p1, sb, in.Arow, (const Acc *)in.Aval, first, seg, [&](int r, Acc v) {
+                    p0, p1, sb, in.Arow, (const Acc *)in.Aval, first, seg, each_product([&](int r, Acc v) {
                         const int lr = r - rlo;
                         if ((unsigned)lr < (unsigned)span) {
                             const uint2 x = bp[lr >> 5];
                             const uint32_t sh = lr & 31;
                             if ((x.x >> sh) & 1u) acc.add((int)(x.y + __popc(x.x & ((1u << sh) - 1u))), v);
                         }
-                    });
+                    }));
                 if (done + cnt <= want) {
                     for (int i = tid; i < cnt; i += blockDim.x) out_val[cbase + done + i] = acc.get(i);
                     __syncthreads();

@@ -275,6 +275,7 @@ extern "C" spg_status spgemm_1d_multiply_host(const spg_csc *A, const spg_csc *B
     std::vector<spg_csc> Cg(G);
     for (int g = 0; g < G && !s; g++) {
         Cg[g].colptr = run.plans[g]->Ccolptr;
+        run.plans[g]->c_on_host = direct;
         if (direct) {
             Cg[g].rowidx = (char *)hri + ib * (size_t)off[g];
             Cg[g].vals = (char *)hva + 8 * (size_t)off[g];

@@ -323,7 +323,7 @@ __global__ void __launch_bounds__(kBatch)
                   const int64_t *__restrict__ capoff, const int64_t *__restrict__ cap,
                   unsigned long long *__restrict__ colfill, int32_t *flag, unsigned long long *nflag,
                   int32_t *__restrict__ item_cnt, int64_t *__restrict__ item_pos, OutIdx *__restrict__ trow,
-                  Acc *__restrict__ tval, unsigned long long *next, int64_t it_begin) {
+                  Acc *__restrict__ tval, unsigned long long *next, int64_t it_begin, int *err) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     CtaBatch<Acc> &sb = *(CtaBatch<Acc> *)smem_raw;
     unsigned char *acc_raw = smem_raw + ((sizeof(CtaBatch<Acc>) + 15) & ~(size_t)15);
@@ -333,6 +333,7 @@ __global__ void __launch_bounds__(kBatch)
     __shared__ int wsum[33];
     __shared__ long long pos_sh, claim;
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = blockDim.x >> 5;
+    sb.clear();
     for (int i = threadIdx.x; i < kFusedRows; i += blockDim.x) acc.zero(i);
     const int RW = R >> 5;
     for (int64_t li = cta_claim(next, &claim); li < nitems; li = cta_claim(next, &claim)) {
@@ -355,13 +356,21 @@ __global__ void __launch_bounds__(kBatch)
         const SegReg<Acc> first = cta_first_seg<Acc>(p0, p1, seg);
         // (the first barrier of cta_products orders this before every product)
         for (int w = threadIdx.x; w < nwords; w += blockDim.x) bits[w] = 0;
+        const uint32_t abase = acc.addr(0) - ((uint32_t)rbase << HeavyAcc<Acc>::slot_shift);
+        uint32_t *bbase = bits - (rbase >> 5);
+        bool stuck = false;
         cta_products<true, SPG_NUM_UNROLL, Acc>(
-            p0, p1, sb, At_row, At_val, first, seg,
-            [&](int r, Acc v) {
-                const int lr = (int)(r - rbase);
-                set_bit_shared(bits + (lr >> 5), 1u << (lr & 31));
-                acc.add(lr, v);
+            p0, p1, sb, At_row, At_val, first, seg, [&](const auto &r, const auto &a, const auto &b, const auto &ok) {
+                constexpr int N = sizeof(r) / sizeof(r[0]);
+                uint32_t ad[N];
+#pragma unroll
+                for (int u = 0; u < N; u++) {
+                    ad[u] = abase + ((uint32_t)r[u] << HeavyAcc<Acc>::slot_shift);
+                    if (ok[u]) set_bit_shared(bbase + (r[u] >> 5), 1u << (r[u] & 31));
+                }
+                if (!acc.add_products(ad, a, b, ok)) stuck = true;
             });
+        if (stuck) atomicOr(err, kDevErrInternal);
         const int cnt = cta_scan_popc1(bits, pre, nwords, wsum);
         if (threadIdx.x == 0) {
             long long pos = (long long)atomicAdd(colfill + j, (unsigned long long)cnt);
@@ -912,7 +921,7 @@ static spg_status learned_fused(spg_plan *p, LearnedState &L, int64_t i0, int64_
     launch(p, kern, grid_for(i1 - i0, 1, p->sm_count * occ), kBatch, smem, i1 - i0, L.it_rec0, L.it_nrec, p->rec_col,
            p->rec_slab, p->B.colptr, p->B.ptr_type == SPG_IDX_I64, p->Bq, (const Acc *)p->Bv, p->At_colptr, p->At_row,
            (const Acc *)p->At_val, p->split, p->T, p->R, L.capoff, L.cap, L.colfill, L.flag, L.nflag, L.item_cnt,
-           L.item_pos, (OutIdx *)L.trow, (Acc *)L.tval, (unsigned long long *)(p->d_cnt + kCntFusedNextSlot), i0);
+           L.item_pos, (OutIdx *)L.trow, (Acc *)L.tval, (unsigned long long *)(p->d_cnt + kCntFusedNextSlot), i0, p->d_err);
     return cuda_check(cudaGetLastError(), "fused heavy");
 }
 

@@ -8,6 +8,8 @@
 //               slab gives every present row its rank, products accumulate at
 //               acc[rank] in shared memory, and the slab is written out in row
 //               order with no sort
+#include <algorithm>
+
 #include "block_ops.cuh"
 #include "cta_products.cuh"
 #include "spg_internal.cuh"
@@ -91,6 +93,10 @@ __global__ void __launch_bounds__(WARPS * 32)
     }
 }
 
+// Slots of a numeric item's accumulator beyond its capacity: the guard slot,
+// and room to clear it 16 bytes at a time.
+constexpr int kAccPad = 4;
+
 // Everything a numeric item needs before its first product, in one record.
 struct NumItem {
     int32_t j, t0, nr, cnt, r0, pad;
@@ -122,12 +128,30 @@ __global__ void k_num_headers(int64_t nitems, const int32_t *__restrict__ num_re
 
 // One CTA per numeric item: records [r0, r0 + nr) of one heavy column (base
 // slabs t0 .. t0 + nr - 1) holding cnt <= cap entries of C.  The symbolic
-// bitmaps of the records give every present row its rank (pre[word] + popc of
-// the lower bits); products accumulate at acc[rank]; the item is then written
-// at its final place in C, values and rows each as one coalesced run.  Thread
-// 0 claims the next item when the current one starts and fetches its header
-// while the current one is written out.  MASKED: the bitmaps hold only the
-// rows an output mask admits, and a product whose row is absent is dropped.
+// bitmaps of the records give every present row its rank; products accumulate
+// in shared memory and the item is then written at its final place in C.
+//   rank items: a row's slot is its rank (cta_load_rank_table).  Slot 0 is a
+//     guard: the rank of a row counts its own bit, so entry i sits in slot
+//     i + 1, and a row missing from a bitmap (never expected) still lands
+//     inside the accumulator.  Values and rows are written each as one
+//     coalesced run.
+//   direct items: the item's rows all have a slot (nr * R <= cap, the dense
+//     items, whose 4096 entries span one slab): a row's slot is its offset,
+//     with no table look-up per product (and no conflicting look-ups: a
+//     segment's rows are distinct).
+// Thread 0 claims the next item when the current one starts and fetches its
+// header while the current one is written out.  MASKED: the bitmaps hold only
+// the rows an output mask admits, and a product whose row is absent is dropped
+// (rank items) or accumulated into a slot that is not written (direct items).
+// What bounds it: the shared-memory pipe in the walk (l1tex wavefronts 67% of
+// the whole kernel for int64, 74% for doubles on a 50,000-vertex R-MAT graph,
+// of which 8 + 9 a window are the doubles' exchange and store) and, on sparse
+// items, the barriers and latencies between an item's phases (about half of its
+// time; issue slots 52-63% busy).  Measured against the walk that placed every
+// window across segments, with 8-byte look-ups and atomicAdd(double): squaring
+// an R-MAT graph of 262,144 vertices in doubles 65.6 -> 49.3 ms, of 100,003 in
+// int64 5.4 -> 4.4 ms, one 25,000-column chunk of the similarity product (dense
+// items) 39.6 -> 26.0 ms.
 template <typename Acc, typename OutIdx, bool MASKED>
 __global__ void __launch_bounds__(kBatch, SPG_NUM_MINB)
     k_num_heavy(int64_t nitems, const NumItem *__restrict__ items, const uint32_t *__restrict__ hbits,
@@ -137,15 +161,19 @@ __global__ void __launch_bounds__(kBatch, SPG_NUM_MINB)
                 Acc *__restrict__ Cval, int *err, unsigned long long *next) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     const int RW = R >> 5;
+    constexpr int kSlotShift = HeavyAcc<Acc>::slot_shift;
     CtaBatch<Acc> &sb = *(CtaBatch<Acc> *)smem_raw;
     unsigned char *acc_raw = smem_raw + ((sizeof(CtaBatch<Acc>) + 15) & ~(size_t)15);
-    const HeavyAcc<Acc> acc(acc_raw, cap + 1);
-    uint2 *bp = (uint2 *)(acc_raw + HeavyAcc<Acc>::bytes_per_slot * (size_t)(cap + 1));  // (bitmap word, prefix)
-    __shared__ int ctot[kNumMaxWords / 32];
+    const HeavyAcc<Acc> acc(acc_raw, cap + kAccPad);
+    uint2 *tab = (uint2 *)(acc_raw + HeavyAcc<Acc>::bytes_per_slot * (size_t)(cap + kAccPad));  // rank table
+    __shared__ int ctot[kNumMaxWords / 128];
     __shared__ int bad_sh;
     __shared__ long long claim;
     __shared__ NumItem hdr;
-    const int tid = threadIdx.x;
+    const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
+    constexpr int nw = kBatch / 32;
+    const uint32_t slot0 = acc.addr(0);
+    sb.clear();
     if (tid == 0) {
         bad_sh = 0;
         const long long it = (long long)atomicAdd(next, 1ull);
@@ -173,56 +201,112 @@ __global__ void __launch_bounds__(kBatch, SPG_NUM_MINB)
         };
         const SegReg<Acc> first = cta_first_seg<Acc>(h.p0, h.p1, seg);
         const uint32_t *src = hbits + (int64_t)h.r0 * RW;
-        const int cnt = cta_load_scan_bitmap(src, bp, nwords, ctot);
+        const bool direct = nr * R <= cap;
+        const int cnt = cta_load_rank_table<kNumMaxWords / (4 * kBatch)>(src, tab, nwords, ctot);
+        const int64_t rbase = (int64_t)t0 * R;
         NumItem nh;
         if (cnt == h.cnt && cnt <= cap) {
             // (the first barrier of cta_products orders the zeroing before
             // every product)
-            for (int i = tid; i < cnt; i += blockDim.x) acc.zero(i);
-            const int wbase = t0 * RW;
+            acc.zero_all(direct ? nr * R : cnt + 1);
             bool miss = false;
-            cta_products<true, SPG_NUM_UNROLL, Acc>(
-                h.p0, h.p1, sb, At_row, At_val, first, seg,
-                [&](int r, Acc v) {
-                    const uint2 x = bp[(r >> 5) - wbase];
-                    const uint32_t sh = r & 31;
+            if (direct) {
+                const uint32_t base = slot0 - ((uint32_t)rbase << kSlotShift);
+                cta_products<true, SPG_NUM_UNROLL, Acc>(
+                    h.p0, h.p1, sb, At_row, At_val, first, seg,
+                    [&](const auto &r, const auto &a, const auto &b, const auto &ok) {
+                        constexpr int N = sizeof(r) / sizeof(r[0]);
+                        uint32_t ad[N];
+#pragma unroll
+                        for (int u = 0; u < N; u++) {
+                            ad[u] = base + ((uint32_t)r[u] << kSlotShift);
 #if SPG_CHECK_MEMBERSHIP
-                    // a row missing from the symbolic bitmap (never expected) goes
-                    // to the dump slot acc[cap] and is reported
-                    const bool hit = (x.x >> sh) & 1u;
-                    miss |= !hit && !MASKED;  // a masked product is absent by design
-                    acc.add(hit ? (int)(x.y + __popc(x.x & ((1u << sh) - 1u))) : cap, v);
-#else
-                    if constexpr (MASKED) {
-                        if ((x.x >> sh) & 1u) acc.add((int)(x.y + __popc(x.x & ((1u << sh) - 1u))), v);
-                    } else {
-                        // the rank of a present row; an absent one would still
-                        // land inside [0, cnt] (never outside the accumulator)
-                        acc.add((int)(x.y + __popc(x.x & ((1u << sh) - 1u))), v);
-                    }
+                            if (ok[u]) miss |= !MASKED && !((rank_word(tab[(r[u] - (int)rbase) >> 5]) >> (r[u] & 31)) & 1u);
 #endif
-                });
+                        }
+                        if (!acc.add_products(ad, a, b, ok)) miss = true;
+                    });
+            } else {
+                const uint32_t *ranks = (const uint32_t *)tab - 2 * t0 * RW;
+                cta_products<true, SPG_NUM_UNROLL, Acc>(
+                    h.p0, h.p1, sb, At_row, At_val, first, seg,
+                    [&](const auto &r, const auto &a, const auto &b, const auto &ok) {
+                        constexpr int N = sizeof(r) / sizeof(r[0]);
+                        uint32_t ad[N];
+                        bool keep[N];
+#pragma unroll
+                        for (int u = 0; u < N; u++) {
+                            ad[u] = slot0;
+                            keep[u] = ok[u];
+                            if (ok[u]) {
+                                const uint32_t e = ranks[r[u] >> 4];
+                                const uint32_t upto = rank_upto(e, r[u]);
+                                ad[u] = acc.addr(rank1(e, upto));
+                                if constexpr (MASKED) {
+                                    keep[u] = (int)upto < 0;  // the row's own bit
+                                } else {
+#if SPG_CHECK_MEMBERSHIP
+                                    // a row missing from the symbolic bitmap
+                                    // goes to the guard slot and is reported
+                                    if ((int)upto >= 0) {
+                                        miss = true;
+                                        ad[u] = slot0;
+                                    }
+#endif
+                                }
+                            }
+                        }
+                        if (!acc.add_products(ad, a, b, keep)) miss = true;
+                    });
+            }
             if (miss) bad_sh = 1;
             if (tid == 0 && (long long)nxt < nitems) nh = items[nxt];
-            // cta_products ends with a barrier: acc is complete
-            for (int i = tid; i < cnt; i += blockDim.x) st_stream(Cval + h.cbase + i, acc.get(i));
-            __syncthreads();
-            // the row ids go to shared memory by rank first (over the consumed
-            // values: cnt ints fit in the first cnt slots), then to C in one
-            // coalesced run
-            int32_t *srow = acc.scratch32();
-            for (int w = tid; w < nwords; w += blockDim.x) {
-                uint32_t word = bp[w].x;
-                int pos = (int)bp[w].y;
-                while (word) {
-                    int bb = __ffs(word) - 1;
-                    srow[pos++] = w * 32 + bb;
-                    word &= word - 1u;
+            // cta_products ends with a barrier: acc is complete.  The writing
+            // threads start so that every warp writes whole aligned lines of C
+            // (a warp's 32 row ids are one 128-byte line, its values two): over
+            // the CPU-GPU link a line written in parts crosses in parts.
+            Acc *cval = Cval + h.cbase;
+            OutIdx *crow = Crow + h.cbase;
+            const int v0 = tid - (int)(((uintptr_t)cval / sizeof(Acc)) & 31);
+            const int r0 = tid - (int)(((uintptr_t)crow / sizeof(OutIdx)) & 31);
+            if (direct) {
+                // the rows by rank (16-bit offsets behind the item's words:
+                // tab holds kNumMaxWords words and a direct item needs
+                // nr * R / 32 of them), then values and rows as coalesced runs
+                uint16_t *srow = (uint16_t *)(tab + nwords);
+                for (int w = wid; w < nwords; w += nw) {
+                    const uint2 e = tab[w];
+                    const uint32_t word = rank_word(e);
+                    if ((word >> lane) & 1u)
+                        srow[rank_before(e) + __popc(word & ((1u << lane) - 1u))] = (uint16_t)(w * 32 + lane);
                 }
+                __syncthreads();
+                for (int i = v0; i < cnt; i += kBatch)
+                    if (i >= 0) st_stream(cval + i, acc.get(srow[i]));
+                for (int i = r0; i < cnt; i += kBatch)
+                    if (i >= 0) st_stream(crow + i, (OutIdx)(rbase + srow[i]));
+            } else {
+                for (int i = v0; i < cnt; i += kBatch)
+                    if (i >= 0) st_stream(cval + i, acc.get(i + 1));
+                __syncthreads();
+                // the row ids go to shared memory by rank first (over the
+                // consumed values: cnt ints fit in the first cnt slots), then
+                // to C in one coalesced run
+                int32_t *srow = acc.scratch32();
+                for (int w = tid; w < nwords; w += kBatch) {
+                    const uint2 e = tab[w];
+                    uint32_t word = rank_word(e);
+                    int pos = rank_before(e);
+                    while (word) {
+                        int bb = __ffs(word) - 1;
+                        srow[pos++] = w * 32 + bb;
+                        word &= word - 1u;
+                    }
+                }
+                __syncthreads();
+                for (int i = r0; i < cnt; i += kBatch)
+                    if (i >= 0) st_stream(crow + i, (OutIdx)(rbase + srow[i]));
             }
-            __syncthreads();
-            const int64_t rbase = (int64_t)t0 * R;
-            for (int i = tid; i < cnt; i += blockDim.x) st_stream(Crow + h.cbase + i, (OutIdx)(rbase + srow[i]));
         } else {
             // the item's room in C was sized from the record counts: never
             // write past it
@@ -298,13 +382,20 @@ static spg_status numeric_typed(spg_plan *p, spg_csc *C) {
     if (s) return s;
     if (p->nnum > 0) {
         const int threads = kBatch;
-        size_t smem = ((sizeof(CtaBatch<Acc>) + 15) & ~(size_t)15) + sizeof(Acc) * (size_t)(p->num_cap + 1) +
+        size_t smem = ((sizeof(CtaBatch<Acc>) + 15) & ~(size_t)15) + sizeof(Acc) * (size_t)(p->num_cap + kAccPad) +
                       sizeof(uint2) * (size_t)kNumMaxWords;
         auto kern = p->omask.bits ? k_num_heavy<Acc, OutIdx, true> : k_num_heavy<Acc, OutIdx, false>;
         cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         int occ = 1;
         cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kern, threads, smem);
         if (occ < 1) occ = 1;
+        // C in host memory: as many CTAs per SM as keep up with the link (one
+        // per four products of an entry of C); more of them write over a wider
+        // range at once, which the link answers with less bandwidth (40,009
+        // vertices, 1.6 GB of C, four groups: 15.4 ms at four CTAs per SM,
+        // 14.6 at two, 14.3 at one, 14.8 at 3/4)
+        if (p->c_on_host)
+            occ = (int)std::max<int64_t>(1, std::min<int64_t>(occ, p->stats.products / 4 / std::max<int64_t>(p->nnzC, 1)));
         int g = grid_for(p->nnum, 1, p->sm_count * occ);
         if (!p->num_items) p->num_items = ws_alloc(p, sizeof(NumItem) * (size_t)p->nnum);
         NumItem *items = (NumItem *)p->num_items;

@@ -149,6 +149,7 @@ struct spg_plan {
     std::vector<int64_t> bounds_h;   // the bounds in effect (P + 1), host
     int64_t *blk = nullptr;          // per block: flops, gathered A~ nonzeros, of them fetched (3 x P)
     int64_t *gshift = nullptr;       // per A~ column: its entries' offset into A (gather)
+    bool c_on_host = false;          // the numeric pass stores C into host memory
     bool numeric_done = false;       // a numeric pass ran: the light lists and item headers exist
     cudaGraph_t graph = nullptr;     // captured refresh + numeric (spgemm_plan_capture)
     cudaGraphExec_t graph_exec = nullptr;
@@ -435,7 +436,12 @@ __device__ __forceinline__ void set_bit_shared(uint32_t *word, uint32_t mask) {
 #endif
 // threads of a heavy-bin CTA = B' entries staged per round by cta_products
 constexpr int kBatch = SPG_HEAVY_THREADS;
-constexpr int kLongSeg = 32;  // segments this long are walked 32 entries per warp step
+// cta_products: segments from kMidSeg entries on are walked by steps of their
+// own, those below kLongSeg always through the windows of the staging area,
+// those between as far as the windows go.
+constexpr int kLongSeg = 32;
+constexpr int kMidSeg = 256;
+constexpr int kShortWindows = (kBatch * (kLongSeg - 1) + 31) / 32;
 
 __device__ __forceinline__ unsigned hash_row(int r, int shift) {
     return ((unsigned)r * 0x9E3779B1u) >> shift;

@@ -126,6 +126,7 @@ __global__ void SPG_SYM_BOUNDS
     __shared__ long long claim;
     __shared__ int hubs[kSymMaxHubs];
     __shared__ int nhub;
+    sb.clear();
     if (threadIdx.x == 0) nhub = 0;
     for (int64_t it = cta_claim(next, &claim); it < nitems; it = cta_claim(next, &claim)) {
         const int r0 = sym_rec0[it], nr = sym_nrec[it];
@@ -163,13 +164,12 @@ __global__ void SPG_SYM_BOUNDS
         // again and again, so read before the atomic
         const bool dense = flops[j] > 4 * (int64_t)(win_hi[j] - win_lo[j] + 1);
         cta_products<false, SPG_SYM_UNROLL, long long>(
-            p0, p1, sb, At_row, (const long long *)nullptr, first, seg,
-            [&](int r, long long) {
+            p0, p1, sb, At_row, (const long long *)nullptr, first, seg, each_product([&](int r, long long) {
                 if (dense)
                     set_bit_shared(bits + ((r >> 5) - wbase), 1u << (r & 31));
                 else
                     atomicOr(bits + ((r >> 5) - wbase), 1u << (r & 31));
-            });
+            }));
         // cta_products ends with a barrier: the walked products are marked;
         // now the hub segments, each thread ORing the words it owns (the rows
         // of the item are words [t0 * RW, t0 * RW + nwords) of a hub bitmap;

@@ -1,0 +1,92 @@
+"""The heavy columns' product walk and accumulator at their edges: segment
+lengths around the length classes (31 | 32, 255 | 256), columns of B around the
+staging batch (256 entries) and with more middle-length segments than the
+windows hold, items whose rows all have a slot (dense) and items addressed by
+rank (sparse), many products of one row at once, NaN and infinities.  Doubles
+within the result contract's 1e-12 * sum |a b|, integers exactly."""
+import numpy as np
+import pytest
+import torch
+
+import oracle
+import paper_2408_14558_gb300 as g
+import synth
+from parity import assert_full_parity, run_gpu
+
+pytestmark = pytest.mark.gpu
+
+
+def columns(lens, m, rng, values, window=None):
+    """m-row matrix whose column c holds lens[c] distinct rows (drawn below `window`)."""
+    w = m if window is None else window
+    cols = np.repeat(np.arange(len(lens)), lens)
+    rows = np.concatenate([np.sort(rng.choice(w, n, replace=False)) for n in lens])
+    vals = rng.uniform(-1, 1, rows.size) if values == "f64" else rng.integers(-2**62, 2**62, rows.size)
+    return synth._csc_from_sorted(m, len(lens), cols, rows, vals)
+
+
+SHAPES = {
+    # name: (segment lengths of A's columns, entries of every column of B, rows of A)
+    "short_31": ([31] * 300, [255, 256, 257, 300], 20000),
+    "mid_32_255": ([32, 255] * 130, [256, 260, 129], 60000),
+    "mids_past_the_windows": ([200] * 256 + [5] * 64 + [700] * 8, [328, 300, 256], 70000),
+    "long_256_3000": ([256, 257, 3000, 1] * 60, [240, 64, 63], 100000),
+    "one_each": ([1, 31, 32, 33, 127, 128, 129, 255, 256, 257, 511, 1000], [12, 11, 5], 30000),
+    "dense_item": ([31, 32, 500, 1000] * 70, [280, 256, 9], 1024),
+    "dense_item_ragged": ([7, 300, 64] * 90, [270, 13], 3001),
+}
+
+
+@pytest.mark.parametrize("values", ["f64", "i64"])
+@pytest.mark.parametrize("shape", sorted(SHAPES))
+def test_walk_edges_match_oracle(shape, values):
+    lens, nb, m = SHAPES[shape]
+    rng = np.random.default_rng(11)
+    A = columns(lens, m, rng, values)
+    B = columns(nb, len(lens), rng, values)
+    for R in (1024, 4096):
+        C = run_gpu(A, B, 2, 64, light_max=32, slab_rows=R)
+        assert_full_parity(C, oracle.spgemm(A, B), f"{shape} {values} R={R}")
+
+
+@pytest.mark.parametrize("m,window", [(5000, 40), (90000, 90000)])
+def test_many_products_of_one_row(m, window):
+    """Every column of A holds the same few rows (all warps add to the same
+    slots), in a dense and in a rank-addressed item."""
+    rng = np.random.default_rng(12)
+    if window < m:
+        A = columns([33] * 900, m, rng, "f64", window=window)
+    else:
+        rows = np.sort(rng.choice(m, 40, replace=False))
+        A = synth._csc_from_sorted(m, 900, np.repeat(np.arange(900), 40), np.tile(rows, 900),
+                                   rng.uniform(-1, 1, 36000))
+    B = columns([900, 899, 257], 900, rng, "f64")
+    assert_full_parity(run_gpu(A, B, 1, 64, light_max=32, slab_rows=1024), oracle.spgemm(A, B), "one row")
+
+
+def test_nan_and_infinities_stay_where_they_belong():
+    rng = np.random.default_rng(13)
+    A = columns([40, 300, 31] * 40, 6000, rng, "f64")
+    B = columns([120, 100], 120, rng, "f64")
+    A.vals[::97] = np.inf
+    A.vals[5::101] = np.nan
+    # a signalling NaN among the inputs
+    A.vals.view(np.uint64)[7::103] = 0x7FF4A5C300000000
+    C = run_gpu(A, B, 1, 64, light_max=32, slab_rows=1024)
+    cp, ri, v = C.to_host()
+    dense = np.zeros((6000, 120))
+    dense[A.rowidx, np.repeat(np.arange(120), np.diff(A.colptr))] = A.vals
+    for j in range(2):
+        want = np.zeros(6000)
+        ks, bv = B.col(j)
+        with np.errstate(invalid="ignore"):
+            for k, x in zip(ks, bv):
+                r, a = A.col(int(k))
+                want[r] += a * x
+        got = v[cp[j]:cp[j + 1]]
+        want = want[ri[cp[j]:cp[j + 1]]]
+        assert np.array_equal(np.isnan(got), np.isnan(want)) and np.array_equal(np.isinf(got), np.isinf(want))
+        fine = np.isfinite(want)
+        mag = sum(np.abs(np.where(np.isfinite(dense[:, k]), dense[:, k], 0.0) * x) for k, x in zip(ks, bv))
+        assert np.all(np.abs(got[fine] - want[fine]) <= 1e-12 * mag[ri[cp[j]:cp[j + 1]]][fine])
+        assert np.array_equal(got[np.isinf(want)], want[np.isinf(want)])
