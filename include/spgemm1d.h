@@ -181,8 +181,7 @@ spg_status spgemm_symbolic(spg_plan *plan, void *C_colptr, int64_t *nnzC);
  * spgemm_symbolic (int64, n + 1), C->rowidx room for nnzC entries of the
  * inputs' idx_type and C->vals room for nnzC doubles (double inputs) or int64
  * (integer inputs).  C's size fields and type codes are set by this call.
- * The first call for a plan synchronises the stream once (the sizes of the
- * light columns' bins are read back); otherwise stream-ordered.
+ * Stream-ordered.
  */
 spg_status spgemm_numeric(spg_plan *plan, spg_csc *C);
 

@@ -135,15 +135,10 @@ extern "C" spg_status spgemm_plan_replay(spg_plan *p) {
     return cuda_check(cudaGraphLaunch(p->graph_exec, p->st), "graph launch");
 }
 
-extern "C" spg_status spgemm_plan_stats(const spg_plan *pc, spg_stats *st) {
-    clear_error();
-    if (!pc || !st) {
-        set_error("plan and stats must not be NULL");
-        return SPG_INVALID_ARGUMENT;
-    }
-    spg_plan *p = const_cast<spg_plan *>(pc);
-    spg_status s = cuda_check(cudaStreamSynchronize(p->st), "stats sync");
-    if (s) return s;
+void spg::collect_stats(spg_plan *p, spg_stats *st) {
+    float plan_ms = 0;
+    if (cudaEventElapsedTime(&plan_ms, p->ev[0], p->ev[1]) == cudaSuccess) p->stats.ms_plan = plan_ms;
+    cudaGetLastError();
     if (p->symbolic_done) {
         float ms = 0;
         if (cudaEventQuery(p->ev[5]) == cudaSuccess && cudaEventElapsedTime(&ms, p->ev[4], p->ev[5]) == cudaSuccess)
@@ -160,6 +155,18 @@ extern "C" spg_status spgemm_plan_stats(const spg_plan *pc, spg_stats *st) {
     }
     p->stats.kernel_launches = p->launches;
     *st = p->stats;
+}
+
+extern "C" spg_status spgemm_plan_stats(const spg_plan *pc, spg_stats *st) {
+    clear_error();
+    if (!pc || !st) {
+        set_error("plan and stats must not be NULL");
+        return SPG_INVALID_ARGUMENT;
+    }
+    spg_plan *p = const_cast<spg_plan *>(pc);
+    spg_status s = cuda_check(cudaStreamSynchronize(p->st), "stats sync");
+    if (s) return s;
+    collect_stats(p, st);
     return read_dev_err(p, "stats");
 }
 
@@ -225,7 +232,8 @@ extern "C" spg_status spgemm_1d_multiply(const spg_csc *A, const spg_csc *B, con
         return s;
     }
     spg_stats st{};
-    if (spgemm_plan_stats(p, &st) == SPG_OK) remember_multiply_stats(st);
+    collect_stats(p, &st);
+    remember_multiply_stats(st);
     spgemm_plan_destroy(p);
     return SPG_OK;
 }

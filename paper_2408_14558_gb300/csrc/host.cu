@@ -263,9 +263,7 @@ extern "C" spg_status spgemm_1d_multiply_host(const spg_csc *A, const spg_csc *B
     S.nnzB = B->nnz;
     S.P = opt->P;
     S.b = opt->b;
-    // every group's numeric set-up (it reads bin sizes back: done before any
-    // copy of C occupies the copy engine) and every group's C first
-    for (int g = 0; g < G && !s; g++) s = prepare_numeric(run.plans[g]);
+    // every group's C first
     // direct: the numeric kernels store C's rows and values straight into the
     // host arrays (page-locked memory the GPU addresses with the same
     // pointers), with no device copy of C and no copy engine; otherwise each

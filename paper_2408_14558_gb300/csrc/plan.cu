@@ -9,6 +9,7 @@
 //                    column its place in D~ (Algorithm 1, D~ = H_i AND D)
 //   k_dtilde         the ascending list D~_i
 //   k_fetch          Algorithm 2 with groups of b consecutive column ids
+//   k_block_dt       each block's range of D~
 //   k_gather_len / k_gather_shift / k_gather_copy   A~_i = A(:, D~_i) for all
 //                    blocks in one entry-balanced copy (on one GPU the chosen
 //                    fetch blocks only give the volume Algorithm 2 transfers)
@@ -112,17 +113,7 @@ int grid_for(int64_t work, int per_block, int max_blocks) {
     return (int)g;
 }
 
-spg_status read_dev_err(spg_plan *p, const char *phase) {
-    // the error word lands in the last pinned slot so that other read-backs
-    // queued before this call stay intact
-    int64_t *slot = p->h_pinned + 63;
-    *slot = 0;
-    spg_status s = cuda_check(
-        cudaMemcpyAsync(slot, p->d_err, sizeof(int), cudaMemcpyDeviceToHost, p->st), phase);
-    if (s) return s;
-    s = cuda_check(cudaStreamSynchronize(p->st), phase);
-    if (s) return s;
-    int e = *(int *)slot;
+static spg_status dev_err_status(int e, const char *phase) {
     if (e & kDevErrInput) {
         set_error("%s: input matrix is not canonical CSC (colptr not monotone, or a row id out of range, unsorted or repeated)", phase);
         return SPG_INVALID_INPUT;
@@ -136,6 +127,24 @@ spg_status read_dev_err(spg_plan *p, const char *phase) {
         return SPG_CUDA_ERROR;
     }
     return SPG_OK;
+}
+
+// The error word lands in the last pinned slot, so that it can ride along with
+// other read-backs: dev_err_queue, then (once the stream is synchronised)
+// dev_err_read.
+spg_status dev_err_queue(spg_plan *p, const char *phase) {
+    p->h_pinned[kPinnedErr] = 0;
+    return cuda_check(cudaMemcpyAsync(p->h_pinned + kPinnedErr, p->d_err, sizeof(int), cudaMemcpyDeviceToHost, p->st),
+                      phase);
+}
+spg_status dev_err_read(spg_plan *p, const char *phase) {
+    return dev_err_status(*(int *)(p->h_pinned + kPinnedErr), phase);
+}
+
+spg_status read_dev_err(spg_plan *p, const char *phase) {
+    spg_status s = dev_err_queue(p, phase);
+    if (!s) s = cuda_check(cudaStreamSynchronize(p->st), phase);
+    return s ? s : dev_err_read(p, phase);
 }
 
 // ------------------------------------------------------------------ kernels
@@ -154,36 +163,70 @@ enum {
     kCntSlots = 24
 };
 
-// Input checks, in two passes that read the matrix once, coalesced.
+// Input checks, in two passes that read each matrix once, coalesced; blockIdx.y
+// picks the matrix (A, or B when it is another one).
 // Per column: 0 <= colptr[j] <= colptr[j+1] <= nnz, colptr[0] = 0 and
 // colptr[ncols] = nnz; the first entry of every non-empty column is marked in
 // `starts` (one bit per entry, zeroed by the caller).
-__global__ void k_validate_cols(const void *colptr, int p64, int64_t ncols, int64_t nnz, uint32_t *starts,
-                                int *err) {
+struct ValidateArg {
+    const void *colptr, *rowidx;
+    int p64, i64;
+    int64_t ncols, nnz, nrows;
+    uint32_t *starts;
+};
+struct ValidateArgs {
+    ValidateArg m[2];
+};
+
+__global__ void k_validate_cols(ValidateArgs args, int *err) {
+    const ValidateArg &v = args.m[blockIdx.y];
     const int64_t t0 = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (t0 == 0 && (ld_ptr(colptr, p64, 0) != 0 || ld_ptr(colptr, p64, ncols) != nnz)) atomicOr(err, kDevErrInput);
-    for (int64_t j = t0; j < ncols; j += (int64_t)gridDim.x * blockDim.x) {
-        const int64_t s = ld_ptr(colptr, p64, j), e = ld_ptr(colptr, p64, j + 1);
-        if (s > e || s < 0 || e > nnz)
+    if (t0 == 0 && (ld_ptr(v.colptr, v.p64, 0) != 0 || ld_ptr(v.colptr, v.p64, v.ncols) != v.nnz))
+        atomicOr(err, kDevErrInput);
+    for (int64_t j = t0; j < v.ncols; j += (int64_t)gridDim.x * blockDim.x) {
+        const int64_t s = ld_ptr(v.colptr, v.p64, j), e = ld_ptr(v.colptr, v.p64, j + 1);
+        if (s > e || s < 0 || e > v.nnz)
             atomicOr(err, kDevErrInput);
         else if (s < e)
-            atomicOr(starts + (s >> 5), 1u << (s & 31));
+            atomicOr(v.starts + (s >> 5), 1u << (s & 31));
     }
 }
 
 // Per entry: 0 <= row < nrows, and rows strictly increase inside a column: a
-// row not above its predecessor is allowed only where a column starts.
-__global__ void k_validate_rows(const void *rowidx, int i64, int64_t nnz, int64_t nrows,
-                                const uint32_t *__restrict__ starts, int *err) {
+// row not above its predecessor is allowed only where a column starts.  A
+// thread takes four consecutive entries (one 16-byte load when the row ids are
+// int32 and aligned: 14.6M entries took 75 us at one entry per thread).
+__global__ void k_validate_rows(ValidateArgs args, int *err) {
+    const ValidateArg &v = args.m[blockIdx.y];
+    const bool vec = !v.i64 && ((uintptr_t)v.rowidx & 15) == 0;
     bool bad = false;
-    for (int64_t q = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; q < nnz; q += (int64_t)gridDim.x * blockDim.x) {
-        const int64_t r = ld_ptr(rowidx, i64, q);
-        if (r < 0 || r >= nrows)
-            bad = true;
-        else if (q > 0 && ld_ptr(rowidx, i64, q - 1) >= r && !((starts[q >> 5] >> (q & 31)) & 1u))
-            bad = true;
+    const int64_t n4 = (v.nnz + 3) >> 2;
+    for (int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; t < n4; t += (int64_t)gridDim.x * blockDim.x) {
+        const int64_t q = t * 4;
+        const int n = (int)min((int64_t)4, v.nnz - q);
+        int64_t r[4], prev = q > 0 ? ld_ptr(v.rowidx, v.i64, q - 1) : -1;
+        if (vec && n == 4) {
+            const int4 x = __ldg((const int4 *)v.rowidx + t);
+            r[0] = x.x;
+            r[1] = x.y;
+            r[2] = x.z;
+            r[3] = x.w;
+        } else {
+#pragma unroll
+            for (int u = 0; u < 4; u++) r[u] = u < n ? ld_ptr(v.rowidx, v.i64, q + u) : 0;
+        }
+        const uint32_t first = v.starts[q >> 5] >> (q & 31);  // (q is a multiple of 4: all four bits are here)
+#pragma unroll
+        for (int u = 0; u < 4; u++)
+            if (u < n) {
+                if (r[u] < 0 || r[u] >= v.nrows)
+                    bad = true;
+                else if (q + u > 0 && prev >= r[u] && !((first >> u) & 1u))
+                    bad = true;
+                prev = r[u];
+            }
     }
-    if (__any_sync(kFull, bad) && (threadIdx.x & 31) == 0) atomicOr(err, kDevErrInput);
+    if (bad) atomicOr(err, kDevErrInput);
 }
 
 __global__ void k_nonempty_bits(const void *colptr, int p64, int64_t k, int64_t W, uint32_t *D) {
@@ -281,10 +324,13 @@ __device__ __forceinline__ int block_of_entry(int64_t q, const int64_t *__restri
 }
 
 // H_i: one atomicOr per entry of B into its block's bitmap (entry-parallel).
-__global__ void k_mark_H(const void *rowidx, int i64, int64_t nnz, int P, int64_t W, uint32_t *H,
+// It runs before the host has read the validation's result: a row outside
+// [0, k) is skipped.
+__global__ void k_mark_H(const void *rowidx, int i64, int64_t nnz, int P, int64_t k, int64_t W, uint32_t *H,
                          const int64_t *__restrict__ eoff) {
     for (int64_t q = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; q < nnz; q += (int64_t)gridDim.x * blockDim.x) {
         const int64_t r = ld_ptr(rowidx, i64, q);
+        if ((uint64_t)r >= (uint64_t)k) continue;
         const int i = block_of_entry(q, eoff, P);
         atomicOr(H + (int64_t)i * W + (r >> 5), 1u << (r & 31));
     }
@@ -354,49 +400,85 @@ __global__ void k_fetch(const uint32_t *H, const uint32_t *D, const int64_t *ran
     }
 }
 
-// Length of every A~ column, the longest, and the entries whose column lies
-// outside the block's own column range [floor(i*k/P), floor((i+1)*k/P)) of A
-// (what a distributed run fetches from other owners); dt_base (P + 1) gives
-// each block's range of D~ entries.
-__global__ void k_gather_len(const int32_t *dtilde, int64_t ndt, const void *Acolptr, int p64,
-                             int64_t *len, long long *maxlen, const int64_t *dt_base, int P, int64_t k,
-                             long long *remote, long long *blk_gathered, long long *blk_remote) {
+// First index in D~ of every block (P + 1).
+__global__ void k_block_dt(const int64_t *rankpre, int64_t W, int P, int64_t *dt_base) {
+    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i <= P; i += gridDim.x * blockDim.x)
+        dt_base[i] = rankpre[(int64_t)i * W];
+}
+
+// Length of every A~ column (0 for [|D~|, n): the caller may not know |D~| =
+// dt_base[P] yet), the longest, and the entries whose column lies outside the
+// block's own column range [floor(i*k/P), floor((i+1)*k/P)) of A (what a
+// distributed run fetches from other owners); dt_base (P + 1) gives each
+// block's range of D~ entries.  A CTA takes a run of consecutive columns, which
+// meets a block or two, and sums per block in shared memory (up to
+// kGatherLenBlocks blocks; the bounds sit there too): an atomic per warp on the
+// blocks' sums took 60 us for 2.1M columns of 32 blocks.
+constexpr int kGatherLenBlocks = 512;
+
+__global__ void __launch_bounds__(256)
+    k_gather_len(const int32_t *dtilde, int64_t n, const void *Acolptr, int p64, int64_t *len, long long *maxlen,
+                 const int64_t *dt_base, int P, int64_t k, long long *remote, long long *blk_gathered,
+                 long long *blk_remote) {
+    __shared__ int64_t dts[kGatherLenBlocks + 1], own[kGatherLenBlocks + 1];
+    __shared__ unsigned long long sum_all[kGatherLenBlocks], sum_rem[kGatherLenBlocks];
+    const bool in_shared = P <= kGatherLenBlocks;
+    if (in_shared)
+        for (int i = threadIdx.x; i <= P; i += blockDim.x) {
+            dts[i] = dt_base[i];
+            own[i] = (int64_t)i * k / P;
+            if (i < P) sum_all[i] = sum_rem[i] = 0;
+        }
+    __syncthreads();
+    unsigned long long *to_all = in_shared ? sum_all : (unsigned long long *)blk_gathered;
+    unsigned long long *to_rem = in_shared ? sum_rem : (unsigned long long *)blk_remote;
+    const int64_t *dt = in_shared ? dts : dt_base;
     const int lane = threadIdx.x & 31;
+    const int64_t ndt = dt[P];
     long long mx = 0, rem = 0;
-    for (int64_t base = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) & ~(int64_t)31; base < ndt;
-         base += (int64_t)gridDim.x * blockDim.x) {
+    const int64_t per = (n + gridDim.x - 1) / gridDim.x;
+    const int64_t g1 = min(n, (blockIdx.x + 1) * per);
+    for (int64_t base = blockIdx.x * per + (threadIdx.x & ~31); base < g1; base += blockDim.x) {
         const int64_t g = base + lane;
-        const bool valid = g < ndt;
+        const bool valid = g < min(g1, ndt);
         long long l = 0, lr = 0;
         int lo = -1;
         if (valid) {
             const int64_t h = dtilde[g];
             l = ld_ptr(Acolptr, p64, h + 1) - ld_ptr(Acolptr, p64, h);
-            len[g] = l;
             mx = max(mx, l);
             lo = 0;
-            int hi = P;  // the block i with dt_base[i] <= g < dt_base[i + 1]
+            int hi = P;  // the block i with dt[i] <= g < dt[i + 1]
             while (hi - lo > 1) {
                 const int mid = (lo + hi) >> 1;
-                if (dt_base[mid] <= g)
+                if (dt[mid] <= g)
                     lo = mid;
                 else
                     hi = mid;
             }
-            if (h < (int64_t)lo * k / P || h >= (int64_t)(lo + 1) * k / P) lr = l;
+            const int64_t o0 = in_shared ? own[lo] : (int64_t)lo * k / P;
+            const int64_t o1 = in_shared ? own[lo + 1] : (int64_t)(lo + 1) * k / P;
+            if (h < o0 || h >= o1) lr = l;
             rem += lr;
         }
+        if (g < g1) len[g] = l;
         // per-block sums, one atomic per warp when its entries share a block
         const int b0 = __shfl_sync(kFull, lo, 0);
         if (__all_sync(kFull, !valid || lo == b0)) {
             const long long tl = warp_sum_ll(l), tr = warp_sum_ll(lr);
-            if (lane == 0 && tl) atomicAdd((unsigned long long *)(blk_gathered + b0), (unsigned long long)tl);
-            if (lane == 0 && tr) atomicAdd((unsigned long long *)(blk_remote + b0), (unsigned long long)tr);
+            if (lane == 0 && tl) atomicAdd(to_all + b0, (unsigned long long)tl);
+            if (lane == 0 && tr) atomicAdd(to_rem + b0, (unsigned long long)tr);
         } else if (valid) {
-            if (l) atomicAdd((unsigned long long *)(blk_gathered + lo), (unsigned long long)l);
-            if (lr) atomicAdd((unsigned long long *)(blk_remote + lo), (unsigned long long)lr);
+            if (l) atomicAdd(to_all + lo, (unsigned long long)l);
+            if (lr) atomicAdd(to_rem + lo, (unsigned long long)lr);
         }
     }
+    __syncthreads();
+    if (in_shared)
+        for (int i = threadIdx.x; i < P; i += blockDim.x) {
+            if (sum_all[i]) atomicAdd((unsigned long long *)(blk_gathered + i), sum_all[i]);
+            if (sum_rem[i]) atomicAdd((unsigned long long *)(blk_remote + i), sum_rem[i]);
+        }
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) {
         mx = max(mx, __shfl_xor_sync(kFull, mx, o));
@@ -514,8 +596,15 @@ __device__ __forceinline__ int light_bin(long long U, int light_max) {
     return bin;
 }
 
-// Warp per output column: flops_j, the row window of its products, the MLP
-// features and the symbolic bin (bound U = min(flops_j, window)).
+// Per output column: flops_j, the row window of its products, the MLP features
+// and the symbolic bin (bound U = min(flops_j, window)).  A warp takes four
+// columns, eight lanes each with four entries in flight per lane; a column of
+// more than kStatsLong entries is done by the whole warp afterwards.  (A warp
+// per column: 262,144 columns of 8 entries 85 us, of 32 entries 140 us, most
+// lanes or loads idle; 16 lanes per column whatever its length: a skewed graph
+// of 100,003 columns 170 us instead of 97.)
+constexpr int kStatsLong = 64;
+
 __global__ void k_col_stats(const void *Bcolptr, int p64, int64_t n, const int32_t *Bq,
                             const int64_t *At_colptr, const int32_t *At_row, int light_max,
                             int64_t *flops, int32_t *win_lo, int32_t *win_hi, int32_t *nnzb,
@@ -525,21 +614,24 @@ __global__ void k_col_stats(const void *Bcolptr, int p64, int64_t n, const int32
     if (threadIdx.x < kNumBins) hist[threadIdx.x] = 0;
     if (threadIdx.x == 0) prod_sh = 0;
     __syncthreads();
-    int lane = threadIdx.x & 31;
-    int64_t warp = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
+    const int lane = threadIdx.x & 31, gl = lane & 7;
+    const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
     long long prod_local = 0;
-    for (int64_t j = warp; j < n; j += nwarps) {
-        int64_t s = ld_ptr(Bcolptr, p64, j), e = ld_ptr(Bcolptr, p64, j + 1);
-        long long fl = 0;
-        int mx = 0, lo = INT32_MAX, hi = -1;
-        // four entries per lane and step, each stage's loads issued together
-        // (long columns of B would otherwise be a chain of dependent loads)
-        for (int64_t q0 = s + lane; q0 < e; q0 += 32 * 4) {
+    long long fl;
+    int mx, lo, hi;
+    // this lane's share of the entries s + first, s + first + stride, ... of a
+    // column (each stage's loads issued together: long columns would otherwise
+    // be a chain of dependent loads)
+    auto walk = [&](int64_t s, int64_t e, int first, int stride) {
+        fl = 0;
+        mx = 0;
+        lo = INT32_MAX;
+        hi = -1;
+        for (int64_t q0 = s + first; q0 < e; q0 += stride * 4) {
             int loc[4];
             int64_t a0[4], a1[4];
 #pragma unroll
-            for (int u = 0; u < 4; u++) loc[u] = q0 + 32 * u < e ? Bq[q0 + 32 * u] : -1;
+            for (int u = 0; u < 4; u++) loc[u] = q0 + stride * u < e ? Bq[q0 + stride * u] : -1;
 #pragma unroll
             for (int u = 0; u < 4; u++) {
                 a0[u] = loc[u] >= 0 ? At_colptr[loc[u]] : 0;
@@ -556,68 +648,105 @@ __global__ void k_col_stats(const void *Bcolptr, int p64, int64_t n, const int32
                 }
             }
         }
-        fl = warp_sum_ll(fl);
+    };
+    auto reduce = [&](int o) {
+        fl += __shfl_xor_sync(kFull, fl, o);
+        mx = max(mx, __shfl_xor_sync(kFull, mx, o));
+        lo = min(lo, __shfl_xor_sync(kFull, lo, o));
+        hi = max(hi, __shfl_xor_sync(kFull, hi, o));
+    };
+    auto store = [&](int64_t j, int64_t len) {
+        flops[j] = fl;
+        win_lo[j] = fl ? lo : 0;
+        win_hi[j] = fl ? hi : -1;
+        nnzb[j] = (int32_t)len;
+        maxa[j] = mx;
+        long long U = fl ? min(fl, (long long)(hi - lo + 1)) : 0;
+        int bin = light_bin(U, light_max);
+        bin_of[j] = (int8_t)bin;
+        atomicAdd(&hist[bin], 1);
+        prod_local += fl;
+    };
+    for (int64_t j0 = 4 * (((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5); j0 < n; j0 += 4 * nwarps) {
+        const int64_t j = j0 + (lane >> 3);
+        const bool valid = j < n;
+        const int64_t s = valid ? ld_ptr(Bcolptr, p64, j) : 0, e = valid ? ld_ptr(Bcolptr, p64, j + 1) : 0;
+        const bool is_long = e - s > kStatsLong;
+        walk(s, is_long ? s : e, gl, 8);
+        reduce(4);
+        reduce(2);
+        reduce(1);
+        if (gl == 0 && valid && !is_long) store(j, e - s);
+        for (uint32_t todo = __ballot_sync(kFull, gl == 0 && is_long); todo; todo &= todo - 1u) {
+            const int src = __ffs((int)todo) - 1;
+            const int64_t js = j0 + (src >> 3), ss = __shfl_sync(kFull, s, src), es = __shfl_sync(kFull, e, src);
+            walk(ss, es, lane, 32);
 #pragma unroll
-        for (int o = 16; o > 0; o >>= 1) {
-            mx = max(mx, __shfl_xor_sync(kFull, mx, o));
-            lo = min(lo, __shfl_xor_sync(kFull, lo, o));
-            hi = max(hi, __shfl_xor_sync(kFull, hi, o));
-        }
-        if (lane == 0) {
-            flops[j] = fl;
-            win_lo[j] = fl ? lo : 0;
-            win_hi[j] = fl ? hi : -1;
-            nnzb[j] = (int32_t)(e - s);
-            maxa[j] = mx;
-            long long U = fl ? min(fl, (long long)(hi - lo + 1)) : 0;
-            int bin = light_bin(U, light_max);
-            bin_of[j] = (int8_t)bin;
-            atomicAdd(&hist[bin], 1);
-            prod_local += fl;
+            for (int o = 16; o > 0; o >>= 1) reduce(o);
+            if (lane == 0) store(js, es - ss);
         }
     }
-    if (lane == 0 && prod_local) atomicAdd((unsigned long long *)&prod_sh, (unsigned long long)prod_local);
+    if (gl == 0 && prod_local) atomicAdd((unsigned long long *)&prod_sh, (unsigned long long)prod_local);
     __syncthreads();
     if (threadIdx.x < kNumBins && hist[threadIdx.x])
         atomicAdd((unsigned long long *)&bincnt[threadIdx.x], (unsigned long long)hist[threadIdx.x]);
     if (threadIdx.x == 0 && prod_sh) atomicAdd((unsigned long long *)products, (unsigned long long)prod_sh);
 }
 
-// Stable counting sort of column ids by bin.  Columns are cut into chunks of
-// kBinChunk; cnt[bin * nchunks + chunk] counts each chunk's columns per bin, a
-// scan of cnt (bin-major) gives every (bin, chunk) its first slot, and the
-// scatter keeps column order inside each chunk.  Within a bin the columns are
-// therefore ascending, so the heavy items of block i run before those of
-// block i + 1 and share A~_i in L2.
-constexpr int kBinChunk = 2048;
+// Stable counting sort of column ids by bin.  Columns are cut into at most
+// kBinMaxChunks chunks; cnt[bin * nchunks + chunk] counts each chunk's columns
+// per bin.  The scatter's CTA adds up, one warp per bin, the counts before its
+// chunk (at most 64 loads a lane), so that no scan and no launch stands between
+// the two kernels, and keeps column order inside its chunk.  Within a bin the
+// columns are therefore ascending, so the heavy items of block i run before
+// those of block i + 1 and share A~_i in L2.
+constexpr int kBinChunk = 2048, kBinMaxChunks = 2048;
 
-__global__ void k_bin_chunk_count(const int8_t *bin_of, int64_t n, int64_t nchunks, int32_t *cnt) {
+__global__ void k_bin_chunk_count(const int8_t *bin_of, int64_t n, int64_t chunk, int64_t nchunks, int32_t *cnt) {
     __shared__ int h[kNumBins];
     for (int64_t c = blockIdx.x; c < nchunks; c += gridDim.x) {
         if (threadIdx.x < kNumBins) h[threadIdx.x] = 0;
         __syncthreads();
-        const int64_t j0 = c * kBinChunk;
-        for (int i = threadIdx.x; i < kBinChunk; i += blockDim.x) {
-            int64_t j = j0 + i;
-            if (j < n) atomicAdd(&h[bin_of[j]], 1);
-        }
+        const int64_t j1 = min(n, (c + 1) * chunk);
+        for (int64_t j = c * chunk + threadIdx.x; j < j1; j += blockDim.x) atomicAdd(&h[bin_of[j]], 1);
         __syncthreads();
         if (threadIdx.x < kNumBins) cnt[(int64_t)threadIdx.x * nchunks + c] = h[threadIdx.x];
         __syncthreads();
     }
 }
 
-__global__ void __launch_bounds__(256)
-    k_bin_chunk_scatter(const int8_t *bin_of, int64_t n, int64_t nchunks, const int64_t *off, int32_t *list) {
-    __shared__ int run[kNumBins];
-    __shared__ int wcnt[8][kNumBins];
-    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = blockDim.x >> 5;
+// off: the bins' first slots and their total (kNumBins + 1).
+__global__ void __launch_bounds__(32 * kNumBins)
+    k_bin_chunk_scatter(const int8_t *bin_of, int64_t n, int64_t chunk, int64_t nchunks,
+                        const int32_t *__restrict__ cnt, int64_t *off, int32_t *list) {
+    __shared__ int64_t run[kNumBins], total[kNumBins];
+    __shared__ int wcnt[kNumBins][kNumBins];
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    constexpr int nw = kNumBins;
     for (int64_t c = blockIdx.x; c < nchunks; c += gridDim.x) {
-        if (threadIdx.x < kNumBins) run[threadIdx.x] = 0;
+        long long before = 0, all = 0;  // of bin `wid`
+        for (int64_t x = lane; x < nchunks; x += 32) {
+            const int v = cnt[(int64_t)wid * nchunks + x];
+            all += v;
+            if (x < c) before += v;
+        }
+        before = warp_sum_ll(before);
+        all = warp_sum_ll(all);
+        if (lane == 0) total[wid] = all;
         __syncthreads();
-        for (int r = 0; r < kBinChunk; r += blockDim.x) {
-            const int64_t j = c * kBinChunk + r + threadIdx.x;
-            const int b = j < n ? bin_of[j] : -1;
+        if (lane == 0) {
+            int64_t first = 0;
+            for (int b = 0; b < wid; b++) first += total[b];
+            run[wid] = first + before;
+            if (c == 0) {
+                off[wid] = first;
+                if (wid == kNumBins - 1) off[kNumBins] = first + all;
+            }
+        }
+        __syncthreads();
+        for (int64_t r = 0; r < chunk; r += blockDim.x) {
+            const int64_t j = c * chunk + r + threadIdx.x;
+            const int b = r + threadIdx.x < chunk && j < n ? bin_of[j] : -1;
             int myrank = 0;
 #pragma unroll
             for (int bb = 0; bb < kNumBins; bb++) {
@@ -627,9 +756,9 @@ __global__ void __launch_bounds__(256)
             }
             __syncthreads();
             if (b >= 0) {
-                int before = run[b];
-                for (int w = 0; w < wid; w++) before += wcnt[w][b];
-                list[off[(int64_t)b * nchunks + c] + before + myrank] = (int32_t)j;
+                int64_t at = run[b];
+                for (int w = 0; w < wid; w++) at += wcnt[w][b];
+                list[at + myrank] = (int32_t)j;
             }
             __syncthreads();
             if (threadIdx.x < kNumBins) {
@@ -642,57 +771,63 @@ __global__ void __launch_bounds__(256)
     }
 }
 
-spg_status bin_columns(spg_plan *p, const int8_t *bin_of, int32_t *list, int64_t *off_host) {
+// Launches only; the bins' offsets arrive in h_pinned[kPinnedBins ..] once the
+// stream is synchronised (bin_offsets).
+spg_status bin_columns_queue(spg_plan *p, const int8_t *bin_of, int32_t *list) {
     const int64_t n = p->n;
-    const int64_t nchunks = (n + kBinChunk - 1) / kBinChunk;
-    const int64_t ncnt = nchunks * kNumBins;
-    int32_t *cnt = (int32_t *)ws_alloc(p, sizeof(int32_t) * (size_t)(ncnt + 1));
-    int64_t *off = (int64_t *)ws_alloc(p, sizeof(int64_t) * (size_t)(ncnt + 1));
+    const int64_t chunk = std::max<int64_t>(kBinChunk, ((n + kBinMaxChunks - 1) / kBinMaxChunks + 255) / 256 * 256);
+    const int64_t nchunks = (n + chunk - 1) / chunk;
+    int32_t *cnt = (int32_t *)ws_alloc(p, sizeof(int32_t) * (size_t)(nchunks * kNumBins + 1));
+    int64_t *off = (int64_t *)ws_alloc(p, sizeof(int64_t) * (size_t)(kNumBins + 1));
     if (!cnt || !off) return SPG_OUT_OF_MEMORY;
     const int g = grid_for(nchunks, 1, p->sm_count * 8);
-    launch(p, k_bin_chunk_count, g, 256, 0, bin_of, n, nchunks, cnt);
-    spg_status s = scan_exclusive_i32(p, cnt, off, ncnt);
+    launch(p, k_bin_chunk_count, g, 256, 0, bin_of, n, chunk, nchunks, cnt);
+    launch(p, k_bin_chunk_scatter, g, 32 * kNumBins, 0, bin_of, n, chunk, nchunks, (const int32_t *)cnt, off, list);
+    spg_status s = cuda_check(cudaGetLastError(), "bins");
     if (s) return s;
-    for (int b = 0; b <= kNumBins; b++) {
-        s = cuda_check(cudaMemcpyAsync(p->h_pinned + b, off + (int64_t)b * nchunks, sizeof(int64_t),
-                                       cudaMemcpyDeviceToHost, p->st), "bin readback");
-        if (s) return s;
-    }
-    launch(p, k_bin_chunk_scatter, g, 256, 0, bin_of, n, nchunks, (const int64_t *)off, list);
-    s = cuda_check(cudaGetLastError(), "bin scatter");
-    if (s) return s;
-    s = cuda_check(cudaStreamSynchronize(p->st), "bin readback");
-    if (s) return s;
-    for (int b = 0; b <= kNumBins; b++) off_host[b] = p->h_pinned[b];
-    return SPG_OK;
+    return cuda_check(cudaMemcpyAsync(p->h_pinned + kPinnedBins, off, sizeof(int64_t) * (kNumBins + 1),
+                                      cudaMemcpyDeviceToHost, p->st), "bin readback");
+}
+void bin_offsets(const spg_plan *p, int64_t *off_host) {
+    for (int b = 0; b <= kNumBins; b++) off_host[b] = p->h_pinned[kPinnedBins + b];
+}
+spg_status bin_columns(spg_plan *p, const int8_t *bin_of, int32_t *list, int64_t *off_host) {
+    spg_status s = bin_columns_queue(p, bin_of, list);
+    if (!s) s = cuda_check(cudaStreamSynchronize(p->st), "bin readback");
+    if (!s) bin_offsets(p, off_host);
+    return s;
 }
 
-// Heavy bins: slabs [t_lo, t_hi] of every heavy column from its row window.
+// Heavy bins: slabs [t_lo, t_hi] of every heavy column from its row window, and
+// the symbolic items (groups of <= smr consecutive slabs) it needs.
 __global__ void k_heavy_nslab(const int32_t *list, int64_t nheavy, const int32_t *win_lo,
-                              const int32_t *win_hi, const int32_t *nnzb, int R, int64_t *nslab,
-                              long long *nnzb_heavy) {
+                              const int32_t *win_hi, const int32_t *nnzb, int R, int smr, int64_t *nslab,
+                              int64_t *nsym, long long *nnzb_heavy) {
     long long sb = 0;
     for (int64_t h = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; h < nheavy; h += (int64_t)gridDim.x * blockDim.x) {
         int j = list[h];
-        nslab[h] = (int64_t)(win_hi[j] / R - win_lo[j] / R + 1);
+        const int64_t slabs = win_hi[j] / R - win_lo[j] / R + 1;
+        nslab[h] = slabs;
+        nsym[h] = (slabs + smr - 1) / smr;
         sb += nnzb[j];
     }
     sb = warp_sum_ll(sb);
     if ((threadIdx.x & 31) == 0 && sb) atomicAdd((unsigned long long *)nnzb_heavy, (unsigned long long)sb);
 }
 
-// Records (column, base slab) of every heavy column, and the number of
-// symbolic items (groups of <= smr consecutive records) it needs.
-__global__ void k_heavy_records(const int32_t *list, int64_t nheavy, const int32_t *win_lo, int R, int smr,
-                                const int64_t *rec_first, int32_t *rec_col, int32_t *rec_slab, int64_t *nsym) {
-    for (int64_t h = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; h < nheavy; h += (int64_t)gridDim.x * blockDim.x) {
-        int j = list[h];
-        int t0 = win_lo[j] / R;
-        for (int64_t r = rec_first[h]; r < rec_first[h + 1]; r++) {
+// Records (column, base slab) of every heavy column, a warp per column.
+__global__ void k_heavy_records(const int32_t *list, int64_t nheavy, const int32_t *win_lo, int R,
+                                const int64_t *rec_first, int32_t *rec_col, int32_t *rec_slab) {
+    const int lane = threadIdx.x & 31;
+    for (int64_t h = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; h < nheavy;
+         h += ((int64_t)gridDim.x * blockDim.x) >> 5) {
+        const int j = list[h];
+        const int t0 = win_lo[j] / R;
+        const int64_t r0 = rec_first[h], r1 = rec_first[h + 1];
+        for (int64_t r = r0 + lane; r < r1; r += 32) {
             rec_col[r] = j;
-            rec_slab[r] = t0 + (int)(r - rec_first[h]);
+            rec_slab[r] = t0 + (int)(r - r0);
         }
-        nsym[h] = (rec_first[h + 1] - rec_first[h] + smr - 1) / smr;
     }
 }
 
@@ -744,8 +879,11 @@ spg_status copy_operands(spg_plan *p) {
     if (p->ndt > 0 && p->nAt > 0) {
         if (!p->gshift) p->gshift = (int64_t *)ws_alloc(p, sizeof(int64_t) * (size_t)p->ndt);
         if (!p->gshift) return SPG_OUT_OF_MEMORY;
-        // about 2048 entries per warp, at most 32 CTAs of 8 warps per SM
-        const int64_t warps = std::max<int64_t>(1, std::min<int64_t>((p->nAt + 2047) / 2048, (int64_t)sm * 32 * 8));
+        // at least 128 entries per warp, about 2048 once that fills the GPU
+        // (226,000 entries: 35 us in 2048s, 110 warps), at most 32 CTAs of 8
+        // warps per SM
+        const int64_t per = std::min<int64_t>(2048, std::max<int64_t>(128, p->nAt / ((int64_t)sm * 32)));
+        const int64_t warps = std::max<int64_t>(1, std::min<int64_t>((p->nAt + per - 1) / per, (int64_t)sm * 32 * 8));
         const int64_t chunk = ((p->nAt + warps - 1) / warps + 31) & ~(int64_t)31;
         const int64_t g = (((p->nAt + chunk - 1) / chunk) + 7) / 8;
         group_begin(p, kKGather);
@@ -773,6 +911,9 @@ spg_status copy_operands(spg_plan *p) {
     }
     return SPG_OK;
 }
+
+// Lists of D~ up to this many entries are sized by their bound (plan_build).
+constexpr int64_t kEarlyLists = 1 << 20;
 
 static bool valid_type(int32_t v, int maxv) { return v >= 0 && v <= maxv; }
 
@@ -814,39 +955,46 @@ static spg_status plan_build(spg_plan *p) {
     const int p64B = B.ptr_type == SPG_IDX_I64, i64B = B.idx_type == SPG_IDX_I64;
     const size_t accsz = 8;
 
-    p->d_err = (int *)ws_alloc(p, sizeof(int) * 4);
-    p->d_cnt = (int64_t *)ws_alloc(p, sizeof(int64_t) * kCntSlots);
-    p->d_bincur = (int64_t *)ws_alloc(p, sizeof(int64_t) * kNumBins);
-    if (!p->d_err || !p->d_cnt || !p->d_bincur) return SPG_OUT_OF_MEMORY;
-    TRY(cuda_check(cudaMemsetAsync(p->d_err, 0, sizeof(int) * 4, st), "memset"));
-    TRY(cuda_check(cudaMemsetAsync(p->d_cnt, 0, sizeof(int64_t) * kCntSlots, st), "memset"));
+    // everything that starts at zero, cleared by one memset: error word,
+    // counters, per-block sums
+    const size_t zero_words = 2 + kCntSlots + 3 * (size_t)P;
+    int64_t *zeroed = (int64_t *)ws_alloc(p, sizeof(int64_t) * zero_words);
+    if (!zeroed) return SPG_OUT_OF_MEMORY;
+    p->d_err = (int *)zeroed;
+    p->d_cnt = zeroed + 2;
+    p->blk = p->d_cnt + kCntSlots;
+    TRY(cuda_check(cudaMemsetAsync(zeroed, 0, sizeof(int64_t) * zero_words, st), "memset"));
     cudaEventRecord(p->ev[0], st);
 
+    // Validation.  Its result is read back together with |D~| (the kernels up
+    // to there index nothing by unchecked contents), except ahead of the flop
+    // split, which walks B's columns.
+    const bool split_flops = p->opt.split == SPG_SPLIT_FLOPS && P > 1 && n > 0;
     if (p->opt.validate) {
-        const int64_t sw = (std::max<int64_t>(A.nnz, B.nnz) + 31) / 32 + 1;
-        uint32_t *starts = (uint32_t *)ws_alloc(p, sizeof(uint32_t) * (size_t)sw);
+        const bool same = A.colptr == B.colptr && A.rowidx == B.rowidx && A.nnz == B.nnz && A.ncols == B.ncols &&
+                          A.nrows == B.nrows && A.ptr_type == B.ptr_type && A.idx_type == B.idx_type;
+        const int nm = same ? 1 : 2;
+        const size_t wa = (size_t)(A.nnz / 32 + 1), wb = same ? 0 : (size_t)(B.nnz / 32 + 1);
+        uint32_t *starts = (uint32_t *)ws_alloc(p, sizeof(uint32_t) * (wa + wb));
         if (!starts) return SPG_OUT_OF_MEMORY;
+        TRY(cuda_check(cudaMemsetAsync(starts, 0, sizeof(uint32_t) * (wa + wb), st), "memset"));
+        ValidateArgs va;
         const spg_csc *M[2] = {&A, &B};
-        for (int i = 0; i < 2; i++) {
-            const int pp = M[i]->ptr_type == SPG_IDX_I64, ii = M[i]->idx_type == SPG_IDX_I64;
-            TRY(cuda_check(cudaMemsetAsync(starts, 0, sizeof(uint32_t) * (size_t)sw, st), "memset"));
-            launch(p, k_validate_cols, grid_for(M[i]->ncols + 1, 256, sm * 8), 256, 0, M[i]->colptr, pp,
-                   M[i]->ncols, M[i]->nnz, starts, p->d_err);
-            if (M[i]->nnz > 0)
-                launch(p, k_validate_rows, grid_for(M[i]->nnz, 256, sm * 16), 256, 0, M[i]->rowidx, ii, M[i]->nnz,
-                       M[i]->nrows, (const uint32_t *)starts, p->d_err);
-        }
+        for (int i = 0; i < 2; i++)
+            va.m[i] = ValidateArg{M[i]->colptr, M[i]->rowidx, M[i]->ptr_type == SPG_IDX_I64,
+                                  M[i]->idx_type == SPG_IDX_I64, M[i]->ncols, M[i]->nnz, M[i]->nrows,
+                                  starts + (i == 0 ? 0 : wa)};
+        const int64_t mc = same ? A.ncols : std::max(A.ncols, B.ncols), mz = same ? A.nnz : std::max(A.nnz, B.nnz);
+        launch(p, k_validate_cols, dim3(grid_for(mc + 1, 256, sm * 8), nm), 256, 0, va, p->d_err);
+        if (mz > 0) launch(p, k_validate_rows, dim3(grid_for((mz + 3) / 4, 256, sm * 16), nm), 256, 0, va, p->d_err);
         LAUNCH_OK("validate");
-        TRY(read_dev_err(p, "input validation"));
+        if (split_flops) TRY(read_dev_err(p, "input validation"));
     }
 
     // --- column blocks: uniform, or contiguous with balanced flops
-    p->blk = (int64_t *)ws_alloc(p, sizeof(int64_t) * 3 * (size_t)P);
-    if (!p->blk) return SPG_OUT_OF_MEMORY;
-    TRY(cuda_check(cudaMemsetAsync(p->blk, 0, sizeof(int64_t) * 3 * (size_t)P, st), "memset"));
     p->bounds_h.resize(P + 1);
     for (int i = 0; i <= P; i++) p->bounds_h[i] = (int64_t)i * n / P;
-    if (p->opt.split == SPG_SPLIT_FLOPS && P > 1 && n > 0) {
+    if (split_flops) {
         int64_t *fl = (int64_t *)ws_alloc(p, sizeof(int64_t) * (size_t)(n + 1));
         int64_t *pre = (int64_t *)ws_alloc(p, sizeof(int64_t) * (size_t)(n + 1));
         p->bounds_d = (int64_t *)ws_alloc(p, sizeof(int64_t) * (size_t)(P + 1));
@@ -856,7 +1004,7 @@ static spg_status plan_build(spg_plan *p) {
         TRY(scan_exclusive_i64(p, fl, pre, n));
         launch(p, k_split_bounds, grid_for(P + 1, 256, sm), 256, 0, pre, n, P, p->bounds_d);
         LAUNCH_OK("flop split");
-        int64_t *hb = p->h_pinned + 64;
+        int64_t *hb = p->h_pinned + kPinnedBlocks;
         TRY(cuda_check(cudaMemcpyAsync(hb, p->bounds_d, sizeof(int64_t) * (size_t)(P + 1), cudaMemcpyDeviceToHost, st),
                        "split readback"));
         TRY(cuda_check(cudaStreamSynchronize(st), "split readback"));
@@ -880,7 +1028,7 @@ static spg_status plan_build(spg_plan *p) {
     launch(p, k_block_eoff, grid_for(P + 1, 256, sm), 256, 0, B.colptr, p64B, n, P, (const int64_t *)p->bounds_d,
            p->eoff);
     if (B.nnz > 0)
-        launch(p, k_mark_H, grid_for(B.nnz, 256, sm * 16), 256, 0, B.rowidx, i64B, B.nnz, P, W, p->Hbits,
+        launch(p, k_mark_H, grid_for(B.nnz, 256, sm * 16), 256, 0, B.rowidx, i64B, B.nnz, P, k, W, p->Hbits,
                (const int64_t *)p->eoff);
     LAUNCH_OK("mark H");
 
@@ -890,43 +1038,55 @@ static spg_status plan_build(spg_plan *p) {
         launch(p, k_popc_HD, grid_for(PW, 256, sm * 8), 256, 0, p->Hbits, p->Dbits, W, PW, popc,
                                                             (long long *)(p->d_cnt + kCntSumH));
     TRY(scan_exclusive_i32(p, popc, p->rankpre, PW));
-    // |D~| in total and per block: read the block boundaries of the scan
-    std::vector<int64_t> idx(P + 1);
-    for (int i = 0; i <= P; i++) idx[i] = (int64_t)i * W;
-    int64_t *hb = p->h_pinned + 64;
-    for (int i = 0; i <= P; i++)
-        TRY(cuda_check(cudaMemcpyAsync(hb + i, p->rankpre + idx[i], sizeof(int64_t), cudaMemcpyDeviceToHost, st),
-                       "rank readback"));
+    // |D~| in total and per block: the block boundaries of the scan
+    int64_t *d_dt_base = (int64_t *)ws_alloc(p, sizeof(int64_t) * (size_t)(P + 1));
+    if (!d_dt_base) return SPG_OUT_OF_MEMORY;
+    launch(p, k_block_dt, grid_for(P + 1, 256, sm), 256, 0, (const int64_t *)p->rankpre, W, P, d_dt_base);
+    int64_t *hb = p->h_pinned + kPinnedBlocks;
+    TRY(cuda_check(cudaMemcpyAsync(hb, d_dt_base, sizeof(int64_t) * (size_t)(P + 1), cudaMemcpyDeviceToHost, st),
+                   "rank readback"));
+    TRY(dev_err_queue(p, "input validation"));
+    // the lists of D~ and the lengths of A~'s columns, for `cap` entries >= |D~|
+    int64_t *glen = nullptr;
+    auto dtilde_lists = [&](int64_t cap) -> spg_status {
+        p->dtilde = (int32_t *)ws_alloc(p, sizeof(int32_t) * (size_t)(cap + 1));
+        p->At_colptr = (int64_t *)ws_alloc(p, sizeof(int64_t) * (size_t)(cap + 1));
+        glen = (int64_t *)ws_alloc(p, sizeof(int64_t) * (size_t)(cap + 1));
+        if (!p->dtilde || !p->At_colptr || !glen) return SPG_OUT_OF_MEMORY;
+        if (PW > 0)
+            launch(p, k_dtilde, grid_for(PW, 256, sm * 8), 256, 0, p->Hbits, p->Dbits, p->rankpre, W, PW, p->dtilde);
+        if (P * p->nfb > 0)
+            launch(p, k_fetch, grid_for(P * p->nfb, 256, sm * 8), 256, 0, p->Hbits, p->Dbits, p->rankpre, W, k, p->b,
+                   p->nfb, P, A.colptr, p64A, p->fetch, (long long *)(p->d_cnt + kCntFetchChosen),
+                   (long long *)(p->d_cnt + kCntVolBlock));
+        LAUNCH_OK("dtilde / fetch");
+        // --- step 3: gather A~
+        if (cap > 0)
+            launch(p, k_gather_len, grid_for(cap, 256, sm * 8), 256, 0, p->dtilde, cap, A.colptr, p64A, glen,
+                   (long long *)(p->d_cnt + kCntMaxAcol), d_dt_base, P, k, (long long *)(p->d_cnt + kCntRemote),
+                   (long long *)(p->blk + P), (long long *)(p->blk + 2 * P));
+        TRY(scan_exclusive_i64(p, glen, p->At_colptr, cap));
+        TRY(cuda_check(cudaMemcpyAsync(p->h_pinned, p->At_colptr + cap, sizeof(int64_t), cudaMemcpyDeviceToHost, st), "readback"));
+        return cuda_check(cudaMemcpyAsync(p->h_pinned + 1, p->d_cnt + kCntMaxAcol, sizeof(int64_t), cudaMemcpyDeviceToHost, st), "readback");
+    };
+    // A small product does not wait for |D~|: its lists are sized by a bound
+    // and one synchronisation serves both sizes (a wait costs about 15 us; a
+    // bound of 2^20 entries costs 20 MB and a few us of scanning zeros).
+    const int64_t dt_cap = std::min<int64_t>(B.nnz, PW * 32);
+    const bool early = dt_cap <= kEarlyLists;
+    if (early) TRY(dtilde_lists(dt_cap));
     TRY(cuda_check(cudaStreamSynchronize(st), "rank readback"));
+    TRY(dev_err_read(p, "input validation"));
     p->dt_base.assign(hb, hb + P + 1);
     p->ndt = p->dt_base[P];
     if (p->ndt >= INT32_MAX) {
         set_error("sum of |D~_i| (%lld) exceeds int32", (long long)p->ndt);
         return SPG_UNSUPPORTED;
     }
-    p->dtilde = (int32_t *)ws_alloc(p, sizeof(int32_t) * (size_t)(p->ndt + 1));
-    p->At_colptr = (int64_t *)ws_alloc(p, sizeof(int64_t) * (size_t)(p->ndt + 1));
-    int64_t *glen = (int64_t *)ws_alloc(p, sizeof(int64_t) * (size_t)(p->ndt + 1));
-    int64_t *d_dt_base = (int64_t *)ws_alloc(p, sizeof(int64_t) * (size_t)(P + 1));
-    if (!p->dtilde || !p->At_colptr || !glen || !d_dt_base) return SPG_OUT_OF_MEMORY;
-    TRY(cuda_check(cudaMemcpyAsync(d_dt_base, hb, sizeof(int64_t) * (size_t)(P + 1), cudaMemcpyHostToDevice, st),
-                   "block offsets"));
-    if (PW > 0) launch(p, k_dtilde, grid_for(PW, 256, sm * 8), 256, 0, p->Hbits, p->Dbits, p->rankpre, W, PW, p->dtilde);
-    if (P * p->nfb > 0)
-        launch(p, k_fetch, grid_for(P * p->nfb, 256, sm * 8), 256, 0,
-            p->Hbits, p->Dbits, p->rankpre, W, k, p->b, p->nfb, P, A.colptr, p64A, p->fetch,
-            (long long *)(p->d_cnt + kCntFetchChosen), (long long *)(p->d_cnt + kCntVolBlock));
-    LAUNCH_OK("dtilde / fetch");
-
-    // --- step 3: gather A~
-    if (p->ndt > 0)
-        launch(p, k_gather_len, grid_for(p->ndt, 256, sm * 8), 256, 0, p->dtilde, p->ndt, A.colptr, p64A, glen,
-                                                                  (long long *)(p->d_cnt + kCntMaxAcol), d_dt_base, P, k, (long long *)(p->d_cnt + kCntRemote),
-               (long long *)(p->blk + P), (long long *)(p->blk + 2 * P));
-    TRY(scan_exclusive_i64(p, glen, p->At_colptr, p->ndt));
-    TRY(cuda_check(cudaMemcpyAsync(p->h_pinned, p->At_colptr + p->ndt, sizeof(int64_t), cudaMemcpyDeviceToHost, st), "readback"));
-    TRY(cuda_check(cudaMemcpyAsync(p->h_pinned + 1, p->d_cnt + kCntMaxAcol, sizeof(int64_t), cudaMemcpyDeviceToHost, st), "readback"));
-    TRY(cuda_check(cudaStreamSynchronize(st), "readback"));
+    if (!early) {
+        TRY(dtilde_lists(p->ndt));
+        TRY(cuda_check(cudaStreamSynchronize(st), "readback"));
+    }
     p->nAt = p->h_pinned[0];
     if (p->h_pinned[1] >= (1LL << 26)) {
         set_error("a column of A holds %lld nonzeros; this build supports < 2^26 per column", (long long)p->h_pinned[1]);
@@ -952,14 +1112,23 @@ static spg_status plan_build(spg_plan *p) {
     if (!p->flops || !p->win_lo || !p->win_hi || !p->nnzb || !p->maxa || !p->bin_of || !p->binlist ||
         !p->nnzcol || !p->Ccolptr)
         return SPG_OUT_OF_MEMORY;
+    // the counters, the bins and the error word, one wait for all
+    auto read_counters = [&]() -> spg_status {
+        TRY(cuda_check(cudaMemcpyAsync(p->h_pinned, p->d_cnt, sizeof(int64_t) * kCntSlots, cudaMemcpyDeviceToHost, st), "stats"));
+        TRY(dev_err_queue(p, "plan"));
+        TRY(cuda_check(cudaStreamSynchronize(st), "plan readback"));
+        return dev_err_read(p, "plan");
+    };
     if (n > 0) {
-        launch(p, k_col_stats, grid_for(n * 32, 256, sm * 16), 256, 0,
-            B.colptr, p64B, n, p->Bq, p->At_colptr, p->At_row, p->light_max, p->flops, p->win_lo, p->win_hi,
-            p->nnzb, p->maxa, p->bin_of, (long long *)(p->d_cnt + kCntBin0), (long long *)(p->d_cnt + kCntProducts));
+        launch(p, k_col_stats, grid_for(n * 8, 256, sm * 16), 256, 0, B.colptr, p64B, n, p->Bq, p->At_colptr,
+               p->At_row, p->light_max, p->flops, p->win_lo, p->win_hi, p->nnzb, p->maxa, p->bin_of,
+               (long long *)(p->d_cnt + kCntBin0), (long long *)(p->d_cnt + kCntProducts));
         launch(p, k_block_flops, grid_for(n, 256, sm * 8), 256, 0, p->flops, n, P, p->bounds_d, (long long *)p->blk);
         LAUNCH_OK("column stats");
-        TRY(bin_columns(p, p->bin_of, p->binlist, p->bin_off));
+        TRY(bin_columns_queue(p, p->bin_of, p->binlist));
     }
+    TRY(read_counters());
+    if (n > 0) bin_offsets(p, p->bin_off);
     p->nheavy = p->bin_off[kBinHeavy + 1] - p->bin_off[kBinHeavy];
 
     // --- heavy bins: slab items and the split index of A~
@@ -973,11 +1142,16 @@ static spg_status plan_build(spg_plan *p) {
         p->rec_first = (int64_t *)ws_alloc(p, sizeof(int64_t) * (size_t)(p->nheavy + 1));
         if (!nslab || !nsym || !sym_first || !p->rec_first) return SPG_OUT_OF_MEMORY;
         launch(p, k_heavy_nslab, grid_for(p->nheavy, 256, sm * 8), 256, 0, hl, p->nheavy, p->win_lo, p->win_hi,
-               p->nnzb, p->R, nslab, (long long *)(p->d_cnt + kCntNnzBHeavy));
+               p->nnzb, p->R, p->sym_max_recs, nslab, nsym, (long long *)(p->d_cnt + kCntNnzBHeavy));
         TRY(scan_exclusive_i64(p, nslab, p->rec_first, p->nheavy));
-        TRY(cuda_check(cudaMemcpyAsync(p->h_pinned, p->rec_first + p->nheavy, sizeof(int64_t), cudaMemcpyDeviceToHost, st), "records"));
-        TRY(cuda_check(cudaStreamSynchronize(st), "records"));
-        p->nrec = p->h_pinned[0];
+        TRY(scan_exclusive_i64(p, nsym, sym_first, p->nheavy));
+        TRY(hub_histogram_queue(p));
+        TRY(cuda_check(cudaMemcpyAsync(p->h_pinned + kPinnedRec, p->rec_first + p->nheavy, sizeof(int64_t), cudaMemcpyDeviceToHost, st), "records"));
+        TRY(cuda_check(cudaMemcpyAsync(p->h_pinned + kPinnedRec + 1, sym_first + p->nheavy, sizeof(int64_t), cudaMemcpyDeviceToHost, st), "items"));
+        TRY(read_counters());
+        hub_histogram_read(p);
+        p->nrec = p->h_pinned[kPinnedRec];
+        p->nsym = p->h_pinned[kPinnedRec + 1];
         if (p->nrec >= INT32_MAX) {
             set_error("too many heavy slab records (%lld)", (long long)p->nrec);
             return SPG_UNSUPPORTED;
@@ -988,17 +1162,13 @@ static spg_status plan_build(spg_plan *p) {
         p->rec_off = (int64_t *)ws_alloc(p, sizeof(int64_t) * (size_t)p->nrec);
         p->hbits = (uint32_t *)ws_alloc(p, sizeof(uint32_t) * (size_t)p->nrec * (size_t)(p->R / 32));
         p->split = (int32_t *)ws_alloc(p, sizeof(int32_t) * (size_t)(p->ndt + 1) * (size_t)(p->T + 1));
-        if (!p->rec_col || !p->rec_slab || !p->rec_cnt || !p->rec_off || !p->hbits || !p->split)
-            return SPG_OUT_OF_MEMORY;
-        launch(p, k_heavy_records, grid_for(p->nheavy, 256, sm * 8), 256, 0, hl, p->nheavy, p->win_lo, p->R,
-               p->sym_max_recs, p->rec_first, p->rec_col, p->rec_slab, nsym);
-        TRY(scan_exclusive_i64(p, nsym, sym_first, p->nheavy));
-        TRY(cuda_check(cudaMemcpyAsync(p->h_pinned, sym_first + p->nheavy, sizeof(int64_t), cudaMemcpyDeviceToHost, st), "items"));
-        TRY(cuda_check(cudaStreamSynchronize(st), "items"));
-        p->nsym = p->h_pinned[0];
         p->sym_rec0 = (int32_t *)ws_alloc(p, sizeof(int32_t) * (size_t)p->nsym);
         p->sym_nrec = (int32_t *)ws_alloc(p, sizeof(int32_t) * (size_t)p->nsym);
-        if (!p->sym_rec0 || !p->sym_nrec) return SPG_OUT_OF_MEMORY;
+        if (!p->rec_col || !p->rec_slab || !p->rec_cnt || !p->rec_off || !p->hbits || !p->split || !p->sym_rec0 ||
+            !p->sym_nrec)
+            return SPG_OUT_OF_MEMORY;
+        launch(p, k_heavy_records, grid_for(p->nheavy * 32, 256, sm * 8), 256, 0, hl, p->nheavy, p->win_lo, p->R,
+               p->rec_first, p->rec_col, p->rec_slab);
         launch(p, k_sym_items, grid_for(p->nheavy, 256, sm * 8), 256, 0, p->nheavy, p->sym_max_recs, p->rec_first,
                sym_first, p->sym_rec0, p->sym_nrec);
         if (p->ndt > 0)
@@ -1008,9 +1178,8 @@ static spg_status plan_build(spg_plan *p) {
     }
     cudaEventRecord(p->ev[1], st);
 
-    // statistics
-    TRY(cuda_check(cudaMemcpyAsync(p->h_pinned, p->d_cnt, sizeof(int64_t) * kCntSlots, cudaMemcpyDeviceToHost, st), "stats"));
-    TRY(cuda_check(cudaStreamSynchronize(st), "stats"));
+    // statistics (the counters are on the host; the phase times are taken when
+    // they are asked for)
     spg_stats &S = p->stats;
     S.m = m; S.k = k; S.n = n; S.nnzA = p->nnzA; S.nnzB = p->nnzB; S.P = P; S.b = p->b;
     S.products = p->h_pinned[kCntProducts];
@@ -1028,11 +1197,7 @@ static spg_status plan_build(spg_plan *p) {
     S.nnzB_heavy = p->h_pinned[kCntNnzBHeavy];
     S.gathered_nnz_remote = p->h_pinned[kCntRemote];
     S.nnzC_heavy = -1;
-    float ms = 0;
-    cudaEventElapsedTime(&ms, p->ev[0], p->ev[1]);
-    S.ms_plan = ms;
-    if (p->kev_used[kKGather] && cudaEventElapsedTime(&ms, p->kev[0], p->kev[1]) == cudaSuccess) S.ms_gather = ms;
-    return read_dev_err(p, "plan");
+    return SPG_OK;
 }
 
 }  // namespace spg
@@ -1146,8 +1311,9 @@ extern "C" spg_status spgemm_plan(const spg_csc *A, const spg_csc *B, const spg_
     int dev = 0;
     spg_status s = cuda_check(cudaGetDevice(&dev), "cudaGetDevice");
     if (!s) s = cuda_check(cudaDeviceGetAttribute(&p->sm_count, cudaDevAttrMultiProcessorCount, dev), "attr");
-    // slots 0..63: counters and the error word; 64..64+P: the per-block D~ offsets
-    if (!s) s = cuda_check(cudaMallocHost(&p->h_pinned, sizeof(int64_t) * (64 + (size_t)p->P + 1)), "cudaMallocHost");
+    if (!s)
+        s = cuda_check(cudaMallocHost(&p->h_pinned, sizeof(int64_t) * (kPinnedBlocks + (size_t)p->P + 1)),
+                       "cudaMallocHost");
     for (int i = 0; i < 8 && !s; i++) s = cuda_check(cudaEventCreate(&p->ev[i]), "event");
     for (int i = 0; i < 10 && !s; i++) s = cuda_check(cudaEventCreate(&p->kev[i]), "event");
     if (!s) s = plan_build(p);
@@ -1167,7 +1333,6 @@ extern "C" spg_status spgemm_plan_destroy(spg_plan *p) {
     if (p->graph_exec) cudaGraphExecDestroy(p->graph_exec);
     if (p->graph) cudaGraphDestroy(p->graph);
     ws_free_all(p);
-    cudaStreamSynchronize(p->st);
     for (int i = 0; i < 8; i++)
         if (p->ev[i]) cudaEventDestroy(p->ev[i]);
     for (int i = 0; i < 10; i++)

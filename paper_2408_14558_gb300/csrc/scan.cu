@@ -1,4 +1,8 @@
-// Exclusive prefix sums (reduce-then-scan, three launches, no spin waits).
+// Exclusive prefix sums (no spin waits).  Up to kScanOne elements: one CTA, one
+// launch.  Up to kScanTiles tiles: two launches, the tile sums and the tiles,
+// every tile adding up the sums before its own (at most 16 loads a thread).
+// Beyond: three launches, the sums scanned by one CTA in between.  A launch
+// costs about 3 us in the chain of a small plan, which has five scans.
 // Used for the rank of required columns, the gathered column pointers, the
 // heavy-slab item lists and the column pointers of C.
 #include "spg_internal.cuh"
@@ -29,9 +33,8 @@ __global__ void k_scan_reduce(const T *__restrict__ in, int64_t n, long long *__
     }
 }
 
-// One block scans the per-tile partial sums in place (exclusive) and writes
-// the grand total to *total.
-__global__ void k_scan_partials(long long *part, int64_t ntiles, long long *total) {
+// One block scans the per-tile partial sums in place (exclusive).
+__global__ void k_scan_partials(long long *part, int64_t ntiles) {
     __shared__ long long carry_sh;
     __shared__ long long wsum[32];
     if (threadIdx.x == 0) carry_sh = 0;
@@ -66,13 +69,16 @@ __global__ void k_scan_partials(long long *part, int64_t ntiles, long long *tota
         if (threadIdx.x == blockDim.x - 1) carry_sh = carry + wsum[wid] + incl;
         __syncthreads();
     }
-    if (threadIdx.x == 0) *total = carry_sh;
 }
 
-template <typename T>
-__global__ void k_scan_tiles(const T *__restrict__ in, int64_t n, const long long *__restrict__ part,
-                             const long long *__restrict__ total, int64_t *__restrict__ out) {
-    __shared__ long long wsum[kScanThreads / 32];
+constexpr int64_t kScanOne = 4 * 8192, kScanTiles = 4096;
+
+// SUM: part holds the tiles' sums (this tile adds up those before it), else
+// their scanned prefixes.
+template <bool SUM, typename T>
+__global__ void __launch_bounds__(kScanThreads)
+    k_scan_tiles(const T *__restrict__ in, int64_t n, const long long *__restrict__ part, int64_t *__restrict__ out) {
+    __shared__ long long wsum[kScanThreads / 32], psum[kScanThreads / 32];
     int64_t base = (int64_t)blockIdx.x * kScanTile;
     // each thread owns kScanPer consecutive elements
     long long v[kScanPer];
@@ -91,25 +97,60 @@ __global__ void k_scan_tiles(const T *__restrict__ in, int64_t n, const long lon
         if (lane >= o) incl += t;
     }
     if (lane == 31) wsum[wid] = incl;
-    __syncthreads();
-    if (wid == 0) {
-        long long w = lane < kScanThreads / 32 ? wsum[lane] : 0;
-        long long wi = w;
-#pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-            long long t = __shfl_up_sync(kFull, wi, o);
-            if (lane >= o) wi += t;
-        }
-        if (lane < kScanThreads / 32) wsum[lane] = wi - w;
+    if (SUM) {
+        long long p = 0;
+        for (int t = threadIdx.x; t < (int)blockIdx.x; t += kScanThreads) p += part[t];
+        p = warp_sum_ll(p);
+        if (lane == 0) psum[wid] = p;
     }
     __syncthreads();
-    long long acc = part[blockIdx.x] + wsum[wid] + incl - run;
+    long long acc = (SUM ? 0 : part[blockIdx.x]) + incl - run;
+#pragma unroll
+    for (int w = 0; w < kScanThreads / 32; w++) {
+        if (SUM) acc += psum[w];
+        if (w < wid) acc += wsum[w];
+    }
 #pragma unroll
     for (int i = 0; i < kScanPer; i++) {
         if (my + i < n) out[my + i] = acc;
         acc += v[i];
+        if (my + i == n - 1) out[n] = acc;
     }
-    if (blockIdx.x == 0 && threadIdx.x == 0) out[n] = *total;
+}
+
+// The whole scan by one CTA, 8192 elements at a time.
+template <typename T>
+__global__ void __launch_bounds__(1024) k_scan_one(const T *__restrict__ in, int64_t n, int64_t *__restrict__ out) {
+    __shared__ long long wsum[2][32];
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    long long carry = 0;
+    int flip = 0;
+    for (int64_t base = 0; base < n; base += 1024 * kScanPer, flip ^= 1) {
+        const int64_t my = base + (int64_t)threadIdx.x * kScanPer;
+        long long v[kScanPer], run = 0;
+#pragma unroll
+        for (int i = 0; i < kScanPer; i++) {
+            v[i] = my + i < n ? (long long)in[my + i] : 0;
+            run += v[i];
+        }
+        long long incl = run;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const long long t = __shfl_up_sync(kFull, incl, o);
+            if (lane >= o) incl += t;
+        }
+        if (lane == 31) wsum[flip][wid] = incl;
+        __syncthreads();  // (the other half of wsum is free again: every thread has passed this barrier since)
+        const long long w = wsum[flip][lane];
+        long long acc = carry + warp_sum_ll(lane < wid ? w : 0) + incl - run;
+        carry += warp_sum_ll(w);
+#pragma unroll
+        for (int i = 0; i < kScanPer; i++) {
+            if (my + i < n) out[my + i] = acc;
+            acc += v[i];
+        }
+    }
+    if (threadIdx.x == 0) out[n] = carry;
 }
 
 template <typename T>
@@ -117,12 +158,20 @@ static spg_status scan_impl(spg_plan *p, const T *in, int64_t *out, int64_t n) {
     if (n == 0) {
         return cuda_check(cudaMemsetAsync(out, 0, sizeof(int64_t), p->st), "scan memset");
     }
+    if (n <= kScanOne) {
+        launch(p, k_scan_one<T>, 1, 1024, 0, in, n, out);
+        return cuda_check(cudaGetLastError(), "scan launch");
+    }
     int64_t ntiles = (n + kScanTile - 1) / kScanTile;
     long long *part = (long long *)ws_alloc(p, sizeof(long long) * (size_t)(ntiles + 1));
     if (!part) return SPG_OUT_OF_MEMORY;
     launch(p, k_scan_reduce<T>, (unsigned)ntiles, kScanThreads, 0, in, n, part);
-    launch(p, k_scan_partials, 1, 1024, 0, part, ntiles, part + ntiles);
-    launch(p, k_scan_tiles<T>, (unsigned)ntiles, kScanThreads, 0, in, n, part, part + ntiles, out);
+    if (ntiles <= kScanTiles) {
+        launch(p, k_scan_tiles<true, T>, (unsigned)ntiles, kScanThreads, 0, in, n, part, out);
+    } else {
+        launch(p, k_scan_partials, 1, 1024, 0, part, ntiles);
+        launch(p, k_scan_tiles<false, T>, (unsigned)ntiles, kScanThreads, 0, in, n, part, out);
+    }
     return cuda_check(cudaGetLastError(), "scan launch");
 }
 

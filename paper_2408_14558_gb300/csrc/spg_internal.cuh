@@ -116,7 +116,8 @@ struct spg_plan {
     int8_t *bin_of = nullptr;
     int32_t *binlist = nullptr;
     int64_t bin_off[spg::kNumBins + 1] = {0};
-    int64_t *d_bincur = nullptr;
+
+    int64_t hub_hist[32] = {0};  // columns of A by floor(log2(length)) (heavy plans)
 
     // heavy bins.  A record is one (heavy column, base slab of R rows) inside
     // the column's row window; the records of a column are consecutive.
@@ -154,6 +155,7 @@ struct spg_plan {
     cudaGraph_t graph = nullptr;     // captured refresh + numeric (spgemm_plan_capture)
     cudaGraphExec_t graph_exec = nullptr;
     int64_t nbin_off[spg::kNumBins + 1] = {0};
+    bool nbins_queued = false;       // their read-back is on the stream
 
     spg_stats stats{};
     // ev[0..1] plan, ev[2..3] symbolic, ev[4..5] numeric; kev[2g], kev[2g+1]
@@ -205,10 +207,22 @@ spg_status cuda_check(cudaError_t e, const char *what);
 void *ws_alloc(spg_plan *p, size_t bytes);
 void ws_free_all(spg_plan *p);
 spg_status copy_operands(spg_plan *p);
-spg_status prepare_numeric(spg_plan *p);
+spg_status queue_numeric_bins(spg_plan *p);
+void read_numeric_bins(spg_plan *p);
 // Memory handed to the caller (C's arrays): through opt->alloc, else cudaMallocAsync.
 void *alloc_user(const spg_options *opt, size_t bytes);
 spg_status read_dev_err(spg_plan *p, const char *phase);
+spg_status dev_err_queue(spg_plan *p, const char *phase);
+spg_status dev_err_read(spg_plan *p, const char *phase);
+// The plan's counters without waiting or reading the error word (api.cu); the
+// stream must be idle.
+void collect_stats(spg_plan *p, spg_stats *st);
+// Slots of plan->h_pinned: the device counters or single sizes from 0, the
+// counts of heavy records and items, the hub histogram, bin offsets, the error
+// word, and from kPinnedBlocks on one value per column block.  (The learned
+// path keeps its own sizes in the histogram's slots, which are read in the
+// plan.)
+constexpr int kPinnedHist = 24, kPinnedBins = 56, kPinnedErr = 66, kPinnedRec = 68, kPinnedBlocks = 72;
 int grid_for(int64_t work, int per_block, int max_blocks);
 
 // ---- scans (scan.cu): out[0..n] = exclusive prefix of in[0..n), out[n] = total.
@@ -217,6 +231,12 @@ spg_status scan_exclusive_i64(spg_plan *p, const int64_t *in, int64_t *out, int6
 
 // ---- binning (plan.cu): group the columns whose bin id is in bin_of into binlist.
 spg_status bin_columns(spg_plan *p, const int8_t *bin_of, int32_t *list, int64_t *off_host);
+spg_status bin_columns_queue(spg_plan *p, const int8_t *bin_of, int32_t *list);
+void bin_offsets(const spg_plan *p, int64_t *off_host);
+
+// ---- hub columns of A (symbolic.cu): lengths by power of two, read back in the plan
+spg_status hub_histogram_queue(spg_plan *p);
+void hub_histogram_read(spg_plan *p);
 
 // ---- phases
 spg_status run_symbolic(spg_plan *p);

@@ -285,48 +285,57 @@ static spg_status launch_sym_light(spg_plan *p, const int32_t *list, int64_t cnt
 }
 
 // Hub columns of A for the heavy symbolic pass: the threshold is the smallest
-// power of two >= kHubMinDeg whose hubs' bitmaps fit kHubBytes (one
-// histogram read-back).  No hubs (also when one hub's bitmap, rows / 8
+// power of two >= kHubMinDeg whose hubs' bitmaps fit kHubBytes.  No hubs (also when one hub's bitmap, rows / 8
 // bytes, exceeds kHubMaxSmem of shared memory): *hubbits stays NULL.
 constexpr int64_t kHubMinDeg = 1024;
 constexpr size_t kHubBytes = size_t(64) << 20;
 constexpr size_t kHubMaxSmem = size_t(192) << 10;  // bitmap words of one hub (rows / 8 bytes) at most
 
+// words of a hub bitmap: every base slab of the heavy items (a multiple of 4)
+static int64_t hub_words(const spg_plan *p) { return (int64_t)p->T * (p->R / 32); }
+
+// Launches only: the histogram rides on the plan's read-back.
+spg_status hub_histogram_queue(spg_plan *p) {
+    // a hub's bitmap is built in one CTA's shared memory
+    if (p->k == 0 || (size_t)hub_words(p) * sizeof(uint32_t) > kHubMaxSmem) return SPG_OK;
+    unsigned long long *hist = (unsigned long long *)ws_alloc(p, sizeof(unsigned long long) * 64);
+    if (!hist) return SPG_OUT_OF_MEMORY;
+    spg_status s = cuda_check(cudaMemsetAsync(hist, 0, sizeof(unsigned long long) * 64, p->st), "memset");
+    if (s) return s;
+    launch(p, k_deg_hist, grid_for(p->k, 256, p->sm_count * 4), 256, 0, p->A.colptr, p->A.ptr_type == SPG_IDX_I64,
+           p->k, hist);
+    for (int b = 0; b < 32; b++) p->h_pinned[kPinnedHist + b] = 0;
+    return cuda_check(cudaMemcpyAsync(p->h_pinned + kPinnedHist, hist, sizeof(int64_t) * 32, cudaMemcpyDeviceToHost,
+                                      p->st), "hub histogram");
+}
+void hub_histogram_read(spg_plan *p) {
+    if (p->k == 0 || (size_t)hub_words(p) * sizeof(uint32_t) > kHubMaxSmem) return;
+    for (int b = 0; b < 32; b++) p->hub_hist[b] = p->h_pinned[kPinnedHist + b];
+}
+
 static spg_status build_hubs(spg_plan *p, int32_t **hubidx, uint4 **hubbits, int64_t *Wa4) {
     *hubidx = nullptr;
     *hubbits = nullptr;
     *Wa4 = 0;
-    const int64_t k = p->k;
-    if (k == 0) return SPG_OK;
+    const int64_t k = p->k, Wa = hub_words(p);
+    if (k == 0 || (size_t)Wa * sizeof(uint32_t) > kHubMaxSmem) return SPG_OK;
     cudaStream_t st = p->st;
     const int ap64 = p->A.ptr_type == SPG_IDX_I64;
-    // words of a hub bitmap: every base slab of the heavy items (a multiple of 4)
-    const int64_t Wa = (int64_t)p->T * (p->R / 32);
-    // a hub's bitmap is built in one CTA's shared memory
-    if ((size_t)Wa * sizeof(uint32_t) > kHubMaxSmem) return SPG_OK;
-    unsigned long long *hist = (unsigned long long *)ws_alloc(p, sizeof(unsigned long long) * 64);
-    int *count = (int *)ws_alloc(p, sizeof(int) * 4);
-    if (!hist || !count) return SPG_OUT_OF_MEMORY;
-    spg_status s = cuda_check(cudaMemsetAsync(hist, 0, sizeof(unsigned long long) * 64, st), "memset");
-    if (s) return s;
-    launch(p, k_deg_hist, grid_for(k, 256, p->sm_count * 4), 256, 0, p->A.colptr, ap64, k, hist);
-    s = cuda_check(cudaMemcpyAsync(p->h_pinned + 16, hist, sizeof(int64_t) * 32, cudaMemcpyDeviceToHost, st),
-                   "hub histogram");
-    if (!s) s = cuda_check(cudaStreamSynchronize(st), "hub histogram");
-    if (s) return s;
+    spg_status s;
     int lg = 0;
     while ((int64_t(1) << lg) < kHubMinDeg) lg++;
     int64_t nh = 0;
     for (; lg < 32; lg++) {
         nh = 0;
-        for (int b = lg; b < 32; b++) nh += p->h_pinned[16 + b];
+        for (int b = lg; b < 32; b++) nh += p->hub_hist[b];
         if ((size_t)nh * (size_t)Wa * sizeof(uint32_t) <= kHubBytes) break;
     }
     if (nh == 0 || lg >= 32) return SPG_OK;
     int32_t *idx = (int32_t *)ws_alloc(p, sizeof(int32_t) * (size_t)k);
     int32_t *col = (int32_t *)ws_alloc(p, sizeof(int32_t) * (size_t)nh);
     uint32_t *bits = (uint32_t *)ws_alloc(p, sizeof(uint32_t) * (size_t)(nh * Wa));
-    if (!idx || !col || !bits) return SPG_OUT_OF_MEMORY;
+    int *count = (int *)ws_alloc(p, sizeof(int) * 4);
+    if (!idx || !col || !bits || !count) return SPG_OUT_OF_MEMORY;
     s = cuda_check(cudaMemsetAsync(count, 0, sizeof(int), st), "memset");
     if (s) return s;
     launch(p, k_hub_index, grid_for(k, 256, p->sm_count * 4), 256, 0, p->A.colptr, ap64, k, int64_t(1) << lg, idx,
@@ -377,14 +386,13 @@ static spg_status symbolic_heavy(spg_plan *p) {
            p->rec_off, p->nnzcol, p->num_cap, p->num_max_recs, nnum, (long long *)(p->d_cnt + kCntNnzCHeavySlot));
     spg_status s = scan_exclusive_i64(p, nnum, num_first, p->nheavy);
     if (s) return s;
+    // every item holds at least one record: the lists are sized by that bound
+    // and the count is read with nnz(C)
     s = cuda_check(cudaMemcpyAsync(p->h_pinned + 2, num_first + p->nheavy, sizeof(int64_t), cudaMemcpyDeviceToHost, st),
                    "numeric items");
     if (s) return s;
-    s = cuda_check(cudaStreamSynchronize(st), "numeric items");
-    if (s) return s;
-    p->nnum = p->h_pinned[2];
-    p->num_rec0 = (int32_t *)ws_alloc(p, sizeof(int32_t) * (size_t)(p->nnum + 1));
-    p->num_nrec = (int32_t *)ws_alloc(p, sizeof(int32_t) * (size_t)(p->nnum + 1));
+    p->num_rec0 = (int32_t *)ws_alloc(p, sizeof(int32_t) * (size_t)(p->nrec + 1));
+    p->num_nrec = (int32_t *)ws_alloc(p, sizeof(int32_t) * (size_t)(p->nrec + 1));
     if (!p->num_rec0 || !p->num_nrec) return SPG_OUT_OF_MEMORY;
     launch(p, k_num_items, gh, 256, 0, p->nheavy, p->rec_first, p->rec_cnt, p->num_cap, p->num_max_recs, num_first,
            p->num_rec0,
@@ -429,8 +437,14 @@ spg_status run_symbolic(spg_plan *p) {
     s = cuda_check(cudaMemcpyAsync(p->h_pinned + 1, p->d_cnt + kCntNnzCHeavySlot, sizeof(int64_t),
                                    cudaMemcpyDeviceToHost, st), "nnz readback");
     if (s) return s;
+    // the light columns' numeric bins and the number of heavy numeric items
+    // arrive with the same wait
+    s = queue_numeric_bins(p);
+    if (s) return s;
     s = read_dev_err(p, "symbolic");
     if (s) return s;
+    read_numeric_bins(p);
+    p->nnum = p->nrec > 0 ? p->h_pinned[2] : 0;
     p->nnzC = p->h_pinned[0];
     p->stats.nnzC = p->nnzC;
     p->stats.nnzC_heavy = p->h_pinned[1];
