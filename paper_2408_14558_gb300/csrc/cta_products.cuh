@@ -121,7 +121,7 @@ __device__ __forceinline__ EachProduct<F> each_product(F f) {
 // item's row range).  Ends with a barrier.
 static_assert(kLongSeg >= 32, "a 32-product window must meet at most two long segments");
 static_assert(kBatch * (kLongSeg - 1) <= 32 * kShortWindows, "segments below kLongSeg always fit the windows");
-static_assert(kBatch < 512 && kBatch * (kMidSeg - 1) < 65536 && kBatch * (kLongSeg - 1) < 32768,
+static_assert(kBatch < 1024 && kBatch * (kMidSeg - 1) < 65536 && kBatch * (kLongSeg - 1) < 32768,
               "the packed scan counters hold a batch");
 
 template <bool NEED_VAL, int U, typename Acc, typename SegFn, typename Body>

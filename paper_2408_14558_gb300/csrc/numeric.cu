@@ -96,6 +96,9 @@ __global__ void __launch_bounds__(WARPS * 32)
 // Slots of a numeric item's accumulator beyond its capacity: the guard slot,
 // and room to clear it 16 bytes at a time.
 constexpr int kAccPad = 4;
+// Rows of a direct item at most: its row list (2 bytes a row) sits in the rank
+// table's area behind the item's own words (8 bytes per 32 rows).
+constexpr int kDirectRows = kNumMaxWords * 8 * 4 / 9;
 
 // Everything a numeric item needs before its first product, in one record.
 struct NumItem {
@@ -135,8 +138,9 @@ __global__ void k_num_headers(int64_t nitems, const int32_t *__restrict__ num_re
 //     i + 1, and a row missing from a bitmap (never expected) still lands
 //     inside the accumulator.  Values and rows are written each as one
 //     coalesced run.
-//   direct items: the item's rows all have a slot (nr * R <= cap, the dense
-//     items, whose 4096 entries span one slab): a row's slot is its offset,
+//   direct items: the item's rows all have a slot (nr * R <= cap and
+//     kDirectRows, the dense items, whose 4096 entries span one slab): a row's
+//     slot is its offset,
 //     with no table look-up per product (and no conflicting look-ups: a
 //     segment's rows are distinct).
 // Thread 0 claims the next item when the current one starts and fetches its
@@ -201,7 +205,7 @@ __global__ void __launch_bounds__(kBatch, SPG_NUM_MINB)
         };
         const SegReg<Acc> first = cta_first_seg<Acc>(h.p0, h.p1, seg);
         const uint32_t *src = hbits + (int64_t)h.r0 * RW;
-        const bool direct = nr * R <= cap;
+        const bool direct = nr * R <= min(cap, kDirectRows);
         const int cnt = cta_load_rank_table<kNumMaxWords / (4 * kBatch)>(src, tab, nwords, ctot);
         const int64_t rbase = (int64_t)t0 * R;
         NumItem nh;
@@ -270,9 +274,8 @@ __global__ void __launch_bounds__(kBatch, SPG_NUM_MINB)
             const int v0 = tid - (int)(((uintptr_t)cval / sizeof(Acc)) & 31);
             const int r0 = tid - (int)(((uintptr_t)crow / sizeof(OutIdx)) & 31);
             if (direct) {
-                // the rows by rank (16-bit offsets behind the item's words:
-                // tab holds kNumMaxWords words and a direct item needs
-                // nr * R / 32 of them), then values and rows as coalesced runs
+                // the rows by rank (16-bit offsets behind the item's words),
+                // then values and rows as coalesced runs
                 uint16_t *srow = (uint16_t *)(tab + nwords);
                 for (int w = wid; w < nwords; w += nw) {
                     const uint2 e = tab[w];

@@ -460,7 +460,10 @@ constexpr int kBatch = SPG_HEAVY_THREADS;
 // own, those below kLongSeg always through the windows of the staging area,
 // those between as far as the windows go.
 constexpr int kLongSeg = 32;
-constexpr int kMidSeg = 256;
+#ifndef SPG_MID_SEG
+#define SPG_MID_SEG 256
+#endif
+constexpr int kMidSeg = SPG_MID_SEG;
 constexpr int kShortWindows = (kBatch * (kLongSeg - 1) + 31) / 32;
 
 __device__ __forceinline__ unsigned hash_row(int r, int shift) {

@@ -34,6 +34,7 @@ SHAPES = {
     "one_each": ([1, 31, 32, 33, 127, 128, 129, 255, 256, 257, 511, 1000], [12, 11, 5], 30000),
     "dense_item": ([31, 32, 500, 1000] * 70, [280, 256, 9], 1024),
     "dense_item_ragged": ([7, 300, 64] * 90, [270, 13], 3001),
+    "dense_slabs": ([3000, 255, 31] * 60, [180, 150], 20000),
 }
 
 
@@ -44,7 +45,7 @@ def test_walk_edges_match_oracle(shape, values):
     rng = np.random.default_rng(11)
     A = columns(lens, m, rng, values)
     B = columns(nb, len(lens), rng, values)
-    for R in (1024, 4096):
+    for R in (1024, 4096, 8192, 16384):
         C = run_gpu(A, B, 2, 64, light_max=32, slab_rows=R)
         assert_full_parity(C, oracle.spgemm(A, B), f"{shape} {values} R={R}")
 
