@@ -49,14 +49,27 @@ __global__ void k_bc_init(const int32_t *src, int s, int64_t W, int64_t *colptr,
     }
 }
 
-__global__ void k_bc_mark(const int64_t *Fcp, const void *Frow, int i64, int64_t s, uint32_t *V, int64_t W) {
-    const int lane = threadIdx.x & 31;
-    for (int64_t j = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; j < s;
-         j += ((int64_t)gridDim.x * blockDim.x) >> 5)
-        for (int64_t e = Fcp[j] + lane; e < Fcp[j + 1]; e += 32) {
-            const int64_t r = ld_ptr(Frow, i64, e);
-            atomicOr(V + j * W + (r >> 5), 1u << (r & 31));
+// The warps of a frontier kernel: column j's entries in pieces of kBcPiece, one
+// warp each (blockIdx.y-th CTA row of a column takes every gridDim.y-th group
+// of pieces).  A batch has few columns of up to n entries: one warp per column
+// left most of the GPU idle (1024 columns of 22,000 entries: marking 0.5 ms,
+// the dependencies 2.5 ms a level; 0.1 and 0.3 ms in pieces).
+constexpr int kBcPiece = 256, kBcWarps = 8;
+
+__global__ void __launch_bounds__(32 * kBcWarps)
+    k_bc_mark(const int64_t *Fcp, const void *Frow, int i64, int64_t s, uint32_t *V, int64_t W) {
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    for (int64_t j = blockIdx.x; j < s; j += gridDim.x) {
+        const int64_t f1 = Fcp[j + 1];
+        for (int64_t p0 = Fcp[j] + (int64_t)(blockIdx.y * kBcWarps + wid) * kBcPiece; p0 < f1;
+             p0 += (int64_t)gridDim.y * kBcWarps * kBcPiece) {
+            const int64_t p1 = min(f1, p0 + kBcPiece);
+            for (int64_t e = p0 + lane; e < p1; e += 32) {
+                const int64_t r = ld_ptr(Frow, i64, e);
+                atomicOr(V + j * W + (r >> 5), 1u << (r & 31));
+            }
         }
+    }
 }
 
 __global__ void k_bc_weights(const double *sigma, const double *delta, int64_t nnz, double *w) {
@@ -64,30 +77,58 @@ __global__ void k_bc_weights(const double *sigma, const double *delta, int64_t n
         w[i] = (1.0 + (delta ? delta[i] : 0.0)) / sigma[i];
 }
 
-// delta(v, j) = T(v, j) * sigma(v, j) over F(:, j)'s entries (T's column,
-// whose rows are a subset of F's, is searched for row v); added into bc[v]
-// when `add`.
-__global__ void k_bc_delta(const int64_t *Fcp, const void *Frow, const double *Fsig, const int64_t *Tcp,
-                           const void *Trow, const double *Tval, int i64, int64_t s, double *delta, double *bc,
-                           int add) {
-    const int lane = threadIdx.x & 31;
-    for (int64_t j = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; j < s;
-         j += ((int64_t)gridDim.x * blockDim.x) >> 5) {
-        const int64_t t0 = Tcp[j], t1 = Tcp[j + 1];
-        for (int64_t e = Fcp[j] + lane; e < Fcp[j + 1]; e += 32) {
-            const int64_t r = ld_ptr(Frow, i64, e);
-            int64_t lo = t0, hi = t1;
-            while (lo < hi) {
-                const int64_t mid = (lo + hi) >> 1;
-                if (ld_ptr(Trow, i64, mid) < r)
-                    lo = mid + 1;
-                else
-                    hi = mid;
+// delta(v, j) = T(v, j) * sigma(v, j) over F(:, j)'s entries; added into bc[v]
+// when `add`.  T's column holds a subset of F's rows, both ascending: a warp
+// finds the first T row of its piece of F once (32-way search), then 32 entries
+// of F meet at most the next 32 of T, which the lanes load together and search
+// by shuffles.
+__global__ void __launch_bounds__(32 * kBcWarps)
+    k_bc_delta(const int64_t *Fcp, const void *Frow, const double *Fsig, const int64_t *Tcp, const void *Trow,
+               const double *Tval, int i64, int64_t s, double *delta, double *bc, int add) {
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    for (int64_t j = blockIdx.x; j < s; j += gridDim.x) {
+        const int64_t f1 = Fcp[j + 1], t1 = Tcp[j + 1];
+        for (int64_t p0 = Fcp[j] + (int64_t)(blockIdx.y * kBcWarps + wid) * kBcPiece; p0 < f1;
+             p0 += (int64_t)gridDim.y * kBcWarps * kBcPiece) {
+            const int64_t p1 = min(f1, p0 + kBcPiece);
+            // lo: the first entry of T whose row is >= the piece's first row
+            const int64_t r0 = ld_ptr(Frow, i64, p0);
+            int64_t lo = Tcp[j], hi = t1;
+            while (hi - lo > 0) {
+                const int64_t step = (hi - lo + 31) >> 5;
+                const int64_t at = lo + lane * step;
+                const uint32_t below = __ballot_sync(kFull, at < hi && ld_ptr(Trow, i64, at) < r0);
+                if (below == 0) {
+                    hi = lo;
+                } else {  // lanes below form a prefix: the answer lies behind the last of them
+                    const int64_t last = lo + (31 - __clz(below)) * step;
+                    hi = min(hi, last + step);
+                    lo = last + 1;
+                }
             }
-            const double t = (lo < t1 && ld_ptr(Trow, i64, lo) == r) ? Tval[lo] : 0.0;
-            const double d = t * Fsig[e];
-            delta[e] = d;
-            if (add && d != 0.0) atomicAdd(bc + r, d);
+            for (int64_t e0 = p0; e0 < p1; e0 += 32) {
+                const int64_t e = e0 + lane;
+                const bool valid = e < p1;
+                const int64_t r = valid ? ld_ptr(Frow, i64, e) : INT64_MAX;
+                const int64_t tq = lo + lane;
+                const int64_t tr = tq < t1 ? ld_ptr(Trow, i64, tq) : INT64_MAX;
+                const double tv = tq < t1 ? Tval[tq] : 0.0;
+                int pos = 0;  // T rows of the window below r
+#pragma unroll
+                for (int stp = 16; stp > 0; stp >>= 1) {
+                    const int64_t x = __shfl_sync(kFull, tr, pos + stp - 1);
+                    if (x < r) pos += stp;
+                }
+                const int64_t x = __shfl_sync(kFull, tr, pos & 31);
+                const double t = __shfl_sync(kFull, tv, pos & 31);
+                if (valid) {
+                    const double d = (x == r ? t : 0.0) * Fsig[e];
+                    delta[e] = d;
+                    if (add && d != 0.0) atomicAdd(bc + r, d);
+                }
+                const int64_t rlast = __shfl_sync(kFull, r, (int)min((int64_t)31, p1 - e0 - 1));
+                lo += __popc(__ballot_sync(kFull, tr <= rlast));
+            }
         }
     }
 }
@@ -125,6 +166,13 @@ struct BcRun {
         ws_free_all(&w);
     }
 };
+
+// CTAs of a frontier kernel: the columns times the pieces of a mean column.
+dim3 bc_grid(int64_t s, int64_t nnz) {
+    const int64_t per = (int64_t)kBcWarps * kBcPiece;
+    const int64_t y = std::max<int64_t>(1, std::min<int64_t>(64, (nnz / std::max<int64_t>(s, 1) + per - 1) / per));
+    return dim3((unsigned)std::min<int64_t>(s, 65535), (unsigned)y);
+}
 
 spg_status multiply_f64(const spg_csc *A, const spg_csc *B, const spg_options *opt, spg_csc *C, int64_t *products,
                         spg_bc_stats *S) {
@@ -239,12 +287,13 @@ extern "C" spg_status spgemm_bc_batch(const spg_csc *A, const int32_t *sources, 
             while (true) {
                 spg_csc T{};
                 BC_TRY(multiply_f64(&G, &run.F.back(), &fo, &T, &S.products_forward, &S));
+                fo.validate = 0;  // A has been checked; the frontiers are this library's
                 if (T.nnz == 0) {
                     run.free_csc(T);
                     break;
                 }
-                launch(w, k_bc_mark, grid_for(s * 32, 256, sm * 16), 256, 0, (const int64_t *)T.colptr, T.rowidx,
-                       i64, (int64_t)s, V, W);
+                launch(w, k_bc_mark, bc_grid(s, T.nnz), 32 * kBcWarps, 0, (const int64_t *)T.colptr, T.rowidx, i64,
+                       (int64_t)s, V, W);
                 run.F.push_back(T);
                 BC_TRY(cuda_check(cudaGetLastError(), "frontier kernels"));
                 S.frontier_nnz += T.nnz;
@@ -262,12 +311,13 @@ extern "C" spg_status spgemm_bc_batch(const spg_csc *A, const int32_t *sources, 
                    (const double *)run.delta[d], Wd.nnz, (double *)Wd.vals);
             const spg_csc &Fp = run.F[d - 1];
             BC_TRY(cuda_check(cudaMemsetAsync(Mb, 0, sizeof(uint32_t) * (size_t)(s * W + 1), st), "memset"));
-            launch(w, k_bc_mark, grid_for(s * 32, 256, sm * 16), 256, 0, (const int64_t *)Fp.colptr, Fp.rowidx, i64,
+            launch(w, k_bc_mark, bc_grid(s, Fp.nnz), 32 * kBcWarps, 0, (const int64_t *)Fp.colptr, Fp.rowidx, i64,
                    (int64_t)s, Mb, W);
             spg_options bo = *opt;
             bo.mask = Mb;
             bo.mask_words = W;
             bo.mask_complement = 0;
+            bo.validate = 0;
             spg_csc T{};
             BC_TRY(multiply_f64(&G, &Wd, &bo, &T, &S.products_backward, &S));
             run.delta[d - 1] = (double *)alloc_user(opt, 8 * (size_t)std::max<int64_t>(Fp.nnz, 1));
@@ -275,7 +325,7 @@ extern "C" spg_status spgemm_bc_batch(const spg_csc *A, const int32_t *sources, 
                 run.free_csc(T);
                 BC_TRY(SPG_OUT_OF_MEMORY);
             }
-            launch(w, k_bc_delta, grid_for(s * 32, 256, sm * 16), 256, 0, (const int64_t *)Fp.colptr, Fp.rowidx,
+            launch(w, k_bc_delta, bc_grid(s, Fp.nnz), 32 * kBcWarps, 0, (const int64_t *)Fp.colptr, Fp.rowidx,
                    (const double *)Fp.vals, (const int64_t *)T.colptr, T.rowidx, (const double *)T.vals, i64,
                    (int64_t)s, run.delta[d - 1], bc, (int)(d - 1 >= 1));
             rc = cuda_check(cudaGetLastError(), "backward kernels");

@@ -596,37 +596,15 @@ __device__ __forceinline__ int light_bin(long long U, int light_max) {
     return bin;
 }
 
-// Per output column: flops_j, the row window of its products, the MLP features
-// and the symbolic bin (bound U = min(flops_j, window)).  A warp takes four
-// columns, eight lanes each with four entries in flight per lane; a column of
-// more than kStatsLong entries is done by the whole warp afterwards.  (A warp
-// per column: 262,144 columns of 8 entries 85 us, of 32 entries 140 us, most
-// lanes or loads idle; 16 lanes per column whatever its length: a skewed graph
-// of 100,003 columns 170 us instead of 97.)
-constexpr int kStatsLong = 64;
-
-__global__ void k_col_stats(const void *Bcolptr, int p64, int64_t n, const int32_t *Bq,
-                            const int64_t *At_colptr, const int32_t *At_row, int light_max,
-                            int64_t *flops, int32_t *win_lo, int32_t *win_hi, int32_t *nnzb,
-                            int32_t *maxa, int8_t *bin_of, long long *bincnt, long long *products) {
-    __shared__ int hist[kNumBins];
-    __shared__ long long prod_sh;
-    if (threadIdx.x < kNumBins) hist[threadIdx.x] = 0;
-    if (threadIdx.x == 0) prod_sh = 0;
-    __syncthreads();
-    const int lane = threadIdx.x & 31, gl = lane & 7;
-    const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
-    long long prod_local = 0;
-    long long fl;
-    int mx, lo, hi;
-    // this lane's share of the entries s + first, s + first + stride, ... of a
-    // column (each stage's loads issued together: long columns would otherwise
-    // be a chain of dependent loads)
-    auto walk = [&](int64_t s, int64_t e, int first, int stride) {
-        fl = 0;
-        mx = 0;
-        lo = INT32_MAX;
-        hi = -1;
+// Statistics of one output column, reduced over some lanes.
+struct ColStat {
+    long long fl = 0;                     // flops_j
+    int mx = 0, lo = INT32_MAX, hi = -1;  // longest A~ column, row window
+    // the entries q = s + first, s + first + stride, ... < e of B' (each stage's
+    // loads issued together: long columns would otherwise be a chain of
+    // dependent loads)
+    __device__ __forceinline__ void walk(int64_t s, int64_t e, int first, int stride, const int32_t *Bq,
+                                         const int64_t *At_colptr, const int32_t *At_row) {
         for (int64_t q0 = s + first; q0 < e; q0 += stride * 4) {
             int loc[4];
             int64_t a0[4], a1[4];
@@ -648,45 +626,110 @@ __global__ void k_col_stats(const void *Bcolptr, int p64, int64_t n, const int32
                 }
             }
         }
-    };
-    auto reduce = [&](int o) {
-        fl += __shfl_xor_sync(kFull, fl, o);
-        mx = max(mx, __shfl_xor_sync(kFull, mx, o));
-        lo = min(lo, __shfl_xor_sync(kFull, lo, o));
-        hi = max(hi, __shfl_xor_sync(kFull, hi, o));
-    };
-    auto store = [&](int64_t j, int64_t len) {
-        flops[j] = fl;
-        win_lo[j] = fl ? lo : 0;
-        win_hi[j] = fl ? hi : -1;
-        nnzb[j] = (int32_t)len;
-        maxa[j] = mx;
-        long long U = fl ? min(fl, (long long)(hi - lo + 1)) : 0;
-        int bin = light_bin(U, light_max);
-        bin_of[j] = (int8_t)bin;
-        atomicAdd(&hist[bin], 1);
-        prod_local += fl;
-    };
-    for (int64_t j0 = 4 * (((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5); j0 < n; j0 += 4 * nwarps) {
-        const int64_t j = j0 + (lane >> 3);
-        const bool valid = j < n;
-        const int64_t s = valid ? ld_ptr(Bcolptr, p64, j) : 0, e = valid ? ld_ptr(Bcolptr, p64, j + 1) : 0;
-        const bool is_long = e - s > kStatsLong;
-        walk(s, is_long ? s : e, gl, 8);
-        reduce(4);
-        reduce(2);
-        reduce(1);
-        if (gl == 0 && valid && !is_long) store(j, e - s);
-        for (uint32_t todo = __ballot_sync(kFull, gl == 0 && is_long); todo; todo &= todo - 1u) {
-            const int src = __ffs((int)todo) - 1;
-            const int64_t js = j0 + (src >> 3), ss = __shfl_sync(kFull, s, src), es = __shfl_sync(kFull, e, src);
-            walk(ss, es, lane, 32);
-#pragma unroll
-            for (int o = 16; o > 0; o >>= 1) reduce(o);
-            if (lane == 0) store(js, es - ss);
+    }
+    __device__ __forceinline__ void join(const ColStat &o) {
+        fl += o.fl;
+        mx = max(mx, o.mx);
+        lo = min(lo, o.lo);
+        hi = max(hi, o.hi);
+    }
+    // over lane groups of 2 * `from` lanes (every lane of the warp calls it)
+    __device__ __forceinline__ void reduce(int from) {
+        for (int o = from; o > 0; o >>= 1) {
+            ColStat t;
+            t.fl = __shfl_xor_sync(kFull, fl, o);
+            t.mx = __shfl_xor_sync(kFull, mx, o);
+            t.lo = __shfl_xor_sync(kFull, lo, o);
+            t.hi = __shfl_xor_sync(kFull, hi, o);
+            join(t);
         }
     }
-    if (gl == 0 && prod_local) atomicAdd((unsigned long long *)&prod_sh, (unsigned long long)prod_local);
+};
+struct ColStatOut {
+    int64_t *flops;
+    int32_t *win_lo, *win_hi, *nnzb, *maxa;
+    int8_t *bin_of;
+    int light_max;
+    __device__ __forceinline__ int store(const ColStat &c, int64_t j, int64_t len) const {
+        flops[j] = c.fl;
+        win_lo[j] = c.fl ? c.lo : 0;
+        win_hi[j] = c.fl ? c.hi : -1;
+        nnzb[j] = (int32_t)len;
+        maxa[j] = c.mx;
+        const long long U = c.fl ? min(c.fl, (long long)(c.hi - c.lo + 1)) : 0;
+        const int bin = light_bin(U, light_max);
+        bin_of[j] = (int8_t)bin;
+        return bin;
+    }
+};
+
+// Per output column: flops_j, the row window of its products, the MLP features
+// and the symbolic bin (bound U = min(flops_j, window)).  A warp takes four
+// columns, eight lanes each with four entries in flight per lane; a column of
+// more than kStatsLong entries is done by the whole warp afterwards.  (A warp
+// per column: 262,144 columns of 8 entries 85 us, of 32 entries 140 us, most
+// lanes or loads idle; 16 lanes per column whatever its length: a skewed graph
+// of 100,003 columns 170 us instead of 97.)  CTA: one column per CTA, for few
+// and long columns (mean above kStatsWide entries: the betweenness frontiers,
+// 1024 columns of up to 22,000).
+constexpr int kStatsLong = 64, kStatsWide = 512;
+
+template <bool CTA>
+__global__ void __launch_bounds__(256)
+    k_col_stats(const void *Bcolptr, int p64, int64_t n, const int32_t *Bq, const int64_t *At_colptr,
+                const int32_t *At_row, ColStatOut out, long long *bincnt, long long *products) {
+    __shared__ int hist[kNumBins];
+    __shared__ long long prod_sh;
+    __shared__ ColStat part[8];
+    if (threadIdx.x < kNumBins) hist[threadIdx.x] = 0;
+    if (threadIdx.x == 0) prod_sh = 0;
+    __syncthreads();
+    const int lane = threadIdx.x & 31, gl = lane & 7, wid = threadIdx.x >> 5;
+    long long prod_local = 0;
+    if (CTA) {
+        for (int64_t j = blockIdx.x; j < n; j += gridDim.x) {
+            const int64_t s = ld_ptr(Bcolptr, p64, j), e = ld_ptr(Bcolptr, p64, j + 1);
+            ColStat c;
+            c.walk(s, e, threadIdx.x, blockDim.x, Bq, At_colptr, At_row);
+            c.reduce(16);
+            if (lane == 0) part[wid] = c;
+            __syncthreads();
+            if (threadIdx.x == 0) {
+                for (int w = 1; w < 8; w++) c.join(part[w]);
+                hist[out.store(c, j, e - s)]++;
+                prod_local += c.fl;
+            }
+            __syncthreads();
+        }
+    } else {
+        const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
+        for (int64_t j0 = 4 * (((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5); j0 < n; j0 += 4 * nwarps) {
+            const int64_t j = j0 + (lane >> 3);
+            const bool valid = j < n;
+            const int64_t s = valid ? ld_ptr(Bcolptr, p64, j) : 0, e = valid ? ld_ptr(Bcolptr, p64, j + 1) : 0;
+            const bool is_long = e - s > kStatsLong;
+            ColStat c;
+            c.walk(s, is_long ? s : e, gl, 8, Bq, At_colptr, At_row);
+            c.reduce(4);
+            if (gl == 0 && valid && !is_long) {
+                atomicAdd(&hist[out.store(c, j, e - s)], 1);
+                prod_local += c.fl;
+            }
+            for (uint32_t todo = __ballot_sync(kFull, gl == 0 && is_long); todo; todo &= todo - 1u) {
+                const int src = __ffs((int)todo) - 1;
+                const int64_t js = j0 + (src >> 3);
+                const int64_t ss = __shfl_sync(kFull, s, src), es = __shfl_sync(kFull, e, src);
+                ColStat l;
+                l.walk(ss, es, lane, 32, Bq, At_colptr, At_row);
+                l.reduce(16);
+                if (lane == 0) {
+                    atomicAdd(&hist[out.store(l, js, es - ss)], 1);
+                    prod_local += l.fl;
+                }
+            }
+        }
+    }
+    if (prod_local) atomicAdd((unsigned long long *)&prod_sh, (unsigned long long)prod_local);
     __syncthreads();
     if (threadIdx.x < kNumBins && hist[threadIdx.x])
         atomicAdd((unsigned long long *)&bincnt[threadIdx.x], (unsigned long long)hist[threadIdx.x]);
@@ -1120,9 +1163,12 @@ static spg_status plan_build(spg_plan *p) {
         return dev_err_read(p, "plan");
     };
     if (n > 0) {
-        launch(p, k_col_stats, grid_for(n * 8, 256, sm * 16), 256, 0, B.colptr, p64B, n, p->Bq, p->At_colptr,
-               p->At_row, p->light_max, p->flops, p->win_lo, p->win_hi, p->nnzb, p->maxa, p->bin_of,
-               (long long *)(p->d_cnt + kCntBin0), (long long *)(p->d_cnt + kCntProducts));
+        const ColStatOut out{p->flops, p->win_lo, p->win_hi, p->nnzb, p->maxa, p->bin_of, p->light_max};
+        const bool wide = B.nnz / kStatsWide > n;
+        launch(p, wide ? k_col_stats<true> : k_col_stats<false>,
+               wide ? grid_for(n, 1, sm * 8) : grid_for(n * 8, 256, sm * 16), 256, 0, B.colptr, p64B, n, p->Bq,
+               p->At_colptr, p->At_row, out, (long long *)(p->d_cnt + kCntBin0),
+               (long long *)(p->d_cnt + kCntProducts));
         launch(p, k_block_flops, grid_for(n, 256, sm * 8), 256, 0, p->flops, n, P, p->bounds_d, (long long *)p->blk);
         LAUNCH_OK("column stats");
         TRY(bin_columns_queue(p, p->bin_of, p->binlist));

@@ -91,3 +91,20 @@ def test_nan_and_infinities_stay_where_they_belong():
         mag = sum(np.abs(np.where(np.isfinite(dense[:, k]), dense[:, k], 0.0) * x) for k, x in zip(ks, bv))
         assert np.all(np.abs(got[fine] - want[fine]) <= 1e-12 * mag[ri[cp[j]:cp[j + 1]]][fine])
         assert np.array_equal(got[np.isinf(want)], want[np.isinf(want)])
+
+
+@pytest.mark.parametrize("n,s", [(9000, 3), (700, 40)])
+def test_betweenness_on_long_and_short_frontiers(n, s):
+    """Frontier columns of several pieces (256 entries a warp) and shorter than one."""
+    from oracle import bc as obc
+    rng = np.random.default_rng(14)
+    r, c = rng.integers(0, n, 6 * n), rng.integers(0, n, 6 * n)
+    keep = r != c
+    cols, rows = synth._sort_dedup(np.concatenate([c[keep], r[keep]]), np.concatenate([r[keep], c[keep]]), n)
+    A = synth._csc_from_sorted(n, n, cols, rows, np.ones(cols.size))
+    src = rng.choice(n, s, replace=False).astype(np.int32)
+    bc, _, _ = g.spgemm_bc_batch(g.to_device(A), torch.from_numpy(src).cuda(), P=2, b=64)
+    want = obc.brandes(A, src)
+    want = want[0] if isinstance(want, tuple) else want
+    got = bc.cpu().numpy()
+    assert np.all(np.abs(got - want) <= 1e-9 * np.maximum(1.0, np.abs(want)))

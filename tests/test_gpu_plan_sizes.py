@@ -80,3 +80,14 @@ def test_validation_finds_a_bad_row_at_every_alignment(offset, at):
         assert e.value.status == g.SPG_INVALID_INPUT
         row[at] = keep
     assert_full_parity(g.multiply(M, M, 2, 16), oracle.spgemm(A, A), "restored")
+
+
+@pytest.mark.parametrize("lens", [[520] * 30, [700, 0, 4000, 1, 513] * 4])
+def test_long_columns_of_B(lens):
+    """A mean above 512 entries per column of B: one CTA per column in the statistics."""
+    rng = np.random.default_rng(6)
+    A = banded(5000, 5000, 3, rng)
+    cols = np.repeat(np.arange(len(lens)), lens)
+    rows = np.concatenate([np.sort(rng.choice(5000, k, replace=False)) for k in lens])
+    B = synth._csc_from_sorted(5000, len(lens), cols, rows, rng.uniform(-1, 1, rows.size))
+    assert_full_parity(run_gpu(A, B, 3, 64), oracle.spgemm(A, B), "long columns of B")
