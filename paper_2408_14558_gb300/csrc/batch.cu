@@ -37,6 +37,7 @@
 #include "block_ops.cuh"
 #include "cta_products.cuh"
 #include "spg_internal.cuh"
+#include "warp_hash.cuh"
 
 namespace spg {
 
@@ -184,14 +185,9 @@ __global__ void k_batch_persistent(const BatchInst *__restrict__ insts, const Ba
                                    Acc *__restrict__ out_val, int *err, long long timeout_ns, int stall_inst,
                                    const uint8_t *__restrict__ heavy_col) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    constexpr int S_MAX = 1 << LOGS_MAX;
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nwarps = blockDim.x >> 5;
     WarpSeg<Acc> *segs = (WarpSeg<Acc> *)smem_raw;
-    Acc *vals_all = (Acc *)(segs + nwarps);
-    int *keys_all = (int *)(vals_all + nwarps * S_MAX);
-    int *keys = keys_all + wid * S_MAX;
-    Acc *vals = vals_all + wid * S_MAX;
-    int *hist = keys_all + nwarps * S_MAX + wid * 256;
+    unsigned char *area = (unsigned char *)(segs + nwarps) + wid * WarpTable<Acc>::bytes(LOGS_MAX);
     WarpSeg<Acc> &ws = segs[wid];
     while (true) {
         unsigned long long t = 0;
@@ -212,26 +208,19 @@ __global__ void k_batch_persistent(const BatchInst *__restrict__ insts, const Ba
             for (int j = tk.c0; j < tk.c1; j++) {
                 if (heavy_col[colb + j]) continue;  // counted by the heavy kernel
                 const int64_t p0 = ld_ptr(in.Bcp, in.bcp64, j), p1 = ld_ptr(in.Bcp, in.bcp64, j + 1);
-                // twice the class's largest table, in the warp's value area
-                // (8 bytes per slot of the numeric table: room for 2 x S_MAX
-                // row ids): every column's bound min(flops, m) is <= S_MAX / 2,
-                // so the load factor stays <= 1/4 (a table sized from the
-                // column's own bound probes more: slower)
-                static_assert(sizeof(Acc) == 2 * sizeof(int), "the value area holds 2 x S_MAX row ids");
-                const int logS = LOGS_MAX + 1;
-                const int S = 1 << logS;
-                int *skeys = (int *)vals;
-                for (int s = lane; s < S; s += 32) skeys[s] = kEmptyKey;
+                // twice the class's table, over its values: every column's bound
+                // min(flops, m) is at most a quarter of it
+                constexpr int logS = LOGS_MAX + 1;
+                int *skeys = (int *)area;
+                warp_clear_keys(skeys, logS, lane);
                 __syncwarp();
-                int cnt = 0;
                 bool full = false;
-                warp_products<false, Acc>(
-                    p0, p1, lane, ws, in.Arow, (const Acc *)nullptr, seg, [&](int r, Acc) {
-                        bool fresh;
-                        if (hash_insert(skeys, logS, r, &fresh) < 0) full = true;
-                        cnt += fresh ? 1 : 0;
+                warp_walk<false, 4, Acc>(
+                    p0, p1, lane, ws, in.Arow, seg, [](long long) { return Acc(0); },
+                    [&](int r, Acc, Acc, bool ok) {
+                        if (warp_hash_slot(skeys, logS, r, ok) < 0 && ok) full = true;
                     });
-                cnt = warp_sum_i(cnt);
+                const int cnt = warp_count_keys(skeys, logS, lane);
                 if (__any_sync(kFull, full) && lane == 0) atomicOr(err, kDevErrInternal);
                 if (lane == 0) nnz[colb + j] = cnt;
                 __syncwarp();
@@ -258,51 +247,27 @@ __global__ void k_batch_persistent(const BatchInst *__restrict__ insts, const Ba
                 const int64_t p0 = ld_ptr(in.Bcp, in.bcp64, j), p1 = ld_ptr(in.Bcp, in.bcp64, j + 1);
                 // >= 4 x the column's count (at most the class's table): a
                 // sparser table probes less, which outweighs clearing more
-                const int logS = min(LOGS_MAX, log_table(want > 0 ? want : 1) + 1);
-                const int S = 1 << logS;
-                for (int s = lane; s < S; s += 32) {
-                    keys[s] = kEmptyKey;
-                    vals[s] = Acc(0);
-                }
-                __syncwarp();
+                const WarpTable<Acc> tab(area, min(LOGS_MAX, log_table(want > 0 ? want : 1) + 1));
+                const HeavyAcc<Acc> acc = tab.acc();
+                tab.clear(lane);
                 bool full = false;
                 // A's values may be stored as double, int32 or int64
-                warp_products_v<true, 4, Acc>(
+                warp_walk<true, 4, Acc>(
                     p0, p1, lane, ws, in.Arow, seg,
                     [&](long long e) { return bval_load<Acc>(in.Aval, in.vt, e); },
-                    [&](int r, Acc v) {
-                        bool fresh;
-                        const int slot = hash_insert(keys, logS, r, &fresh);
-                        if (slot < 0)
-                            full = true;
-                        else
-                            atomic_add_acc(vals + slot, v);
+                    [&](int r, Acc a, Acc b, bool ok) {
+                        if (!tab.add(acc, r, a, b, ok)) full = true;
                     });
                 __syncwarp();
-                int nout = 0;
-                for (int c0 = 0; c0 < S; c0 += 32) {
-                    const int kk = keys[c0 + lane];
-                    const Acc vv = vals[c0 + lane];
-                    const bool occ = kk != kEmptyKey;
-                    const unsigned bal = __ballot_sync(kFull, occ);
-                    __syncwarp();
-                    if (occ) {
-                        const int pos = nout + __popc(bal & ((1u << lane) - 1u));
-                        keys[pos] = kk;
-                        vals[pos] = vv;
-                    }
-                    nout += __popc(bal);
-                    __syncwarp();
-                }
+                const int nout = tab.compact(acc, lane);
                 full = __any_sync(kFull, full);
                 if (full || nout != want) {
                     if (lane == 0) atomicOr(err, kDevErrInternal);
                 } else {
-                    warp_sort_pairs<Acc>(keys, vals, nout, S, hist, lane);
-                    for (int s = lane; s < nout; s += 32) {
-                        out_row[base + s] = (OutIdx)keys[s];
-                        out_val[base + s] = vals[s];
-                    }
+                    tab.emit(acc, nout, lane, [&](int pos, int row, Acc v) {
+                        out_row[base + pos] = (OutIdx)row;
+                        out_val[base + pos] = v;
+                    });
                 }
                 __syncwarp();
             }
@@ -514,21 +479,33 @@ static spg_status batch_launch_class(spg_batch *b, int c, cudaStream_t st) {
     const int64_t t0 = b->class_off[c], nt = b->class_off[c + 1] - t0;
     if (nt == 0) return SPG_OK;
     auto kern = k_batch_persistent<LOGS_MAX, Acc, OutIdx>;
-    const size_t smem = sizeof(WarpSeg<double>) * (size_t)b->warps +
-                        (8 + sizeof(int)) * (size_t)b->warps * (1u << LOGS_MAX) + sizeof(int) * 256 * (size_t)b->warps;
+    // tables of 6, 12 and 24 KB a warp: from half the asked warps per CTA up, the
+    // number that brings most warps onto an SM (what bounds the kernel: 8
+    // resident warps issue in 20% of the cycles)
+    constexpr size_t per_warp = sizeof(WarpSeg<Acc>) + WarpTable<Acc>::bytes(LOGS_MAX);
+    int warps = 0, resident = 0;
+    for (int w = b->warps; w >= b->warps / 2; w--) {
+        const size_t cta = per_warp * (size_t)w;
+        const int r = cta > (size_t(227) << 10) ? 0 : w * (int)((size_t(228) << 10) / (cta + 1024));
+        if (r > resident) {
+            resident = r;
+            warps = w;
+        }
+    }
+    const size_t smem = per_warp * (size_t)warps;
     spg_status s = cuda_check(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem),
                               "batch smem");
     if (s) return s;
     int occ = 0;
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kern, b->warps * 32, smem);
+    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kern, warps * 32, smem);
     if (occ < 1) {
-        set_error("batch kernel does not fit on an SM with %d warps", b->warps);
+        set_error("batch kernel does not fit on an SM with %d warps", warps);
         return SPG_UNSUPPORTED;
     }
     const int grid = b->sm_count * occ;
     b->grid = std::max(b->grid, grid);
     b->smem = std::max(b->smem, smem);
-    kern<<<grid, b->warps * 32, smem, st>>>(
+    kern<<<grid, warps * 32, smem, st>>>(
         b->insts, b->tasks + t0, nt, b->head + c, b->sym_done, b->ready, b->nnz, b->colptr, (OutIdx *)b->out_row,
         (Acc *)b->out_val, b->err, b->opt.timeout_ns, b->opt.stall_instance, b->heavy_col);
     return cuda_check(cudaGetLastError(), "batch kernel launch");

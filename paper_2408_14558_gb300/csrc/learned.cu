@@ -28,6 +28,7 @@
 #include "block_ops.cuh"
 #include "cta_products.cuh"
 #include "spg_internal.cuh"
+#include "warp_hash.cuh"
 
 namespace spg {
 
@@ -235,26 +236,18 @@ __global__ void __launch_bounds__(WARPS * 32)
                     const Acc *__restrict__ At_val, const int64_t *__restrict__ capoff,
                     const int64_t *__restrict__ cap, int64_t *__restrict__ nnz, int32_t *flag,
                     unsigned long long *nflag, OutIdx *__restrict__ trow, Acc *__restrict__ tval) {
-    constexpr int S = 1 << LOGS;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     WarpSeg<Acc> *segs = (WarpSeg<Acc> *)smem_raw;
-    Acc *vals_all = (Acc *)(segs + WARPS);
-    int *keys_all = (int *)(vals_all + WARPS * S);
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-    int *keys = keys_all + wid * S;
-    Acc *vals = vals_all + wid * S;
-    int *hist = keys_all + WARPS * S + wid * 256;
+    const WarpTable<Acc> tab((unsigned char *)(segs + WARPS) + wid * WarpTable<Acc>::bytes(LOGS), LOGS);
+    const HeavyAcc<Acc> acc = tab.acc();
     for (int64_t c = (int64_t)blockIdx.x * WARPS + wid; c < ncols; c += (int64_t)gridDim.x * WARPS) {
         const int j = list[c];
-        for (int s = lane; s < S; s += 32) {
-            keys[s] = kEmptyKey;
-            vals[s] = Acc(0);
-        }
-        __syncwarp();
         const int64_t p0 = ld_ptr(Bcolptr, p64, j), p1 = ld_ptr(Bcolptr, p64, j + 1);
+        tab.clear(lane);
         bool full = false;
-        warp_products<true, Acc>(
-            p0, p1, lane, segs[wid], At_row, At_val,
+        warp_walk<true, 4, Acc>(
+            p0, p1, lane, segs[wid], At_row,
             [&](int64_t p, long long &st, int &len, Acc &bv) {
                 int q = Bq[p];
                 if (q >= 0) {
@@ -263,40 +256,21 @@ __global__ void __launch_bounds__(WARPS * 32)
                     bv = Bv[p];
                 }
             },
-            [&](int r, Acc v) {
-                bool fresh;
-                int slot = hash_insert(keys, LOGS, r, &fresh);
-                if (slot < 0)
-                    full = true;
-                else
-                    atomic_add_acc(vals + slot, v);
+            [&](long long e) { return __ldg(At_val + e); },
+            [&](int r, Acc a, Acc b, bool ok) {
+                if (!tab.add(acc, r, a, b, ok)) full = true;
             });
         __syncwarp();
-        int nout = 0;
-        for (int c0 = 0; c0 < S; c0 += 32) {
-            int kk = keys[c0 + lane];
-            Acc vv = vals[c0 + lane];
-            bool occ = kk != kEmptyKey;
-            unsigned bal = __ballot_sync(kFull, occ);
-            __syncwarp();
-            if (occ) {
-                int pos = nout + __popc(bal & ((1u << lane) - 1u));
-                keys[pos] = kk;
-                vals[pos] = vv;
-            }
-            nout += __popc(bal);
-            __syncwarp();
-        }
+        const int nout = tab.compact(acc, lane);
         full = __any_sync(kFull, full);
-        if (full || nout > cap[j]) {
+        if (full || nout > cap[j]) {  // (cap is at most half the table)
             if (lane == 0) mark_overflow(flag, j, nflag);
         } else {
-            warp_sort_pairs<Acc>(keys, vals, nout, S, hist, lane);
             const int64_t base = capoff[j];
-            for (int s = lane; s < nout; s += 32) {
-                trow[base + s] = (OutIdx)keys[s];
-                tval[base + s] = vals[s];
-            }
+            tab.emit(acc, nout, lane, [&](int pos, int row, Acc v) {
+                trow[base + pos] = (OutIdx)row;
+                tval[base + pos] = v;
+            });
             if (lane == 0) nnz[j] = nout;
         }
         __syncwarp();
@@ -851,8 +825,7 @@ template <int LOGS, int WARPS, typename Acc, typename OutIdx>
 static spg_status launch_light_learned(spg_plan *p, const int32_t *list, int64_t cnt, const int64_t *capoff,
                                        const int64_t *cap, int64_t *nnz, int32_t *flag, unsigned long long *nflag,
                                        void *trow, void *tval) {
-    size_t smem = sizeof(WarpSeg<Acc>) * WARPS + (sizeof(Acc) + sizeof(int)) * (size_t)WARPS * (1 << LOGS) +
-                  sizeof(int) * 256 * (size_t)WARPS;
+    size_t smem = (sizeof(WarpSeg<Acc>) + WarpTable<Acc>::bytes(LOGS)) * WARPS;
     auto kern = k_light_learned<LOGS, WARPS, Acc, OutIdx>;
     cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     int occ = 1;
@@ -896,7 +869,7 @@ static spg_status learned_light(spg_plan *p, LearnedState &L) {
             case 2: s = launch_light_learned<7, 8, Acc, OutIdx>(p, list, cnt, L.capoff, L.cap, L.nnz_light, L.flag, L.nflag, L.trow, L.tval); break;
             case 3: s = launch_light_learned<8, 8, Acc, OutIdx>(p, list, cnt, L.capoff, L.cap, L.nnz_light, L.flag, L.nflag, L.trow, L.tval); break;
             case 4: s = launch_light_learned<9, 8, Acc, OutIdx>(p, list, cnt, L.capoff, L.cap, L.nnz_light, L.flag, L.nflag, L.trow, L.tval); break;
-            case 5: s = launch_light_learned<10, 4, Acc, OutIdx>(p, list, cnt, L.capoff, L.cap, L.nnz_light, L.flag, L.nflag, L.trow, L.tval); break;
+            case 5: s = launch_light_learned<10, 8, Acc, OutIdx>(p, list, cnt, L.capoff, L.cap, L.nnz_light, L.flag, L.nflag, L.trow, L.tval); break;
             default: s = launch_light_learned<11, 4, Acc, OutIdx>(p, list, cnt, L.capoff, L.cap, L.nnz_light, L.flag, L.nflag, L.trow, L.tval); break;
         }
     }

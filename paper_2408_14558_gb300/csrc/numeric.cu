@@ -2,8 +2,8 @@
 // C_i = A~_i * B_i, Gustavson column by column), written at the column
 // pointers produced by the symbolic pass.
 //   light bins: one warp per column, shared open-addressing table of
-//               (row, value) sized >= 2 x nnz_j; afterwards the occupied slots
-//               are compacted in place and sorted by row (warp radix sort)
+//               (row, value) sized >= 2 x nnz_j; afterwards the rows are
+//               compacted and put in order (warp_hash.cuh)
 //   heavy bin:  one CTA per (column, row slab): the symbolic bitmap of the
 //               slab gives every present row its rank, products accumulate at
 //               acc[rank] in shared memory, and the slab is written out in row
@@ -13,36 +13,34 @@
 #include "block_ops.cuh"
 #include "cta_products.cuh"
 #include "spg_internal.cuh"
+#include "warp_hash.cuh"
 
 namespace spg {
 
+// Small tables (up to 256 slots): 32 registers a thread and two windows in
+// flight keep 64 warps on an SM (refresh of A * P_agg on a 128^3 grid: 0.44 ms
+// at 62 registers and four windows, 0.35 so; tables of four times the entries
+// instead of two made no difference).
 template <int LOGS, int WARPS, typename Acc, typename OutIdx>
-__global__ void __launch_bounds__(WARPS * 32)
+__global__ void __launch_bounds__(WARPS * 32, LOGS <= 8 ? 8 : 1)
     k_num_light(const int32_t *__restrict__ list, int64_t ncols, const void *Bcolptr, int p64,
                 const int32_t *__restrict__ Bq, const Acc *__restrict__ Bv, const int64_t *__restrict__ At_colptr,
                 const int32_t *__restrict__ At_row, const Acc *__restrict__ At_val,
                 const int64_t *__restrict__ Ccolptr, OutIdx *__restrict__ Crow, Acc *__restrict__ Cval, int *err,
                 OutMask mask) {
-    constexpr int S = 1 << LOGS;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     WarpSeg<Acc> *segs = (WarpSeg<Acc> *)smem_raw;
-    Acc *vals_all = (Acc *)(segs + WARPS);
-    int *keys_all = (int *)(vals_all + WARPS * S);
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-    int *keys = keys_all + wid * S;
-    Acc *vals = vals_all + wid * S;
-    int *hist = keys_all + WARPS * S + wid * 256;
+    const WarpTable<Acc> tab((unsigned char *)(segs + WARPS) + wid * WarpTable<Acc>::bytes(LOGS), LOGS);
+    const HeavyAcc<Acc> acc = tab.acc();
     for (int64_t c = (int64_t)blockIdx.x * WARPS + wid; c < ncols; c += (int64_t)gridDim.x * WARPS) {
         const int j = list[c];
-        for (int s = lane; s < S; s += 32) {
-            keys[s] = kEmptyKey;
-            vals[s] = Acc(0);
-        }
-        __syncwarp();
         const int64_t p0 = ld_ptr(Bcolptr, p64, j), p1 = ld_ptr(Bcolptr, p64, j + 1);
+        const int64_t base = Ccolptr[j], want = Ccolptr[j + 1] - base;
+        tab.clear(lane);
         bool full = false;
-        warp_products<true, Acc>(
-            p0, p1, lane, segs[wid], At_row, At_val,
+        warp_walk<true, (LOGS <= 8 ? 2 : 4), Acc>(
+            p0, p1, lane, segs[wid], At_row,
             [&](int64_t p, long long &st, int &len, Acc &bv) {
                 int q = Bq[p];
                 if (q >= 0) {
@@ -51,42 +49,20 @@ __global__ void __launch_bounds__(WARPS * 32)
                     bv = Bv[p];
                 }
             },
-            [&](int r, Acc v) {
-                if (mask.bits && !mask_keeps(mask, j, r)) return;
-                bool fresh;
-                int slot = hash_insert(keys, LOGS, r, &fresh);
-                if (slot < 0)
-                    full = true;
-                else
-                    atomic_add_acc(vals + slot, v);
+            [&](long long e) { return __ldg(At_val + e); },
+            [&](int r, Acc a, Acc b, bool ok) {
+                if (mask.bits && ok && !mask_keeps(mask, j, r)) ok = false;
+                if (!tab.add(acc, r, a, b, ok)) full = true;
             });
         __syncwarp();
-        // compact the occupied slots to the front: a write never reaches a slot
-        // of a later, still unread chunk because the count so far is <= c0
-        int nout = 0;
-        for (int c0 = 0; c0 < S; c0 += 32) {
-            int kk = keys[c0 + lane];
-            Acc vv = vals[c0 + lane];
-            bool occ = kk != kEmptyKey;
-            unsigned bal = __ballot_sync(kFull, occ);
-            __syncwarp();
-            if (occ) {
-                int pos = nout + __popc(bal & ((1u << lane) - 1u));
-                keys[pos] = kk;
-                vals[pos] = vv;
-            }
-            nout += __popc(bal);
-            __syncwarp();
-        }
-        const int64_t base = Ccolptr[j];
-        if ((int64_t)nout != Ccolptr[j + 1] - base) {
+        const int nout = tab.compact(acc, lane);
+        if (nout != want) {
             full = true;
         } else {
-            warp_sort_pairs<Acc>(keys, vals, nout, S, hist, lane);
-            for (int s = lane; s < nout; s += 32) {
-                st_stream(Crow + base + s, (OutIdx)keys[s]);
-                st_stream(Cval + base + s, vals[s]);
-            }
+            tab.emit(acc, nout, lane, [&](int pos, int row, Acc v) {
+                st_stream(Crow + base + pos, (OutIdx)row);
+                st_stream(Cval + base + pos, v);
+            });
         }
         if (__any_sync(kFull, full) && lane == 0) atomicOr(err, kDevErrInternal);
         __syncwarp();
@@ -349,8 +325,7 @@ __global__ void k_rebin_numeric(const int8_t *bin_sym, const int64_t *nnzcol, in
 
 template <int LOGS, int WARPS, typename Acc, typename OutIdx>
 static spg_status launch_num_light(spg_plan *p, const int32_t *list, int64_t cnt, spg_csc *C) {
-    size_t smem = sizeof(WarpSeg<Acc>) * WARPS + (sizeof(Acc) + sizeof(int)) * (size_t)WARPS * (1 << LOGS) +
-                  sizeof(int) * 256 * (size_t)WARPS;
+    size_t smem = (sizeof(WarpSeg<Acc>) + WarpTable<Acc>::bytes(LOGS)) * WARPS;
     auto kern = k_num_light<LOGS, WARPS, Acc, OutIdx>;
     cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     int occ = 1;
@@ -377,7 +352,7 @@ static spg_status numeric_typed(spg_plan *p, spg_csc *C) {
             case 2: s = launch_num_light<7, 8, Acc, OutIdx>(p, list, cnt, C); break;
             case 3: s = launch_num_light<8, 8, Acc, OutIdx>(p, list, cnt, C); break;
             case 4: s = launch_num_light<9, 8, Acc, OutIdx>(p, list, cnt, C); break;
-            case 5: s = launch_num_light<10, 4, Acc, OutIdx>(p, list, cnt, C); break;
+            case 5: s = launch_num_light<10, 8, Acc, OutIdx>(p, list, cnt, C); break;
             default: s = launch_num_light<11, 4, Acc, OutIdx>(p, list, cnt, C); break;
         }
     }

@@ -29,6 +29,7 @@
 
 #include "block_ops.cuh"
 #include "spg_internal.cuh"
+#include "warp_hash.cuh"
 
 namespace spg {
 void clear_error();
@@ -161,16 +162,9 @@ __global__ void __launch_bounds__(WARPS * 32) k_small_multiply(SmallArgs a) {
     constexpr int kSlots = 1 << LOGS, kMaxU = kSlots / 2;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     WarpSeg<Acc> *segs = (WarpSeg<Acc> *)smem_raw;
-    int *keys_all = (int *)(segs + WARPS);
-    int *slots_all = keys_all + WARPS * kSlots;
-    Acc *vals_all = (Acc *)(slots_all + WARPS * kSlots);
-    int *hist_all = (int *)(vals_all + WARPS * kSlots);
     __shared__ long long red[WARPS], red2[WARPS];
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-    int *keys = keys_all + wid * kSlots;
-    int *slots = slots_all + wid * kSlots;
-    Acc *vals = vals_all + wid * kSlots;
-    int *hist = hist_all + wid * 256;
+    unsigned char *area = (unsigned char *)(segs + WARPS) + wid * WarpTable<Acc>::bytes(LOGS);
     const int64_t L = (a.n + gridDim.x - 1) / gridDim.x;
     const int64_t j0 = min((int64_t)blockIdx.x * L, a.n), j1 = min(j0 + L, a.n);
 
@@ -197,11 +191,12 @@ __global__ void __launch_bounds__(WARPS * 32) k_small_multiply(SmallArgs a) {
         if (U > kMaxU) {
             if (lane == 0) fail(a.res, SPG_UNSUPPORTED);  // the column's bound exceeds this table class
         } else if (U > 0) {
-            const int lg = table_log(U), S = 1 << lg;
-            for (int s = lane; s < S; s += 32) keys[s] = kEmptyKey;
+            const int lg = table_log(U);
+            int *keys = (int *)area;
+            warp_clear_keys(keys, lg, lane);
             __syncwarp();
             bool full = false;
-            warp_products_v<false, 4, Acc>(
+            warp_walk<false, 4, Acc>(
                 p0, p1, lane, segs[wid], a.Arow,
                 [&](int64_t p, long long &st, int &len, Acc &) {
                     const int64_t kk = ld_ptr(a.Brow, a.bi64, p);
@@ -210,13 +205,11 @@ __global__ void __launch_bounds__(WARPS * 32) k_small_multiply(SmallArgs a) {
                         len = (int)(ld_ptr(a.Acp, a.ap64, kk + 1) - st);
                     }
                 },
-                [&](long long) { return Acc(0); },
-                [&](int r, Acc) {
-                    bool fresh;
-                    if (hash_insert(keys, lg, r, &fresh) < 0) full = true;
-                    c += fresh ? 1 : 0;
+                [](long long) { return Acc(0); },
+                [&](int r, Acc, Acc, bool ok) {
+                    if (warp_hash_slot(keys, lg, r, ok) < 0 && ok) full = true;
                 });
-            c = warp_sum_i(c);
+            c = warp_count_keys(keys, lg, lane);
             if (__any_sync(kFull, full) && lane == 0) fail(a.res, SPG_CUDA_ERROR);
             __syncwarp();
         }
@@ -334,17 +327,12 @@ __global__ void __launch_bounds__(WARPS * 32) k_small_multiply(SmallArgs a) {
     for (int64_t j = j0 + wid; j < j1; j += WARPS) {
         const int64_t base = a.Ccp[j], want = a.Ccp[j + 1] - base;
         if (want == 0) continue;
-        const int lg = table_log(want), S = 1 << lg;
-        // values of the table's S slots (int64 as two 32-bit halves)
-        const HeavyAcc<Acc> acc(vals, S);
-        for (int s = lane; s < S; s += 32) {
-            keys[s] = kEmptyKey;
-            acc.zero(s);
-        }
-        __syncwarp();
+        const WarpTable<Acc> tab(area, table_log(want));
+        const HeavyAcc<Acc> acc = tab.acc();
+        tab.clear(lane);
         const int64_t p0 = ld_ptr(a.Bcp, a.bp64, j), p1 = ld_ptr(a.Bcp, a.bp64, j + 1);
         bool full = false;
-        warp_products_v<true, 4, Acc>(
+        warp_walk<true, 4, Acc>(
             p0, p1, lane, segs[wid], a.Arow,
             [&](int64_t p, long long &st, int &len, Acc &bv) {
                 const int64_t kk = ld_ptr(a.Brow, a.bi64, p);
@@ -355,41 +343,19 @@ __global__ void __launch_bounds__(WARPS * 32) k_small_multiply(SmallArgs a) {
                 }
             },
             [&](long long e) { return ld_val<Acc>(a.Aval, a.avt, e); },
-            [&](int r, Acc v) {
-                bool fresh;
-                const int slot = hash_insert(keys, lg, r, &fresh);
-                if (slot < 0)
-                    full = true;
-                else
-                    acc.add(slot, v);
+            [&](int r, Acc x, Acc y, bool ok) {
+                if (!tab.add(acc, r, x, y, ok)) full = true;
             });
         __syncwarp();
-        // compact the occupied slots to the front (row ids, and the slot
-        // holding each row's value), sort by row, then read the values out
-        int nout = 0;
-        for (int c0 = 0; c0 < S; c0 += 32) {
-            const int kk = keys[c0 + lane];
-            const bool occ = kk != kEmptyKey;
-            const unsigned bal = __ballot_sync(kFull, occ);
-            __syncwarp();
-            if (occ) {
-                const int pos = nout + __popc(bal & ((1u << lane) - 1u));
-                keys[pos] = kk;
-                slots[pos] = c0 + lane;
-            }
-            nout += __popc(bal);
-            __syncwarp();
-        }
-        if (nout != want || full) {
+        const int nout = tab.compact(acc, lane);
+        if (nout != want || __any_sync(kFull, full)) {
             if (lane == 0) fail(a.res, SPG_CUDA_ERROR);
             continue;
         }
-        warp_sort_pairs<int>(keys, slots, nout, S, hist, lane);
-        for (int s = lane; s < nout; s += 32) {
-            a.Crow[base + s] = keys[s];
-            Cval[base + s] = acc.get(slots[s]);
-        }
-        __syncwarp();
+        tab.emit(acc, nout, lane, [&](int pos, int row, Acc v) {
+            a.Crow[base + pos] = row;
+            Cval[base + pos] = v;
+        });
     }
 }
 
@@ -420,7 +386,7 @@ Layout layout_of(int64_t k, int64_t n, int P, int64_t b, int grid) {
 
 template <int LOGS, int WARPS, typename Acc>
 size_t smem_of() {
-    return WARPS * (sizeof(WarpSeg<Acc>) + (size_t(1) << LOGS) * (2 * sizeof(int) + sizeof(Acc)) + 256 * sizeof(int));
+    return WARPS * (sizeof(WarpSeg<Acc>) + WarpTable<Acc>::bytes(LOGS));
 }
 
 template <int LOGS, int WARPS, typename Acc>

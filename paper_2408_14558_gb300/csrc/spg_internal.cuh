@@ -283,88 +283,6 @@ __device__ __forceinline__ long long mul_acc<long long>(long long a, long long b
     return (long long)((unsigned long long)a * (unsigned long long)b);
 }
 
-__device__ __forceinline__ void atomic_add_acc(double *p, double v) { atomicAdd(p, v); }
-__device__ __forceinline__ void atomic_add_acc(long long *p, long long v) {
-    atomicAdd((unsigned long long *)p, (unsigned long long)v);
-}
-
-// Per-warp scratch for walking the products of one output column.
-template <typename Acc>
-struct WarpSeg {
-    int pref[33];
-    long long start[32];
-    Acc bv[32];
-};
-
-// Walk every product of the B' entries [p0, p1) of one output column with a
-// whole warp.  seg(p, start, len, bv) gives the A~ positions [start, start+len)
-// that B' entry p multiplies and its value; aval(e) loads A~'s value e.  The
-// lengths of 32 consecutive entries are prefix-summed so that all 32 lanes stay
-// busy however short the segments are; each step locates and loads U windows
-// of 32 products before any of them is used, so that U loads per lane are in
-// flight.  body(row, product) is called once per product.
-template <bool NEED_VAL, int U, typename Acc, typename SegFn, typename ValFn, typename Body>
-__device__ __forceinline__ void warp_products_v(int64_t p0, int64_t p1, int lane, WarpSeg<Acc> &ws,
-                                                const int32_t *__restrict__ At_row, SegFn seg, ValFn aval,
-                                                Body body) {
-    for (int64_t base = p0; base < p1; base += 32) {
-        int64_t p = base + lane;
-        long long st = 0;
-        int len = 0;
-        Acc bv = Acc(0);
-        if (p < p1) seg(p, st, len, bv);
-        int incl = len;
-#pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-            int t = __shfl_up_sync(kFull, incl, o);
-            if (lane >= o) incl += t;
-        }
-        int total = __shfl_sync(kFull, incl, 31);
-        ws.pref[lane] = incl - len;
-        ws.start[lane] = st;
-        if (NEED_VAL) ws.bv[lane] = bv;
-        __syncwarp();
-        for (int f0 = 0; f0 < total; f0 += 32 * U) {
-            int r[U];
-            Acc a[U], b[U];
-            bool ok[U];
-#pragma unroll
-            for (int u = 0; u < U; u++) {
-                const int fi = f0 + 32 * u + lane;
-                ok[u] = fi < total;
-                r[u] = 0;
-                a[u] = Acc(0);
-                b[u] = Acc(0);
-                if (ok[u]) {
-                    int s = 0;
-#pragma unroll
-                    for (int stp = 16; stp > 0; stp >>= 1)
-                        if (ws.pref[s + stp] <= fi) s += stp;
-                    const long long e = ws.start[s] + (fi - ws.pref[s]);
-                    r[u] = __ldg(At_row + e);
-                    if (NEED_VAL) {
-                        a[u] = aval(e);
-                        b[u] = ws.bv[s];
-                    }
-                }
-            }
-#pragma unroll
-            for (int u = 0; u < U; u++)
-                if (ok[u]) body(r[u], NEED_VAL ? mul_acc<Acc>(a[u], b[u]) : Acc(0));
-        }
-        __syncwarp();
-    }
-}
-
-// The same walk over A~ values stored in the accumulation type.
-template <bool NEED_VAL, typename Acc, typename SegFn, typename Body>
-__device__ __forceinline__ void warp_products(int64_t p0, int64_t p1, int lane, WarpSeg<Acc> &ws,
-                                              const int32_t *__restrict__ At_row,
-                                              const Acc *__restrict__ At_val, SegFn seg, Body body) {
-    warp_products_v<NEED_VAL, 4, Acc>(
-        p0, p1, lane, ws, At_row, seg, [&](long long e) { return __ldg(At_val + e); }, body);
-}
-
 // Heavy items: the rows of a symbolic item have their bitmap in shared memory
 // (at most kSymMaxWords words = 262,144 rows), those of a numeric item their
 // packed (bitmap word, prefix) pairs (at most kNumMaxWords words = 65,536
@@ -468,37 +386,6 @@ constexpr int kShortWindows = (kBatch * (kLongSeg - 1) + 31) / 32;
 
 __device__ __forceinline__ unsigned hash_row(int r, int shift) {
     return ((unsigned)r * 0x9E3779B1u) >> shift;
-}
-
-// Insert row r into an open-addressing table of 2^logS int keys (linear
-// probing).  Returns the slot, and sets *fresh when this call created it.
-// The table is sized >= 2x its final occupancy, so a free slot is always
-// reached; the probe count is still bounded (-1 = table full).
-__device__ __forceinline__ int hash_insert(int *keys, int logS, int r, bool *fresh) {
-    const int mask = (1 << logS) - 1;
-    unsigned h = hash_row(r, 32 - logS);
-    volatile int *vk = keys;
-    for (int probe = 0; probe <= mask; probe++) {
-        int cur = vk[h];
-        if (cur == r) {
-            *fresh = false;
-            return (int)h;
-        }
-        if (cur == kEmptyKey) {
-            int old = atomicCAS(keys + h, kEmptyKey, r);
-            if (old == kEmptyKey) {
-                *fresh = true;
-                return (int)h;
-            }
-            if (old == r) {
-                *fresh = false;
-                return (int)h;
-            }
-        }
-        h = (h + 1) & mask;
-    }
-    *fresh = false;
-    return -1;
 }
 
 __device__ __forceinline__ int warp_sum_i(int v) {

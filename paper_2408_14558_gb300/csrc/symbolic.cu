@@ -8,6 +8,7 @@
 //               product at its final rank without sorting
 #include "cta_products.cuh"
 #include "spg_internal.cuh"
+#include "warp_hash.cuh"
 
 namespace spg {
 
@@ -24,13 +25,12 @@ __global__ void __launch_bounds__(WARPS * 32)
     int *tab = keys_all + wid * S;
     for (int64_t c = (int64_t)blockIdx.x * WARPS + wid; c < ncols; c += (int64_t)gridDim.x * WARPS) {
         const int j = list[c];
-        for (int s = lane; s < S; s += 32) tab[s] = kEmptyKey;
-        __syncwarp();
         const int64_t p0 = ld_ptr(Bcolptr, p64, j), p1 = ld_ptr(Bcolptr, p64, j + 1);
-        int cnt = 0;
+        warp_clear_keys(tab, LOGS, lane);
+        __syncwarp();
         bool full = false;
-        warp_products<false, long long>(
-            p0, p1, lane, segs[wid], At_row, (const long long *)nullptr,
+        warp_walk<false, 4, long long>(
+            p0, p1, lane, segs[wid], At_row,
             [&](int64_t p, long long &st, int &len, long long &) {
                 int q = Bq[p];
                 if (q >= 0) {
@@ -38,13 +38,12 @@ __global__ void __launch_bounds__(WARPS * 32)
                     len = (int)(At_colptr[q + 1] - st);
                 }
             },
-            [&](int r, long long) {
-                if (mask.bits && !mask_keeps(mask, j, r)) return;
-                bool fresh;
-                if (hash_insert(tab, LOGS, r, &fresh) < 0) full = true;
-                cnt += fresh ? 1 : 0;
+            [&](long long) { return 0ll; },
+            [&](int r, long long, long long, bool ok) {
+                if (mask.bits && ok && !mask_keeps(mask, j, r)) ok = false;
+                if (warp_hash_slot(tab, LOGS, r, ok) < 0 && ok) full = true;
             });
-        cnt = warp_sum_i(cnt);
+        const int cnt = warp_count_keys(tab, LOGS, lane);
         if (__any_sync(kFull, full) && lane == 0) atomicOr(err, kDevErrInternal);
         if (lane == 0) nnzcol[j] = cnt;
         __syncwarp();
