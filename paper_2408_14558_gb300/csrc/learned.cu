@@ -302,8 +302,13 @@ __global__ void __launch_bounds__(kBatch)
     CtaBatch<Acc> &sb = *(CtaBatch<Acc> *)smem_raw;
     unsigned char *acc_raw = smem_raw + ((sizeof(CtaBatch<Acc>) + 15) & ~(size_t)15);
     const HeavyAcc<Acc> acc(acc_raw, kFusedRows);  // dense: slot = row within the item
-    uint32_t *bits = (uint32_t *)(acc_raw + HeavyAcc<Acc>::bytes_per_slot * kFusedRows);
+    // one byte per row of the item, set by a plain store per product (a bitmap's
+    // read-modify-write took 5 instructions more per product); the item's bitmap
+    // is put together from them afterwards
+    unsigned char *seen = acc_raw + HeavyAcc<Acc>::bytes_per_slot * kFusedRows;
+    uint32_t *bits = (uint32_t *)(seen + kFusedRows);
     int *pre = (int *)(bits + kFusedRows / 32);
+    for (int i = threadIdx.x; i < kFusedRows / 16; i += blockDim.x) ((uint4 *)seen)[i] = make_uint4(0u, 0u, 0u, 0u);
     __shared__ int wsum[33];
     __shared__ long long pos_sh, claim;
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = blockDim.x >> 5;
@@ -328,10 +333,8 @@ __global__ void __launch_bounds__(kBatch)
             }
         };
         const SegReg<Acc> first = cta_first_seg<Acc>(p0, p1, seg);
-        // (the first barrier of cta_products orders this before every product)
-        for (int w = threadIdx.x; w < nwords; w += blockDim.x) bits[w] = 0;
         const uint32_t abase = acc.addr(0) - ((uint32_t)rbase << HeavyAcc<Acc>::slot_shift);
-        uint32_t *bbase = bits - (rbase >> 5);
+        unsigned char *sbase = seen - rbase;
         bool stuck = false;
         cta_products<true, SPG_NUM_UNROLL, Acc>(
             p0, p1, sb, At_row, At_val, first, seg, [&](const auto &r, const auto &a, const auto &b, const auto &ok) {
@@ -340,11 +343,27 @@ __global__ void __launch_bounds__(kBatch)
 #pragma unroll
                 for (int u = 0; u < N; u++) {
                     ad[u] = abase + ((uint32_t)r[u] << HeavyAcc<Acc>::slot_shift);
-                    if (ok[u]) set_bit_shared(bbase + (r[u] >> 5), 1u << (r[u] & 31));
+                    if (ok[u]) sbase[r[u]] = 1;
                 }
                 if (!acc.add_products(ad, a, b, ok)) stuck = true;
             });
         if (stuck) atomicOr(err, kDevErrInternal);
+        // thread w puts word w together (and clears its bytes); the scan then
+        // takes it from the same thread
+        static_assert(kFusedRows / 32 <= kBatch, "one bitmap word per thread");
+        if (threadIdx.x < nwords) {
+            uint4 *s4 = (uint4 *)(seen + 32 * threadIdx.x);
+            uint32_t word = 0;
+#pragma unroll
+            for (int q = 0; q < 2; q++) {
+                const uint4 x = s4[q];
+                s4[q] = make_uint4(0u, 0u, 0u, 0u);
+                const uint32_t b[4] = {x.x, x.y, x.z, x.w};  // bytes 0 or 1, four to a bitmap nibble
+#pragma unroll
+                for (int c = 0; c < 4; c++) word |= ((b[c] * 0x01020408u >> 24) & 15u) << (16 * q + 4 * c);
+            }
+            bits[threadIdx.x] = word;
+        }
         const int cnt = cta_scan_popc1(bits, pre, nwords, wsum);
         if (threadIdx.x == 0) {
             long long pos = (long long)atomicAdd(colfill + j, (unsigned long long)cnt);
@@ -882,7 +901,7 @@ static spg_status learned_light(spg_plan *p, LearnedState &L) {
 template <typename Acc, typename OutIdx>
 static spg_status learned_fused(spg_plan *p, LearnedState &L, int64_t i0, int64_t i1) {
     if (i1 <= i0) return SPG_OK;
-    size_t smem = ((sizeof(CtaBatch<Acc>) + 15) & ~(size_t)15) + sizeof(Acc) * kFusedRows +
+    size_t smem = ((sizeof(CtaBatch<Acc>) + 15) & ~(size_t)15) + (sizeof(Acc) + 1) * kFusedRows +
                   sizeof(uint32_t) * (kFusedRows / 32) + sizeof(int) * (kFusedRows / 32 + 1);
     auto kern = k_fused_heavy<Acc, OutIdx>;
     spg_status s0 = cuda_check(cudaMemsetAsync(p->d_cnt + kCntFusedNextSlot, 0, sizeof(int64_t), p->st), "memset");
