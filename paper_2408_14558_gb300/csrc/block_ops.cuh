@@ -163,7 +163,7 @@ struct HeavyAcc<double> {
     // the whole CTA: clear slots [0, n) (and up to 3 more, inside the array)
     __device__ __forceinline__ void zero_all(int n) const {
         uint4 *p = (uint4 *)a;
-        for (int i = threadIdx.x; 2 * i < n; i += kBatch) p[i] = make_uint4(0u, 0u, 0u, 0u);
+        for (int i = threadIdx.x; 2 * i < n; i += blockDim.x) p[i] = make_uint4(0u, 0u, 0u, 0u);
     }
     __device__ __forceinline__ void add(int i, double v) const { atomicAdd(a + i, v); }
     __device__ __forceinline__ double get(int i) const { return a[i]; }
@@ -216,7 +216,7 @@ struct HeavyAcc<long long> {
     }
     __device__ __forceinline__ void zero_all(int n) const {
         uint4 *p = (uint4 *)lo, *q = (uint4 *)hi;  // (a multiple of 4 slots: both are 16-byte aligned)
-        for (int i = threadIdx.x; 4 * i < n; i += kBatch) p[i] = q[i] = make_uint4(0u, 0u, 0u, 0u);
+        for (int i = threadIdx.x; 4 * i < n; i += blockDim.x) p[i] = q[i] = make_uint4(0u, 0u, 0u, 0u);
     }
     __device__ __forceinline__ void add(int i, long long v) const {
         const unsigned long long u = (unsigned long long)v;
@@ -270,11 +270,11 @@ __device__ __forceinline__ int rank1(uint32_t e, uint32_t upto) { return (int)(e
 // once, with their final prefix.  ctot holds one int per chunk; src is 16-byte
 // aligned, nwords is a multiple of 4 and at most 128 * MAXC * nw.  Ends with a
 // barrier.
-template <int MAXC>
+template <int MAXC, int NT>
 __device__ __forceinline__ int cta_load_rank_table(const uint32_t *__restrict__ src, uint2 *tab, int nwords,
                                                    int *ctot) {
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-    constexpr int nw = kBatch / 32;
+    constexpr int nw = NT / 32;
     const int nch = (nwords + 127) >> 7;
     uint4 x[MAXC];
     int pre[MAXC];  // entries of the chunk before this lane's words

@@ -8,7 +8,7 @@
 
 namespace spg {
 
-// Staging area of cta_products for one batch of kBatch B' entries: the
+// Staging area of cta_products for one batch of NT B' entries (NT threads): the
 // non-empty A~ segments they multiply.  Window segments sit at [0, ns), long
 // ones at [ns, ns + nl); each part numbers its products consecutively, and
 // start holds a segment's first A~ entry minus its first product's number
@@ -18,11 +18,16 @@ namespace spg {
 // one more than the segment that reaches into the window from the one before,
 // or the segment that begins with the window: a product belongs to segment
 // .y - 1 plus the number of bits up to its own.
-template <typename Acc>
+template <typename Acc, int NT = kBatch>
 struct CtaBatch {
-    long long start[kBatch];
-    int pref[kBatch + 2];
-    Acc bv[kBatch];
+    static constexpr int kShortWindows = short_windows(NT), kMidSeg = mid_seg(NT);
+    static_assert(kLongSeg >= 32, "a 32-product window must meet at most two long segments");
+    static_assert(NT * (kLongSeg - 1) <= 32 * kShortWindows, "segments below kLongSeg always fit the windows");
+    static_assert(NT < 1024 && NT * (kMidSeg - 1) < 65536 && NT * (kLongSeg - 1) < 32768,
+                  "the packed scan counters hold a batch");
+    long long start[NT];
+    int pref[NT + 2];
+    Acc bv[NT];
     int wsum[3][33];
     uint2 win[kShortWindows];
     int cut[2];  // window segments and products of the middle class, if not all of it fits
@@ -30,16 +35,17 @@ struct CtaBatch {
     // all threads, once, before the first cta_products (which leaves the bits
     // clear again); a barrier must follow
     __device__ __forceinline__ void clear() {
-        for (int w = threadIdx.x; w < kShortWindows; w += kBatch) win[w].x = 0u;
+        for (int w = threadIdx.x; w < kShortWindows; w += NT) win[w].x = 0u;
     }
 };
 
 // Exclusive CTA scan of three counters at once; every thread gets the totals
 // in tot[0..2].  One barrier: every warp reads all warp sums and takes its own
 // offsets, so wsum must not be written again before the caller's next barrier.
+template <int NT>
 __device__ __forceinline__ void cta_scan3(const int v[3], int ex[3], int (*wsum)[33], int tot[3]) {
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-    constexpr int nw = kBatch / 32;
+    constexpr int nw = NT / 32;
     int in[3];
 #pragma unroll
     for (int q = 0; q < 3; q++) in[q] = v[q];
@@ -100,7 +106,7 @@ __device__ __forceinline__ EachProduct<F> each_product(F f) {
 }
 
 // Walk every product of the B' entries [p0, p1) of one output column with the
-// whole CTA (all threads must call it; blockDim.x == kBatch); `first` is
+// whole CTA (all threads must call it; blockDim.x == NT); `first` is
 // cta_first_seg(p0, p1, seg), and sb.clear() must have run once.
 // seg(p, start, len, bv) gives the A~ positions [start, start+len) that B'
 // entry p multiplies and its value; body(r, a, b, ok) takes this lane's next
@@ -119,19 +125,15 @@ __device__ __forceinline__ EachProduct<F> each_product(F f) {
 // The long steps are shared evenly by the warps, the windows are claimed.
 // One batch must hold < 2^31 products (heavy items bound their segments to the
 // item's row range).  Ends with a barrier.
-static_assert(kLongSeg >= 32, "a 32-product window must meet at most two long segments");
-static_assert(kBatch * (kLongSeg - 1) <= 32 * kShortWindows, "segments below kLongSeg always fit the windows");
-static_assert(kBatch < 1024 && kBatch * (kMidSeg - 1) < 65536 && kBatch * (kLongSeg - 1) < 32768,
-              "the packed scan counters hold a batch");
-
-template <bool NEED_VAL, int U, typename Acc, typename SegFn, typename Body>
-__device__ __forceinline__ void cta_products(int64_t p0, int64_t p1, CtaBatch<Acc> &sb,
+template <bool NEED_VAL, int U, typename Acc, int NT, typename SegFn, typename Body>
+__device__ __forceinline__ void cta_products(int64_t p0, int64_t p1, CtaBatch<Acc, NT> &sb,
                                              const int32_t *__restrict__ At_row, const Acc *__restrict__ At_val,
                                              SegReg<Acc> first, SegFn seg, Body body) {
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-    constexpr int nw = kBatch / 32;
+    constexpr int nw = NT / 32;
+    constexpr int kShortWindows = CtaBatch<Acc, NT>::kShortWindows, kMidSeg = CtaBatch<Acc, NT>::kMidSeg;
     SegReg<Acc> cur = first;
-    for (int64_t b0 = p0; b0 < p1; b0 += kBatch) {
+    for (int64_t b0 = p0; b0 < p1; b0 += NT) {
         const long long st = cur.st;
         const int len = cur.len;
         const Acc bv = cur.bv;
@@ -143,7 +145,7 @@ __device__ __forceinline__ void cta_products(int64_t p0, int64_t p1, CtaBatch<Ac
         const int v[3] = {len > 0 ? 1 << (10 * cls) : 0, cls == 0 ? len : 0,
                           cls == 1 ? len : cls == 2 ? len << 16 : 0};
         int ex[3], tot[3];
-        cta_scan3(v, ex, sb.wsum, tot);
+        cta_scan3<NT>(v, ex, sb.wsum, tot);
         const int n0 = tot[0] & 1023, n1 = (tot[0] >> 10) & 1023, n2 = tot[0] >> 20;
         const int m1 = tot[2] & 0xffff, m2 = (int)((uint32_t)tot[2] >> 16);
         const bool all_mid = m1 + m2 <= 32 * kShortWindows;
@@ -170,7 +172,7 @@ __device__ __forceinline__ void cta_products(int64_t p0, int64_t p1, CtaBatch<Ac
             if (NEED_VAL) sb.bv[i] = bv;
         }
         __syncthreads();
-        if (b0 + kBatch < p1) cur = cta_first_seg<Acc>(b0 + kBatch, p1, seg);
+        if (b0 + NT < p1) cur = cta_first_seg<Acc>(b0 + NT, p1, seg);
         // window segments [0, ns) with products [0, nsp), long segments
         // [ns, n) with products [lp0, lp1)
         const int kmid = all_mid ? n1 : sb.cut[0];
@@ -189,7 +191,7 @@ __device__ __forceinline__ void cta_products(int64_t p0, int64_t p1, CtaBatch<Ac
             const int f1 = min(lp1, f0 + (sper + (wid < srem ? 1 : 0)) * 32 * U);
             if (f0 < f1) {
                 int s = ns;
-                for (int stp = kBatch >> 1; stp > 0; stp >>= 1)
+                for (int stp = NT >> 1; stp > 0; stp >>= 1)
                     if (s + stp < n && sb.pref[s + stp] <= f0) s += stp;
                 long long baseA = sb.start[s];
                 Acc bvA = NEED_VAL ? sb.bv[s] : Acc(0);

@@ -132,8 +132,8 @@ __global__ void k_num_headers(int64_t nitems, const int32_t *__restrict__ num_re
 // an R-MAT graph of 262,144 vertices in doubles 65.6 -> 49.3 ms, of 100,003 in
 // int64 5.4 -> 4.4 ms, one 25,000-column chunk of the similarity product (dense
 // items) 39.6 -> 26.0 ms.
-template <typename Acc, typename OutIdx, bool MASKED>
-__global__ void __launch_bounds__(kBatch, SPG_NUM_MINB)
+template <typename Acc, typename OutIdx, bool MASKED, int NT>
+__global__ void __launch_bounds__(NT, SPG_NUM_MINB * kBatch / NT)
     k_num_heavy(int64_t nitems, const NumItem *__restrict__ items, const uint32_t *__restrict__ hbits,
                 const int32_t *__restrict__ Bq, const Acc *__restrict__ Bv, const int64_t *__restrict__ At_colptr,
                 const int32_t *__restrict__ At_row, const Acc *__restrict__ At_val,
@@ -142,8 +142,8 @@ __global__ void __launch_bounds__(kBatch, SPG_NUM_MINB)
     extern __shared__ __align__(16) unsigned char smem_raw[];
     const int RW = R >> 5;
     constexpr int kSlotShift = HeavyAcc<Acc>::slot_shift;
-    CtaBatch<Acc> &sb = *(CtaBatch<Acc> *)smem_raw;
-    unsigned char *acc_raw = smem_raw + ((sizeof(CtaBatch<Acc>) + 15) & ~(size_t)15);
+    CtaBatch<Acc, NT> &sb = *(CtaBatch<Acc, NT> *)smem_raw;
+    unsigned char *acc_raw = smem_raw + ((sizeof(CtaBatch<Acc, NT>) + 15) & ~(size_t)15);
     const HeavyAcc<Acc> acc(acc_raw, cap + kAccPad);
     uint2 *tab = (uint2 *)(acc_raw + HeavyAcc<Acc>::bytes_per_slot * (size_t)(cap + kAccPad));  // rank table
     __shared__ int ctot[kNumMaxWords / 128];
@@ -151,7 +151,7 @@ __global__ void __launch_bounds__(kBatch, SPG_NUM_MINB)
     __shared__ long long claim;
     __shared__ NumItem hdr;
     const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
-    constexpr int nw = kBatch / 32;
+    constexpr int nw = NT / 32;
     const uint32_t slot0 = acc.addr(0);
     sb.clear();
     if (tid == 0) {
@@ -182,7 +182,7 @@ __global__ void __launch_bounds__(kBatch, SPG_NUM_MINB)
         const SegReg<Acc> first = cta_first_seg<Acc>(h.p0, h.p1, seg);
         const uint32_t *src = hbits + (int64_t)h.r0 * RW;
         const bool direct = nr * R <= min(cap, kDirectRows);
-        const int cnt = cta_load_rank_table<kNumMaxWords / (4 * kBatch)>(src, tab, nwords, ctot);
+        const int cnt = cta_load_rank_table<kNumMaxWords / (4 * NT), NT>(src, tab, nwords, ctot);
         const int64_t rbase = (int64_t)t0 * R;
         NumItem nh;
         if (cnt == h.cnt && cnt <= cap) {
@@ -260,19 +260,19 @@ __global__ void __launch_bounds__(kBatch, SPG_NUM_MINB)
                         srow[rank_before(e) + __popc(word & ((1u << lane) - 1u))] = (uint16_t)(w * 32 + lane);
                 }
                 __syncthreads();
-                for (int i = v0; i < cnt; i += kBatch)
+                for (int i = v0; i < cnt; i += NT)
                     if (i >= 0) st_stream(cval + i, acc.get(srow[i]));
-                for (int i = r0; i < cnt; i += kBatch)
+                for (int i = r0; i < cnt; i += NT)
                     if (i >= 0) st_stream(crow + i, (OutIdx)(rbase + srow[i]));
             } else {
-                for (int i = v0; i < cnt; i += kBatch)
+                for (int i = v0; i < cnt; i += NT)
                     if (i >= 0) st_stream(cval + i, acc.get(i + 1));
                 __syncthreads();
                 // the row ids go to shared memory by rank first (over the
                 // consumed values: cnt ints fit in the first cnt slots), then
                 // to C in one coalesced run
                 int32_t *srow = acc.scratch32();
-                for (int w = tid; w < nwords; w += kBatch) {
+                for (int w = tid; w < nwords; w += NT) {
                     const uint2 e = tab[w];
                     uint32_t word = rank_word(e);
                     int pos = rank_before(e);
@@ -283,7 +283,7 @@ __global__ void __launch_bounds__(kBatch, SPG_NUM_MINB)
                     }
                 }
                 __syncthreads();
-                for (int i = r0; i < cnt; i += kBatch)
+                for (int i = r0; i < cnt; i += NT)
                     if (i >= 0) st_stream(crow + i, (OutIdx)(rbase + srow[i]));
             }
         } else {
@@ -359,10 +359,14 @@ static spg_status numeric_typed(spg_plan *p, spg_csc *C) {
     if (any_light) group_end(p, kKNumLight);
     if (s) return s;
     if (p->nnum > 0) {
-        const int threads = kBatch;
-        size_t smem = ((sizeof(CtaBatch<Acc>) + 15) & ~(size_t)15) + sizeof(Acc) * (size_t)(p->num_cap + kAccPad) +
+        const bool wide = p->num_wide;
+        const int threads = wide ? kWideBatch : kBatch;
+        const size_t staging = wide ? sizeof(CtaBatch<Acc, kWideBatch>) : sizeof(CtaBatch<Acc>);
+        size_t smem = ((staging + 15) & ~(size_t)15) + sizeof(Acc) * (size_t)(p->num_cap + kAccPad) +
                       sizeof(uint2) * (size_t)kNumMaxWords;
-        auto kern = p->omask.bits ? k_num_heavy<Acc, OutIdx, true> : k_num_heavy<Acc, OutIdx, false>;
+        auto kern = wide            ? k_num_heavy<Acc, OutIdx, true, kWideBatch>
+                    : p->omask.bits ? k_num_heavy<Acc, OutIdx, true, kBatch>
+                                    : k_num_heavy<Acc, OutIdx, false, kBatch>;
         cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         int occ = 1;
         cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kern, threads, smem);

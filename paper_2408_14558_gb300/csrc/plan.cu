@@ -1196,6 +1196,10 @@ static spg_status plan_build(spg_plan *p) {
         TRY(cuda_check(cudaMemcpyAsync(p->h_pinned + kPinnedRec + 1, sym_first + p->nheavy, sizeof(int64_t), cudaMemcpyDeviceToHost, st), "items"));
         TRY(read_counters());
         hub_histogram_read(p);
+        // few products per B entry and slab under a mask: wide items
+        p->num_wide = p->omask.bits && p->R <= kNumWideCap &&
+                      p->h_pinned[kCntProducts] / p->T < kWideProducts * p->h_pinned[kCntNnzBHeavy];
+        if (p->num_wide) p->num_cap = kNumWideCap;
         p->nrec = p->h_pinned[kPinnedRec];
         p->nsym = p->h_pinned[kPinnedRec + 1];
         if (p->nrec >= INT32_MAX) {

@@ -137,6 +137,7 @@ struct spg_plan {
     int64_t nnum = 0;
     int32_t *num_rec0 = nullptr, *num_nrec = nullptr;
     int num_cap = 4096, num_max_recs = 32;
+    bool num_wide = false;  // items of kNumWideCap entries
 
     // symbolic / numeric
     int64_t *nnzcol = nullptr;
@@ -310,6 +311,14 @@ constexpr int kNumMaxWords = SPG_NUM_MAX_WORDS;
 #define SPG_NUM_CAP_MIN 4096
 #endif
 constexpr int kNumCapMin = SPG_NUM_CAP_MIN;
+// Wide numeric items: 10,240 entries, CTAs of kWideBatch threads, two per SM.
+// Every item stages all of its column's B' entries, and where an entry brings
+// few products per slab of rows (A's columns are short and the output mask
+// leaves long columns: the betweenness products) that staging is the work.
+// Measured on the betweenness batch of 1024 sources on 65,536 vertices (about 2
+// products per entry and slab): 45.6 ms with 4096-entry items, 42.7 with these;
+// on the squaring of R-MAT graphs (about 20): 60.0 and 63.1 ms.
+constexpr int kNumWideCap = 10240, kWideProducts = 6;
 // C and the heavy bitmaps pass through L2 once; storing (and reading the
 // bitmaps) with the evict-first hint keeps A~, which the products re-read,
 // resident instead.
@@ -374,15 +383,14 @@ __device__ __forceinline__ void set_bit_shared(uint32_t *word, uint32_t mask) {
 #endif
 // threads of a heavy-bin CTA = B' entries staged per round by cta_products
 constexpr int kBatch = SPG_HEAVY_THREADS;
-// cta_products: segments from kMidSeg entries on are walked by steps of their
-// own, those below kLongSeg always through the windows of the staging area,
-// those between as far as the windows go.
+// threads of the wide numeric CTAs (kNumWideCap)
+constexpr int kWideBatch = 2 * kBatch;
+// cta_products: segments from mid_seg(threads) entries on are walked by steps
+// of their own, those below kLongSeg always through the windows of the staging
+// area, those between as far as the windows go.
 constexpr int kLongSeg = 32;
-#ifndef SPG_MID_SEG
-#define SPG_MID_SEG 256
-#endif
-constexpr int kMidSeg = SPG_MID_SEG;
-constexpr int kShortWindows = (kBatch * (kLongSeg - 1) + 31) / 32;
+constexpr int mid_seg(int threads) { return threads <= 256 ? 256 : 65536 / threads; }
+constexpr int short_windows(int threads) { return (threads * (kLongSeg - 1) + 31) / 32; }
 
 __device__ __forceinline__ unsigned hash_row(int r, int shift) {
     return ((unsigned)r * 0x9E3779B1u) >> shift;

@@ -108,3 +108,26 @@ def test_betweenness_on_long_and_short_frontiers(n, s):
     want = want[0] if isinstance(want, tuple) else want
     got = bc.cpu().numpy()
     assert np.all(np.abs(got - want) <= 1e-9 * np.maximum(1.0, np.abs(want)))
+
+
+@pytest.mark.parametrize("values", ["f64", "i64"])
+@pytest.mark.parametrize("m,R", [(90_000, 1024), (90_000, 4096), (90_000, 8192), (30_000, 16384)])
+def test_wide_masked_items(m, R, values):
+    """Few products per entry and slab under a mask: items of 10,240 entries and
+    512 threads; columns of several items, segments around 127 | 128 entries
+    and more than a batch (512) of entries."""
+    from test_gpu_mask import mask_from_pattern
+    rng = np.random.default_rng(15)
+    lens = [4] * 5000 + [31, 32, 127, 128, 129] * 4
+    A = columns(lens, m, rng, values)
+    B = columns([5020, 5000, 513, 512, 511], len(lens), rng, values)
+    M = columns([m // 2, m // 3, m // 2, 100, m], m, rng, "i64")
+    for complement in (False, True):
+        mask = mask_from_pattern(M)
+        plan = g.spgemm_plan(g.to_device(A), g.to_device(B), 2, 64, light_max=32, slab_rows=R, mask=mask,
+                             mask_complement=complement)
+        g.spgemm_symbolic(plan)
+        C = g.spgemm_numeric(plan)
+        torch.cuda.synchronize()
+        g.spgemm_plan_destroy(plan)
+        assert_full_parity(C, oracle.spgemm_masked(A, B, M, complement), f"wide m={m} R={R} {values} {complement}")
