@@ -139,7 +139,7 @@ void spg::collect_stats(spg_plan *p, spg_stats *st) {
     float plan_ms = 0;
     if (cudaEventElapsedTime(&plan_ms, p->ev[0], p->ev[1]) == cudaSuccess) p->stats.ms_plan = plan_ms;
     cudaGetLastError();
-    if (p->symbolic_done) {
+    if (p->ev_numeric) {
         float ms = 0;
         if (cudaEventQuery(p->ev[5]) == cudaSuccess && cudaEventElapsedTime(&ms, p->ev[4], p->ev[5]) == cudaSuccess)
             p->stats.ms_numeric = ms;

@@ -1206,6 +1206,7 @@ static spg_status learned_run(spg_plan *p, const spg_options *opt, spg_csc *C, i
         p->stats.nnzC_heavy = p->h_pinned[21];
         s = cuda_check(cudaMemcpyAsync(cp_opt, p->Ccolptr, cp_bytes, cudaMemcpyDeviceToDevice, st), "colptr");
         cudaEventRecord(p->ev[5], st);
+        p->ev_numeric = true;
         if (!s) s = read_dev_err(p, "learned");
         if (s) {
             free_opt();
@@ -1339,6 +1340,7 @@ static spg_status learned_run(spg_plan *p, const spg_options *opt, spg_csc *C, i
                              : learned_assemble<long long, int>(p, L, nf, flist, fcolptr, frow, fval, &out);
     }
     cudaEventRecord(p->ev[5], st);
+    p->ev_numeric = true;
     if (!s) s = read_dev_err(p, "learned");
     if (sub) spgemm_plan_destroy(sub);
     if (s) {

@@ -327,11 +327,8 @@ template <int LOGS, int WARPS, typename Acc, typename OutIdx>
 static spg_status launch_num_light(spg_plan *p, const int32_t *list, int64_t cnt, spg_csc *C) {
     size_t smem = (sizeof(WarpSeg<Acc>) + WarpTable<Acc>::bytes(LOGS)) * WARPS;
     auto kern = k_num_light<LOGS, WARPS, Acc, OutIdx>;
-    cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    int occ = 1;
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kern, WARPS * 32, smem);
-    if (occ < 1) occ = 1;
-    int g = grid_for(cnt, WARPS, p->sm_count * occ);
+    struct Tag {};
+    int g = grid_for(cnt, WARPS, p->sm_count * resident_ctas<Tag>(p, kern, WARPS * 32, smem));
     launch(p, kern, g, WARPS * 32, smem, list, cnt, p->B.colptr, p->B.ptr_type == SPG_IDX_I64, p->Bq,
                                          (const Acc *)p->Bv, p->At_colptr, p->At_row, (const Acc *)p->At_val,
                                          p->Ccolptr, (OutIdx *)C->rowidx, (Acc *)C->vals, p->d_err, p->omask);
@@ -434,6 +431,7 @@ spg_status run_numeric(spg_plan *p, spg_csc *C) {
     else
         s = p->out_idx64 ? numeric_typed<long long, long long>(p, C) : numeric_typed<long long, int>(p, C);
     cudaEventRecord(p->ev[5], st);
+    p->ev_numeric = true;
     return s;
 }
 

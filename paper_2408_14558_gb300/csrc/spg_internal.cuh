@@ -19,6 +19,7 @@
 #pragma once
 
 #include <cuda_runtime.h>
+#include <atomic>
 #include <cstdint>
 #include <cstdio>
 #include <string>
@@ -160,14 +161,35 @@ struct spg_plan {
 
     spg_stats stats{};
     // ev[0..1] plan, ev[2..3] symbolic, ev[4..5] numeric; kev[2g], kev[2g+1]
-    // bracket kernel group g (see KernelGroup)
+    // bracket kernel group g (see KernelGroup).  They and h_pinned come from a
+    // pool (plan.cu, take_kit) and may hold an earlier plan's records:
+    // kev_used and ev_numeric tell which this plan has made.
     cudaEvent_t ev[8] = {nullptr};
     cudaEvent_t kev[10] = {nullptr};
     bool kev_used[5] = {false, false, false, false, false};
+    bool ev_numeric = false;
+    size_t pinned_words = 0;
+    int dev = -1;
     int64_t launches = 0;
 };
 
 namespace spg {
+
+// Resident CTAs per SM of a kernel whose shared memory never changes, asked
+// once per device (the two calls take 3 us, a plan has up to twelve such
+// launches); `tag` makes one cache per kernel.
+template <typename Tag, typename Kern>
+inline int resident_ctas(spg_plan *p, Kern kern, int threads, size_t smem) {
+    static std::atomic<int> cached[16];
+    std::atomic<int> *slot = p->dev >= 0 && p->dev < 16 ? cached + p->dev : nullptr;
+    int occ = slot ? slot->load(std::memory_order_relaxed) : 0;
+    if (occ > 0) return occ;
+    cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kern, threads, smem);
+    if (occ < 1) return 1;
+    if (slot) slot->store(occ, std::memory_order_relaxed);
+    return occ;
+}
 
 // Every kernel of the library is launched through here, on the plan's
 // stream, so that the plan can report how many kernels it ran.

@@ -273,11 +273,8 @@ template <int LOGS, int WARPS>
 static spg_status launch_sym_light(spg_plan *p, const int32_t *list, int64_t cnt) {
     size_t smem = sizeof(WarpSeg<long long>) * WARPS + sizeof(int) * (size_t)WARPS * (1 << LOGS);
     auto kern = k_sym_light<LOGS, WARPS>;
-    cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    int occ = 1;
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kern, WARPS * 32, smem);
-    if (occ < 1) occ = 1;
-    int g = grid_for(cnt, WARPS, p->sm_count * occ);
+    struct Tag {};
+    int g = grid_for(cnt, WARPS, p->sm_count * resident_ctas<Tag>(p, kern, WARPS * 32, smem));
     launch(p, kern, g, WARPS * 32, smem, list, cnt, p->B.colptr, p->B.ptr_type == SPG_IDX_I64, p->Bq, p->At_colptr,
            p->At_row, p->nnzcol, p->d_err, p->omask);
     return cuda_check(cudaGetLastError(), "symbolic light");

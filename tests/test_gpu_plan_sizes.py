@@ -91,3 +91,41 @@ def test_long_columns_of_B(lens):
     rows = np.concatenate([np.sort(rng.choice(5000, k, replace=False)) for k in lens])
     B = synth._csc_from_sorted(5000, len(lens), cols, rows, rng.uniform(-1, 1, rows.size))
     assert_full_parity(run_gpu(A, B, 3, 64), oracle.spgemm(A, B), "long columns of B")
+
+
+def test_plans_of_several_threads_and_streams():
+    """Plans take their page-locked words and events from a pool: four threads,
+    each on its own stream, make, keep and destroy plans (more at a time than
+    the pool keeps, and one of more blocks than its words hold)."""
+    import threading
+    rng = np.random.default_rng(7)
+    A = banded(3000, 3000, 4, rng)
+    ref = oracle.spgemm(A, A)
+    bad = []
+
+    def work(i):
+        try:
+            s = torch.cuda.Stream()
+            with torch.cuda.stream(s):
+                dA = g.to_device(A, ptr_dtype=torch.int32, idx_dtype=torch.int32)
+                plans = [g.spgemm_plan(dA, dA, 1 + i, 64) for _ in range(8)]
+                for plan in plans:
+                    g.spgemm_symbolic(plan)
+                Cs = [g.spgemm_numeric(plan) for plan in plans] + [g.multiply(dA, dA, 1500, 64)]
+                s.synchronize()
+                assert all(g.spgemm_plan_stats(p)["ms_numeric"] > 0 for p in plans)
+                fresh = g.spgemm_plan(dA, dA, 1, 64)
+                assert g.spgemm_plan_stats(fresh)["ms_numeric"] == 0
+                for C in Cs:
+                    assert_full_parity(C, ref, f"thread {i}")
+                for plan in plans + [fresh]:
+                    g.spgemm_plan_destroy(plan)
+        except BaseException as e:   # noqa: BLE001
+            bad.append(e)
+
+    threads = [threading.Thread(target=work, args=(i,)) for i in range(4)]
+    for t in threads:
+        t.start()
+    for t in threads:
+        t.join()
+    assert not bad, bad
