@@ -303,26 +303,6 @@ __global__ void __launch_bounds__(NT, SPG_NUM_MINB * kBatch / NT)
     if (tid == 0 && bad_sh) atomicOr(err, kDevErrInternal);
 }
 
-__global__ void k_rebin_numeric(const int8_t *bin_sym, const int64_t *nnzcol, int64_t n, int8_t *bin_num) {
-    for (int64_t j = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; j < n; j += (int64_t)gridDim.x * blockDim.x) {
-        int b = bin_sym[j];
-        if (b != kBinHeavy && b != kBinEmpty) {
-            long long U = nnzcol[j];
-            if (U <= 0) {
-                b = kBinEmpty;
-            } else {
-                long long S = 64;
-                b = 1;
-                while (S < 2 * U) {
-                    S <<= 1;
-                    b++;
-                }
-            }
-        }
-        bin_num[j] = (int8_t)b;
-    }
-}
-
 template <int LOGS, int WARPS, typename Acc, typename OutIdx>
 static spg_status launch_num_light(spg_plan *p, const int32_t *list, int64_t cnt, spg_csc *C) {
     size_t smem = (sizeof(WarpSeg<Acc>) + WarpTable<Acc>::bytes(LOGS)) * WARPS;
@@ -402,10 +382,7 @@ spg_status queue_numeric_bins(spg_plan *p) {
     int8_t *bn = (int8_t *)ws_alloc(p, (size_t)(n + 1));
     p->nbinlist = (int32_t *)ws_alloc(p, sizeof(int32_t) * (size_t)(n + 1));
     if (!bn || !p->nbinlist) return SPG_OUT_OF_MEMORY;
-    launch(p, k_rebin_numeric, grid_for(n, 256, p->sm_count * 8), 256, 0, p->bin_of, p->nnzcol, n, bn);
-    spg_status s = cuda_check(cudaGetLastError(), "rebin");
-    if (s) return s;
-    s = bin_columns_queue(p, bn, p->nbinlist);
+    const spg_status s = bin_columns_queue(p, bn, p->nbinlist, 2);
     p->nbins_queued = s == SPG_OK;
     return s;
 }

@@ -2,15 +2,14 @@
 // for all P column blocks at once, on one GPU.
 //   k_nonempty_bits  D, the nonempty columns of A (Algorithm 1, allgather of
 //                    nonzero column ids: here A.colptr is local)
-//   k_block_eoff     the first entry of B of every column block
 //   k_mark_H         H_i, nonzero rows of B_i (Table 1, Algorithm 1), one
 //                    thread per entry of B
-//   k_popc_HD        popc(H_i & D) per word, then a scan gives each required
-//                    column its place in D~ (Algorithm 1, D~ = H_i AND D)
-//   k_dtilde         the ascending list D~_i
-//   k_fetch          Algorithm 2 with groups of b consecutive column ids
+//   scan_exclusive_bits  a scan of popc(H_i & D) gives each required column its
+//                    place in D~ (Algorithm 1, D~ = H_i AND D)
+//   k_dtilde         the ascending list D~_i, and Algorithm 2 with groups of b
+//                    consecutive column ids
 //   k_block_dt       each block's range of D~
-//   k_gather_len / k_gather_shift / k_gather_copy   A~_i = A(:, D~_i) for all
+//   k_gather_len / k_gather_copy   A~_i = A(:, D~_i) for all
 //                    blocks in one entry-balanced copy (on one GPU the chosen
 //                    fetch blocks only give the volume Algorithm 2 transfers)
 //   k_remap_B        B_i's rows k -> column of A~_i (Algorithm 1's local index)
@@ -230,9 +229,13 @@ __global__ void k_validate_rows(ValidateArgs args, int *err) {
     if (bad) atomicOr(err, kDevErrInput);
 }
 
-__global__ void k_nonempty_bits(const void *colptr, int p64, int64_t k, int64_t W, uint32_t *D) {
-    for (int64_t w = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; w < W;
-         w += (int64_t)gridDim.x * blockDim.x) {
+// D, and the first entry of every column block of B: eoff[i] = colptr[bound_i],
+// i <= P.
+__global__ void k_nonempty_bits(const void *colptr, int p64, int64_t k, int64_t W, uint32_t *D, const void *Bcolptr,
+                                int p64B, int64_t n, int P, const int64_t *bounds, int64_t *eoff) {
+    const int64_t t0 = (int64_t)blockIdx.x * blockDim.x + threadIdx.x, nt = (int64_t)gridDim.x * blockDim.x;
+    for (int64_t i = t0; i <= P; i += nt) eoff[i] = ld_ptr(Bcolptr, p64B, bounds ? bounds[i] : i * n / P);
+    for (int64_t w = t0; w < W; w += nt) {
         uint32_t bits = 0;
         int64_t h0 = w * 32;
         int64_t prev = ld_ptr(colptr, p64, h0);
@@ -283,33 +286,6 @@ __global__ void k_split_bounds(const int64_t *pre, int64_t n, int P, int64_t *bo
     bounds[i] = lo;
 }
 
-// Per-block flops of the plan's split (warp-aggregated when a warp's columns
-// share a block).
-__global__ void k_block_flops(const int64_t *flops, int64_t n, int P, const int64_t *bounds, long long *blk_flops) {
-    const int lane = threadIdx.x & 31;
-    for (int64_t base = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) & ~(int64_t)31; base < n;
-         base += (int64_t)gridDim.x * blockDim.x) {
-        const int64_t j = base + lane;
-        const bool valid = j < n;
-        const int i = valid ? block_of_b(j, n, P, bounds) : -1;
-        const long long f = valid ? flops[j] : 0;
-        const int i0 = __shfl_sync(kFull, i, 0);
-        if (__all_sync(kFull, !valid || i == i0)) {
-            const long long t = warp_sum_ll(f);
-            if (lane == 0 && t) atomicAdd((unsigned long long *)(blk_flops + i0), (unsigned long long)t);
-        } else if (valid && f) {
-            atomicAdd((unsigned long long *)(blk_flops + i), (unsigned long long)f);
-        }
-    }
-}
-
-// Warp per column j of B: set bit r of H_{block(j)} for every stored row r.
-// First entry of every column block of B: eoff[i] = colptr[bound_i], i <= P.
-__global__ void k_block_eoff(const void *colptr, int p64, int64_t n, int P, const int64_t *bounds, int64_t *eoff) {
-    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i <= P; i += gridDim.x * blockDim.x)
-        eoff[i] = ld_ptr(colptr, p64, bounds ? bounds[i] : (int64_t)i * n / P);
-}
-
 // The column block of B's entry q: the largest i < P with eoff[i] <= q
 // (empty blocks share their offset with the next one).
 __device__ __forceinline__ int block_of_entry(int64_t q, const int64_t *__restrict__ eoff, int P) {
@@ -337,20 +313,6 @@ __global__ void k_mark_H(const void *rowidx, int i64, int64_t nnz, int P, int64_
     }
 }
 
-// cnt[i*W + w] = popc(H_i[w] & D[w]); also sum_i |H_i| for the statistics.
-__global__ void k_popc_HD(const uint32_t *H, const uint32_t *D, int64_t W, int64_t total,
-                          int32_t *cnt, long long *sumH) {
-    long long h = 0;
-    for (int64_t x = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; x < total;
-         x += (int64_t)gridDim.x * blockDim.x) {
-        uint32_t hw = H[x];
-        cnt[x] = __popc(hw & D[x % W]);
-        h += __popc(hw);
-    }
-    h = warp_sum_ll(h);
-    if ((threadIdx.x & 31) == 0 && h) atomicAdd((unsigned long long *)sumH, (unsigned long long)h);
-}
-
 // Global index in D~ of the first required column >= x in block i.
 __device__ __forceinline__ int64_t rank_at(const uint32_t *H, const uint32_t *D, const int64_t *rankpre,
                                            int64_t W, int i, int64_t x) {
@@ -360,12 +322,18 @@ __device__ __forceinline__ int64_t rank_at(const uint32_t *H, const uint32_t *D,
     return r;
 }
 
-__global__ void k_dtilde(const uint32_t *H, const uint32_t *D, const int64_t *rankpre, int64_t W,
-                         int64_t total, int32_t *dtilde) {
-    for (int64_t x = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; x < total;
-         x += (int64_t)gridDim.x * blockDim.x) {
+// D~'s lists, and Algorithm 2: fetch block t of block i is chosen iff it
+// contains a required column; also sum_i |H_i| for the statistics.
+__global__ void k_dtilde(const uint32_t *H, const uint32_t *D, const int64_t *rankpre, int64_t W, int64_t total,
+                         int32_t *dtilde, int64_t k, int64_t b, int64_t nfb, int P, const void *Acolptr, int p64,
+                         uint8_t *fetch, long long *chosen, long long *volblock, long long *sumH) {
+    const int64_t t0 = (int64_t)blockIdx.x * blockDim.x + threadIdx.x, nt = (int64_t)gridDim.x * blockDim.x;
+    long long c = 0, v = 0, h = 0;
+    for (int64_t x = t0; x < total; x += nt) {
         int64_t w = x % W;
-        uint32_t bits = H[x] & D[w];
+        const uint32_t hw = H[x];
+        h += __popc(hw);
+        uint32_t bits = hw & D[w];
         int64_t base = rankpre[x];
         while (bits) {
             int bb = __ffs(bits) - 1;
@@ -373,16 +341,7 @@ __global__ void k_dtilde(const uint32_t *H, const uint32_t *D, const int64_t *ra
             bits &= bits - 1;
         }
     }
-}
-
-// Algorithm 2: fetch block t of block i is chosen iff it contains a required column.
-__global__ void k_fetch(const uint32_t *H, const uint32_t *D, const int64_t *rankpre, int64_t W,
-                        int64_t k, int64_t b, int64_t nfb, int P, const void *Acolptr, int p64,
-                        uint8_t *fetch, long long *chosen, long long *volblock) {
-    long long c = 0, v = 0;
-    int64_t total = nfb * P;
-    for (int64_t x = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; x < total;
-         x += (int64_t)gridDim.x * blockDim.x) {
+    for (int64_t x = t0; x < nfb * P; x += nt) {
         int i = (int)(x / nfb);
         int64_t t = x % nfb;
         int64_t lo = t * b, hi = min(k, lo + b);
@@ -395,9 +354,11 @@ __global__ void k_fetch(const uint32_t *H, const uint32_t *D, const int64_t *ran
     }
     c = warp_sum_ll(c);
     v = warp_sum_ll(v);
+    h = warp_sum_ll(h);
     if ((threadIdx.x & 31) == 0) {
         if (c) atomicAdd((unsigned long long *)chosen, (unsigned long long)c);
         if (v) atomicAdd((unsigned long long *)volblock, (unsigned long long)v);
+        if (h) atomicAdd((unsigned long long *)sumH, (unsigned long long)h);
     }
 }
 
@@ -500,13 +461,6 @@ __device__ __forceinline__ long long load_val<long long>(const void *v, int vt, 
     return vt == SPG_VAL_I32 ? (long long)__ldg((const int *)v + i) : (long long)__ldg((const long long *)v + i);
 }
 
-// Per A~ column g: the entry e of A~ sits at position e + shift[g] of A.
-__global__ void k_gather_shift(const int32_t *dtilde, int64_t ndt, const void *Acolptr, int p64,
-                               const int64_t *At_colptr, int64_t *shift) {
-    for (int64_t g = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; g < ndt; g += (int64_t)gridDim.x * blockDim.x)
-        shift[g] = ld_ptr(Acolptr, p64, dtilde[g]) - At_colptr[g];
-}
-
 // A~ = A(:, D~) for all blocks at once (rows narrowed to int32, values widened
 // to the accumulation type), balanced by entries: warp w copies the entries
 // [w * chunk, (w + 1) * chunk) of A~.  It finds the column of its first entry
@@ -515,8 +469,8 @@ __global__ void k_gather_shift(const int32_t *dtilde, int64_t ndt, const void *A
 // step mark distinct positions and one warp OR-reduction gives each lane its
 // column.
 template <typename Acc>
-__global__ void k_gather_copy(const int64_t *__restrict__ At_colptr, const int64_t *__restrict__ shift, int64_t ndt,
-                              int64_t nAt, int64_t chunk, const void *Arow, int i64, const void *Aval, int vt,
+__global__ void k_gather_copy(const int64_t *__restrict__ At_colptr, const int32_t *__restrict__ dtilde,
+                              const void *Acolptr, int p64, int64_t ndt, int64_t nAt, int64_t chunk, const void *Arow, int i64, const void *Aval, int vt,
                               int32_t *__restrict__ At_row, Acc *__restrict__ At_val) {
     const int lane = threadIdx.x & 31;
     const int64_t w = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
@@ -538,10 +492,11 @@ __global__ void k_gather_copy(const int64_t *__restrict__ At_colptr, const int64
     }
     int64_t s0 = lo;  // the column holding entry f
     for (int64_t f = e0; f < e1; f += 32) {
-        // lane k holds column s0 + k: its start and its shift
+        // lane k holds column s0 + k: its start, and how far A's column begins
+        // from there
         const int64_t sk = s0 + lane;
         const int64_t bk = sk < ndt ? At_colptr[sk] : INT64_MAX;
-        const int64_t shk = sk < ndt ? shift[sk] : 0;
+        const int64_t shk = sk < ndt ? ld_ptr(Acolptr, p64, dtilde[sk]) - bk : 0;
         const int64_t pos = bk - f;  // >= 1 for k >= 1
         const uint32_t M = __reduce_or_sync(kFull, (lane > 0 && pos < 32) ? (1u << (int)pos) : 0u);
         const int k = __popc(M & ((2u << lane) - 1u));
@@ -746,13 +701,45 @@ __global__ void __launch_bounds__(256)
 // those of block i + 1 and share A~_i in L2.
 constexpr int kBinChunk = 2048, kBinMaxChunks = 2048;
 
-__global__ void k_bin_chunk_count(const int8_t *bin_of, int64_t n, int64_t chunk, int64_t nchunks, int32_t *cnt) {
+// MODE 0: counts only.  1 (the plan's bins): also the flops of every column
+// block, warp-aggregated when a warp's columns share one.  2 (the numeric
+// bins): bin_of is written first, from the symbolic bin and the exact count.
+template <int MODE>
+__global__ void k_bin_chunk_count(int8_t *bin_of, int64_t n, int64_t chunk, int64_t nchunks, int32_t *cnt,
+                                  const int64_t *flops, int P, const int64_t *bounds, long long *blk_flops,
+                                  const int8_t *bin_sym, const int64_t *nnzcol) {
     __shared__ int h[kNumBins];
+    const int lane = threadIdx.x & 31;
     for (int64_t c = blockIdx.x; c < nchunks; c += gridDim.x) {
         if (threadIdx.x < kNumBins) h[threadIdx.x] = 0;
         __syncthreads();
         const int64_t j1 = min(n, (c + 1) * chunk);
-        for (int64_t j = c * chunk + threadIdx.x; j < j1; j += blockDim.x) atomicAdd(&h[bin_of[j]], 1);
+        for (int64_t base = c * chunk + (threadIdx.x & ~31); base < j1; base += blockDim.x) {
+            const int64_t j = base + lane;
+            const bool valid = j < j1;
+            int b = 0;
+            if (valid) {
+                if (MODE == 2) {
+                    b = bin_sym[j];
+                    if (b != kBinHeavy && b != kBinEmpty) b = light_bin(nnzcol[j], 1 << 30);
+                    bin_of[j] = (int8_t)b;
+                } else {
+                    b = bin_of[j];
+                }
+                atomicAdd(&h[b], 1);
+            }
+            if (MODE == 1) {
+                const int i = valid ? block_of_b(j, n, P, bounds) : -1;
+                const long long f = valid ? flops[j] : 0;
+                const int i0 = __shfl_sync(kFull, i, 0);
+                if (__all_sync(kFull, !valid || i == i0)) {
+                    const long long t = warp_sum_ll(f);
+                    if (lane == 0 && t) atomicAdd((unsigned long long *)(blk_flops + i0), (unsigned long long)t);
+                } else if (valid && f) {
+                    atomicAdd((unsigned long long *)(blk_flops + i), (unsigned long long)f);
+                }
+            }
+        }
         __syncthreads();
         if (threadIdx.x < kNumBins) cnt[(int64_t)threadIdx.x * nchunks + c] = h[threadIdx.x];
         __syncthreads();
@@ -817,7 +804,7 @@ __global__ void __launch_bounds__(32 * kNumBins)
 
 // Launches only; the bins' offsets arrive in h_pinned[kPinnedBins ..] once the
 // stream is synchronised (bin_offsets).
-spg_status bin_columns_queue(spg_plan *p, const int8_t *bin_of, int32_t *list) {
+spg_status bin_columns_queue(spg_plan *p, int8_t *bin_of, int32_t *list, int mode) {
     const int64_t n = p->n;
     const int64_t chunk = std::max<int64_t>(kBinChunk, ((n + kBinMaxChunks - 1) / kBinMaxChunks + 255) / 256 * 256);
     const int64_t nchunks = (n + chunk - 1) / chunk;
@@ -825,8 +812,11 @@ spg_status bin_columns_queue(spg_plan *p, const int8_t *bin_of, int32_t *list) {
     int64_t *off = (int64_t *)ws_alloc(p, sizeof(int64_t) * (size_t)(kNumBins + 1));
     if (!cnt || !off) return SPG_OUT_OF_MEMORY;
     const int g = grid_for(nchunks, 1, p->sm_count * 8);
-    launch(p, k_bin_chunk_count, g, 256, 0, bin_of, n, chunk, nchunks, cnt);
-    launch(p, k_bin_chunk_scatter, g, 32 * kNumBins, 0, bin_of, n, chunk, nchunks, (const int32_t *)cnt, off, list);
+    launch(p, mode == 1 ? k_bin_chunk_count<1> : mode == 2 ? k_bin_chunk_count<2> : k_bin_chunk_count<0>, g, 256, 0,
+           bin_of, n, chunk, nchunks, cnt, p->flops, p->P, p->bounds_d, (long long *)p->blk,
+           (const int8_t *)p->bin_of, p->nnzcol);
+    launch(p, k_bin_chunk_scatter, g, 32 * kNumBins, 0, (const int8_t *)bin_of, n, chunk, nchunks,
+           (const int32_t *)cnt, off, list);
     spg_status s = cuda_check(cudaGetLastError(), "bins");
     if (s) return s;
     return cuda_check(cudaMemcpyAsync(p->h_pinned + kPinnedBins, off, sizeof(int64_t) * (kNumBins + 1),
@@ -835,8 +825,8 @@ spg_status bin_columns_queue(spg_plan *p, const int8_t *bin_of, int32_t *list) {
 void bin_offsets(const spg_plan *p, int64_t *off_host) {
     for (int b = 0; b <= kNumBins; b++) off_host[b] = p->h_pinned[kPinnedBins + b];
 }
-spg_status bin_columns(spg_plan *p, const int8_t *bin_of, int32_t *list, int64_t *off_host) {
-    spg_status s = bin_columns_queue(p, bin_of, list);
+spg_status bin_columns(spg_plan *p, int8_t *bin_of, int32_t *list, int64_t *off_host) {
+    spg_status s = bin_columns_queue(p, bin_of, list, 0);
     if (!s) s = cuda_check(cudaStreamSynchronize(p->st), "bin readback");
     if (!s) bin_offsets(p, off_host);
     return s;
@@ -1009,8 +999,6 @@ spg_status copy_operands(spg_plan *p) {
     const int p64A = A.ptr_type == SPG_IDX_I64, i64A = A.idx_type == SPG_IDX_I64;
     const int i64B = B.idx_type == SPG_IDX_I64;
     if (p->ndt > 0 && p->nAt > 0) {
-        if (!p->gshift) p->gshift = (int64_t *)ws_alloc(p, sizeof(int64_t) * (size_t)p->ndt);
-        if (!p->gshift) return SPG_OUT_OF_MEMORY;
         // at least 128 entries per warp, about 2048 once that fills the GPU
         // (226,000 entries: 35 us in 2048s, 110 warps), at most 32 CTAs of 8
         // warps per SM
@@ -1019,13 +1007,13 @@ spg_status copy_operands(spg_plan *p) {
         const int64_t chunk = ((p->nAt + warps - 1) / warps + 31) & ~(int64_t)31;
         const int64_t g = (((p->nAt + chunk - 1) / chunk) + 7) / 8;
         group_begin(p, kKGather);
-        launch(p, k_gather_shift, grid_for(p->ndt, 256, sm * 8), 256, 0, p->dtilde, p->ndt, A.colptr, p64A,
-               p->At_colptr, p->gshift);
         if (p->acc_f64)
-            launch(p, k_gather_copy<double>, (unsigned)g, 256, 0, p->At_colptr, p->gshift, p->ndt, p->nAt, chunk,
+            launch(p, k_gather_copy<double>, (unsigned)g, 256, 0, p->At_colptr, (const int32_t *)p->dtilde,
+                   A.colptr, p64A, p->ndt, p->nAt, chunk,
                    A.rowidx, i64A, A.vals, A.val_type, p->At_row, (double *)p->At_val);
         else
-            launch(p, k_gather_copy<long long>, (unsigned)g, 256, 0, p->At_colptr, p->gshift, p->ndt, p->nAt, chunk,
+            launch(p, k_gather_copy<long long>, (unsigned)g, 256, 0, p->At_colptr, (const int32_t *)p->dtilde,
+                   A.colptr, p64A, p->ndt, p->nAt, chunk,
                    A.rowidx, i64A, A.vals, A.val_type, p->At_row, (long long *)p->At_val);
         group_end(p, kKGather);
         spg_status s = cuda_check(cudaGetLastError(), "gather");
@@ -1088,14 +1076,21 @@ static spg_status plan_build(spg_plan *p) {
     const size_t accsz = 8;
 
     // everything that starts at zero, cleared by one memset: error word,
-    // counters, per-block sums
-    const size_t zero_words = 2 + kCntSlots + 3 * (size_t)P;
-    int64_t *zeroed = (int64_t *)ws_alloc(p, sizeof(int64_t) * zero_words);
+    // counters, per-block sums, the H_i, and the validation's column starts
+    const bool same = A.colptr == B.colptr && A.rowidx == B.rowidx && A.nnz == B.nnz && A.ncols == B.ncols &&
+                      A.nrows == B.nrows && A.ptr_type == B.ptr_type && A.idx_type == B.idx_type;
+    p->W = (k + 31) / 32;
+    const int64_t W = p->W;
+    const size_t words = 2 + kCntSlots + 3 * (size_t)P, hw = (size_t)(P * W + 2) / 2;
+    const size_t wa = p->opt.validate ? (size_t)(A.nnz / 64 + 1) : 0;
+    const size_t wb = p->opt.validate && !same ? (size_t)(B.nnz / 64 + 1) : 0;
+    int64_t *zeroed = (int64_t *)ws_alloc(p, sizeof(int64_t) * (words + hw + wa + wb));
     if (!zeroed) return SPG_OUT_OF_MEMORY;
     p->d_err = (int *)zeroed;
     p->d_cnt = zeroed + 2;
     p->blk = p->d_cnt + kCntSlots;
-    TRY(cuda_check(cudaMemsetAsync(zeroed, 0, sizeof(int64_t) * zero_words, st), "memset"));
+    p->Hbits = (uint32_t *)(zeroed + words);
+    TRY(cuda_check(cudaMemsetAsync(zeroed, 0, sizeof(int64_t) * (words + hw + wa + wb), st), "memset"));
     cudaEventRecord(p->ev[0], st);
 
     // Validation.  Its result is read back together with |D~| (the kernels up
@@ -1103,19 +1098,14 @@ static spg_status plan_build(spg_plan *p) {
     // split, which walks B's columns.
     const bool split_flops = p->opt.split == SPG_SPLIT_FLOPS && P > 1 && n > 0;
     if (p->opt.validate) {
-        const bool same = A.colptr == B.colptr && A.rowidx == B.rowidx && A.nnz == B.nnz && A.ncols == B.ncols &&
-                          A.nrows == B.nrows && A.ptr_type == B.ptr_type && A.idx_type == B.idx_type;
         const int nm = same ? 1 : 2;
-        const size_t wa = (size_t)(A.nnz / 32 + 1), wb = same ? 0 : (size_t)(B.nnz / 32 + 1);
-        uint32_t *starts = (uint32_t *)ws_alloc(p, sizeof(uint32_t) * (wa + wb));
-        if (!starts) return SPG_OUT_OF_MEMORY;
-        TRY(cuda_check(cudaMemsetAsync(starts, 0, sizeof(uint32_t) * (wa + wb), st), "memset"));
+        uint32_t *starts = (uint32_t *)(zeroed + words + hw);
         ValidateArgs va;
         const spg_csc *M[2] = {&A, &B};
         for (int i = 0; i < 2; i++)
             va.m[i] = ValidateArg{M[i]->colptr, M[i]->rowidx, M[i]->ptr_type == SPG_IDX_I64,
                                   M[i]->idx_type == SPG_IDX_I64, M[i]->ncols, M[i]->nnz, M[i]->nrows,
-                                  starts + (i == 0 ? 0 : wa)};
+                                  starts + (i == 0 ? 0 : 2 * wa)};
         const int64_t mc = same ? A.ncols : std::max(A.ncols, B.ncols), mz = same ? A.nnz : std::max(A.nnz, B.nnz);
         launch(p, k_validate_cols, dim3(grid_for(mc + 1, 256, sm * 8), nm), 256, 0, va, p->d_err);
         if (mz > 0) launch(p, k_validate_rows, dim3(grid_for((mz + 3) / 4, 256, sm * 16), nm), 256, 0, va, p->d_err);
@@ -1144,21 +1134,15 @@ static spg_status plan_build(spg_plan *p) {
     }
 
     // --- step 1: D and H_i
-    p->W = (k + 31) / 32;
-    const int64_t W = p->W;
     p->Dbits = (uint32_t *)ws_alloc(p, sizeof(uint32_t) * (size_t)(W + 1));
-    p->Hbits = (uint32_t *)ws_alloc(p, sizeof(uint32_t) * (size_t)(P * W + 1));
     p->rankpre = (int64_t *)ws_alloc(p, sizeof(int64_t) * (size_t)(P * W + 1));
-    int32_t *popc = (int32_t *)ws_alloc(p, sizeof(int32_t) * (size_t)(P * W + 1));
     p->nfb = (k + p->b - 1) / p->b;
     p->fetch = (uint8_t *)ws_alloc(p, (size_t)(P * p->nfb + 1));
-    if (!p->Dbits || !p->Hbits || !p->rankpre || !popc || !p->fetch) return SPG_OUT_OF_MEMORY;
+    if (!p->Dbits || !p->rankpre || !p->fetch) return SPG_OUT_OF_MEMORY;
     p->eoff = (int64_t *)ws_alloc(p, sizeof(int64_t) * (size_t)(P + 1));
     if (!p->eoff) return SPG_OUT_OF_MEMORY;
-    TRY(cuda_check(cudaMemsetAsync(p->Hbits, 0, sizeof(uint32_t) * (size_t)(P * W + 1), st), "memset H"));
-    if (W > 0) launch(p, k_nonempty_bits, grid_for(W, 256, sm * 8), 256, 0, A.colptr, p64A, k, W, p->Dbits);
-    launch(p, k_block_eoff, grid_for(P + 1, 256, sm), 256, 0, B.colptr, p64B, n, P, (const int64_t *)p->bounds_d,
-           p->eoff);
+    launch(p, k_nonempty_bits, grid_for(std::max<int64_t>(W, P + 1), 256, sm * 8), 256, 0, A.colptr, p64A, k, W,
+           p->Dbits, B.colptr, p64B, n, P, (const int64_t *)p->bounds_d, p->eoff);
     if (B.nnz > 0)
         launch(p, k_mark_H, grid_for(B.nnz, 256, sm * 16), 256, 0, B.rowidx, i64B, B.nnz, P, k, W, p->Hbits,
                (const int64_t *)p->eoff);
@@ -1166,10 +1150,7 @@ static spg_status plan_build(spg_plan *p) {
 
     // --- step 2: D~_i = H_i & D, its ranks and Algorithm 2
     int64_t PW = (int64_t)P * W;
-    if (PW > 0)
-        launch(p, k_popc_HD, grid_for(PW, 256, sm * 8), 256, 0, p->Hbits, p->Dbits, W, PW, popc,
-                                                            (long long *)(p->d_cnt + kCntSumH));
-    TRY(scan_exclusive_i32(p, popc, p->rankpre, PW));
+    TRY(scan_exclusive_bits(p, p->Hbits, p->Dbits, W, p->rankpre, PW));
     // |D~| in total and per block: the block boundaries of the scan
     int64_t *d_dt_base = (int64_t *)ws_alloc(p, sizeof(int64_t) * (size_t)(P + 1));
     if (!d_dt_base) return SPG_OUT_OF_MEMORY;
@@ -1186,11 +1167,10 @@ static spg_status plan_build(spg_plan *p) {
         glen = (int64_t *)ws_alloc(p, sizeof(int64_t) * (size_t)(cap + 1));
         if (!p->dtilde || !p->At_colptr || !glen) return SPG_OUT_OF_MEMORY;
         if (PW > 0)
-            launch(p, k_dtilde, grid_for(PW, 256, sm * 8), 256, 0, p->Hbits, p->Dbits, p->rankpre, W, PW, p->dtilde);
-        if (P * p->nfb > 0)
-            launch(p, k_fetch, grid_for(P * p->nfb, 256, sm * 8), 256, 0, p->Hbits, p->Dbits, p->rankpre, W, k, p->b,
-                   p->nfb, P, A.colptr, p64A, p->fetch, (long long *)(p->d_cnt + kCntFetchChosen),
-                   (long long *)(p->d_cnt + kCntVolBlock));
+            launch(p, k_dtilde, grid_for(std::max(PW, P * p->nfb), 256, sm * 8), 256, 0, p->Hbits, p->Dbits,
+                   p->rankpre, W, PW, p->dtilde, k, p->b, p->nfb, P, A.colptr, p64A, p->fetch,
+                   (long long *)(p->d_cnt + kCntFetchChosen), (long long *)(p->d_cnt + kCntVolBlock),
+                   (long long *)(p->d_cnt + kCntSumH));
         LAUNCH_OK("dtilde / fetch");
         // --- step 3: gather A~
         if (cap > 0)
@@ -1258,9 +1238,8 @@ static spg_status plan_build(spg_plan *p) {
                wide ? grid_for(n, 1, sm * 8) : grid_for(n * 8, 256, sm * 16), 256, 0, B.colptr, p64B, n, p->Bq,
                p->At_colptr, p->At_row, out, (long long *)(p->d_cnt + kCntBin0),
                (long long *)(p->d_cnt + kCntProducts));
-        launch(p, k_block_flops, grid_for(n, 256, sm * 8), 256, 0, p->flops, n, P, p->bounds_d, (long long *)p->blk);
         LAUNCH_OK("column stats");
-        TRY(bin_columns_queue(p, p->bin_of, p->binlist));
+        TRY(bin_columns_queue(p, p->bin_of, p->binlist, 1));
     }
     TRY(read_counters());
     if (n > 0) bin_offsets(p, p->bin_off);

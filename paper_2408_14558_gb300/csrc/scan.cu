@@ -13,15 +13,31 @@ constexpr int kScanThreads = 256;
 constexpr int kScanPer = 8;
 constexpr int kScanTile = kScanThreads * kScanPer;
 
+// What is scanned: an array, or the population counts of H & D (D's W words
+// again for every block of H).
 template <typename T>
-__global__ void k_scan_reduce(const T *__restrict__ in, int64_t n, long long *__restrict__ part) {
+struct ScanArray {
+    const T *in;
+    __device__ __forceinline__ long long operator()(int64_t i) const { return (long long)in[i]; }
+};
+struct ScanBits {
+    const uint32_t *H, *D;
+    int64_t W;
+    __device__ __forceinline__ long long operator()(int64_t i) const {
+        const int64_t w = (i | W) >> 32 ? i % W : (int64_t)((uint32_t)i % (uint32_t)W);
+        return __popc(H[i] & D[w]);
+    }
+};
+
+template <typename T>
+__global__ void k_scan_reduce(const T in, int64_t n, long long *__restrict__ part) {
     __shared__ long long red[kScanThreads / 32];
     int64_t base = (int64_t)blockIdx.x * kScanTile;
     long long s = 0;
 #pragma unroll
     for (int i = 0; i < kScanPer; i++) {
         int64_t idx = base + (int64_t)i * kScanThreads + threadIdx.x;
-        if (idx < n) s += (long long)in[idx];
+        if (idx < n) s += in(idx);
     }
     s = warp_sum_ll(s);
     if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = s;
@@ -77,7 +93,7 @@ constexpr int64_t kScanOne = 1024 * kScanPer, kScanTiles = 4096;
 // their scanned prefixes.
 template <bool SUM, typename T>
 __global__ void __launch_bounds__(kScanThreads)
-    k_scan_tiles(const T *__restrict__ in, int64_t n, const long long *__restrict__ part, int64_t *__restrict__ out) {
+    k_scan_tiles(const T in, int64_t n, const long long *__restrict__ part, int64_t *__restrict__ out) {
     __shared__ long long wsum[kScanThreads / 32], psum[kScanThreads / 32];
     int64_t base = (int64_t)blockIdx.x * kScanTile;
     // each thread owns kScanPer consecutive elements
@@ -86,7 +102,7 @@ __global__ void __launch_bounds__(kScanThreads)
     int64_t my = base + (int64_t)threadIdx.x * kScanPer;
 #pragma unroll
     for (int i = 0; i < kScanPer; i++) {
-        v[i] = (my + i < n) ? (long long)in[my + i] : 0;
+        v[i] = (my + i < n) ? in(my + i) : 0;
         run += v[i];
     }
     int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
@@ -121,7 +137,7 @@ __global__ void __launch_bounds__(kScanThreads)
 // The whole scan by one CTA, 8192 elements at a time (7 us each: one such tile
 // costs as much as two launches).
 template <typename T>
-__global__ void __launch_bounds__(1024) k_scan_one(const T *__restrict__ in, int64_t n, int64_t *__restrict__ out) {
+__global__ void __launch_bounds__(1024) k_scan_one(const T in, int64_t n, int64_t *__restrict__ out) {
     __shared__ long long wsum[2][32];
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
     long long carry = 0;
@@ -131,7 +147,7 @@ __global__ void __launch_bounds__(1024) k_scan_one(const T *__restrict__ in, int
         long long v[kScanPer], run = 0;
 #pragma unroll
         for (int i = 0; i < kScanPer; i++) {
-            v[i] = my + i < n ? (long long)in[my + i] : 0;
+            v[i] = my + i < n ? in(my + i) : 0;
             run += v[i];
         }
         long long incl = run;
@@ -155,7 +171,7 @@ __global__ void __launch_bounds__(1024) k_scan_one(const T *__restrict__ in, int
 }
 
 template <typename T>
-static spg_status scan_impl(spg_plan *p, const T *in, int64_t *out, int64_t n) {
+static spg_status scan_impl(spg_plan *p, const T in, int64_t *out, int64_t n) {
     if (n == 0) {
         return cuda_check(cudaMemsetAsync(out, 0, sizeof(int64_t), p->st), "scan memset");
     }
@@ -177,10 +193,14 @@ static spg_status scan_impl(spg_plan *p, const T *in, int64_t *out, int64_t n) {
 }
 
 spg_status scan_exclusive_i32(spg_plan *p, const int32_t *in, int64_t *out, int64_t n) {
-    return scan_impl<int32_t>(p, in, out, n);
+    return scan_impl(p, ScanArray<int32_t>{in}, out, n);
 }
 spg_status scan_exclusive_i64(spg_plan *p, const int64_t *in, int64_t *out, int64_t n) {
-    return scan_impl<int64_t>(p, in, out, n);
+    return scan_impl(p, ScanArray<int64_t>{in}, out, n);
+}
+
+spg_status scan_exclusive_bits(spg_plan *p, const uint32_t *H, const uint32_t *D, int64_t W, int64_t *out, int64_t n) {
+    return scan_impl(p, ScanBits{H, D, W}, out, n);
 }
 
 }  // namespace spg

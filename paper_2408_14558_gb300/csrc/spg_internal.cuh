@@ -151,7 +151,6 @@ struct spg_plan {
     int64_t *eoff = nullptr;         // first entry of B of every column block (P + 1)
     std::vector<int64_t> bounds_h;   // the bounds in effect (P + 1), host
     int64_t *blk = nullptr;          // per block: flops, gathered A~ nonzeros, of them fetched (3 x P)
-    int64_t *gshift = nullptr;       // per A~ column: its entries' offset into A (gather)
     bool c_on_host = false;          // the numeric pass stores C into host memory
     bool numeric_done = false;       // a numeric pass ran: the light lists and item headers exist
     cudaGraph_t graph = nullptr;     // captured refresh + numeric (spgemm_plan_capture)
@@ -251,10 +250,12 @@ int grid_for(int64_t work, int per_block, int max_blocks);
 // ---- scans (scan.cu): out[0..n] = exclusive prefix of in[0..n), out[n] = total.
 spg_status scan_exclusive_i32(spg_plan *p, const int32_t *in, int64_t *out, int64_t n);
 spg_status scan_exclusive_i64(spg_plan *p, const int64_t *in, int64_t *out, int64_t n);
+// of popc(H[i] & D[i % W])
+spg_status scan_exclusive_bits(spg_plan *p, const uint32_t *H, const uint32_t *D, int64_t W, int64_t *out, int64_t n);
 
 // ---- binning (plan.cu): group the columns whose bin id is in bin_of into binlist.
-spg_status bin_columns(spg_plan *p, const int8_t *bin_of, int32_t *list, int64_t *off_host);
-spg_status bin_columns_queue(spg_plan *p, const int8_t *bin_of, int32_t *list);
+spg_status bin_columns(spg_plan *p, int8_t *bin_of, int32_t *list, int64_t *off_host);
+spg_status bin_columns_queue(spg_plan *p, int8_t *bin_of, int32_t *list, int mode);
 void bin_offsets(const spg_plan *p, int64_t *off_host);
 
 // ---- hub columns of A (symbolic.cu): lengths by power of two, read back in the plan
