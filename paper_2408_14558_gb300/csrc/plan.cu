@@ -183,12 +183,31 @@ __global__ void k_validate_cols(ValidateArgs args, int *err) {
     const int64_t t0 = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (t0 == 0 && (ld_ptr(v.colptr, v.p64, 0) != 0 || ld_ptr(v.colptr, v.p64, v.ncols) != v.nnz))
         atomicOr(err, kDevErrInput);
-    for (int64_t j = t0; j < v.ncols; j += (int64_t)gridDim.x * blockDim.x) {
-        const int64_t s = ld_ptr(v.colptr, v.p64, j), e = ld_ptr(v.colptr, v.p64, j + 1);
-        if (s > e || s < 0 || e > v.nnz)
-            atomicOr(err, kDevErrInput);
-        else if (s < e)
-            atomicOr(v.starts + (s >> 5), 1u << (s & 31));
+    // neighbouring columns mostly start in the same word: a warp ORs the bits of
+    // a run of equal words together first (2.1M one-entry columns: 32 atomics on
+    // a word became one)
+    const int lane = threadIdx.x & 31;
+    for (int64_t j0 = t0 - lane; j0 < v.ncols; j0 += (int64_t)gridDim.x * blockDim.x) {
+        const int64_t j = j0 + lane;
+        int64_t word = -1 - lane;  // (a word of its own: not one of its neighbours')
+        uint32_t bit = 0;
+        if (j < v.ncols) {
+            const int64_t s = ld_ptr(v.colptr, v.p64, j), e = ld_ptr(v.colptr, v.p64, j + 1);
+            if (s > e || s < 0 || e > v.nnz) {
+                atomicOr(err, kDevErrInput);
+            } else if (s < e) {
+                word = s >> 5;
+                bit = 1u << (s & 31);
+            }
+        }
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const int64_t w = __shfl_down_sync(kFull, word, o);
+            const uint32_t x = __shfl_down_sync(kFull, bit, o);
+            if (lane + o < 32 && w == word) bit |= x;
+        }
+        const int64_t before = __shfl_up_sync(kFull, word, 1);
+        if (word >= 0 && (lane == 0 || before != word)) atomicOr(v.starts + word, bit);
     }
 }
 
@@ -490,32 +509,29 @@ __global__ void k_gather_copy(const int64_t *__restrict__ At_colptr, const int32
         const uint32_t b = __ballot_sync(kFull, idx < hi && At_colptr[idx] <= e0);
         lo += 31 - __clz(b);
     }
-    int64_t s0 = lo;  // the column holding entry f
+    // lane k holds column s0 + k: its start, and how far A's column begins from
+    // there; they serve every step up to entry `lim`, where column s0 + 32
+    // begins.  (Loading them anew for every 32 entries, each load waiting for the
+    // step before, took 98 us for 14.6M entries in columns of 7.)
+    int64_t s0 = lo, bk = 0, shk = 0, lim = -1;
     for (int64_t f = e0; f < e1; f += 32) {
-        // lane k holds column s0 + k: its start, and how far A's column begins
-        // from there
-        const int64_t sk = s0 + lane;
-        const int64_t bk = sk < ndt ? At_colptr[sk] : INT64_MAX;
-        const int64_t shk = sk < ndt ? ld_ptr(Acolptr, p64, dtilde[sk]) - bk : 0;
-        const int64_t pos = bk - f;  // >= 1 for k >= 1
-        const uint32_t M = __reduce_or_sync(kFull, (lane > 0 && pos < 32) ? (1u << (int)pos) : 0u);
-        const int k = __popc(M & ((2u << lane) - 1u));
-        const int64_t sh = __shfl_sync(kFull, shk, k);
+        if (f + 32 > lim) {
+            if (lim >= 0) s0 += __popc(__ballot_sync(kFull, bk <= f)) - 1;  // the column holding entry f
+            const int64_t sk = s0 + lane;
+            bk = sk < ndt ? At_colptr[sk] : INT64_MAX;
+            shk = sk < ndt ? ld_ptr(Acolptr, p64, dtilde[sk]) - bk : 0;
+            lim = s0 + 32 < ndt ? At_colptr[s0 + 32] : INT64_MAX;
+        }
+        const int base = __popc(__ballot_sync(kFull, bk <= f)) - 1;
+        const uint64_t pos = (uint64_t)(bk - f);
+        const uint32_t M = __reduce_or_sync(kFull, pos - 1 < 31 ? 1u << (int)pos : 0u);
+        const int64_t sh = __shfl_sync(kFull, shk, base + __popc(M & ((2u << lane) - 1u)));
         const int64_t e = f + lane;
         if (e < e1) {
             const int64_t src = e + sh;
             At_row[e] = (int32_t)ld_ptr(Arow, i64, src);
             At_val[e] = load_val<Acc>(Aval, vt, src);
         }
-        // the column holding f + 32
-        int c = __popc(M);
-        int64_t nb;
-        if (c < 31)
-            nb = __shfl_sync(kFull, bk, c + 1);
-        else
-            nb = s0 + 32 < ndt ? At_colptr[s0 + 32] : INT64_MAX;
-        if (nb == f + 32) c++;
-        s0 += c;
     }
 }
 
