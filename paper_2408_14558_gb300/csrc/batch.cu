@@ -12,7 +12,7 @@
 //     warp that finishes an instance's last symbolic task scans its counts into
 //     the instance's column pointers and publishes a ready flag;
 //   numeric task: waits (bounded) for the instance's flag, then per column a
-//     warp hash of (row, value), compaction, bitonic sort, and the column is
+//     warp table of (row, value), compaction, sort by row, and the column is
 //     written at its place.
 // Because all symbolic tasks precede all numeric ones in the queue, a warp
 // that waits only waits for warps that already hold their tasks.  The wait is

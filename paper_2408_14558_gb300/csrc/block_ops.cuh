@@ -1,53 +1,15 @@
-// CTA- and warp-level helpers shared by the numeric and learned kernels.
+// CTA-level helpers shared by the numeric, learned and batched kernels: scans,
+// accumulators, rank tables.
 #pragma once
 
 #include "spg_internal.cuh"
 
 namespace spg {
 
-// Exclusive scan of popc(bits[w]) over the RW words of a slab by the whole CTA.
-// Writes pre[0..RW) and returns the total to every thread.
-__device__ __forceinline__ int cta_scan_popc(const uint32_t *bits, int *pre, int RW, int *wsum) {
-    const int nt = blockDim.x, tid = threadIdx.x;
-    const int per = (RW + nt - 1) / nt;
-    const int w0 = tid * per;
-    int local = 0;
-    for (int w = w0; w < min(RW, w0 + per); w++) local += __popc(bits[w]);
-    const int lane = tid & 31, wid = tid >> 5;
-    int incl = local;
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-        int t = __shfl_up_sync(kFull, incl, o);
-        if (lane >= o) incl += t;
-    }
-    if (lane == 31) wsum[wid] = incl;
-    __syncthreads();
-    if (wid == 0) {
-        int nw = nt >> 5;
-        int v = lane < nw ? wsum[lane] : 0;
-        int vi = v;
-#pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-            int t = __shfl_up_sync(kFull, vi, o);
-            if (lane >= o) vi += t;
-        }
-        if (lane < nw) wsum[lane] = vi - v;
-        if (lane == 31) wsum[32] = vi;
-    }
-    __syncthreads();
-    int run = wsum[wid] + incl - local;
-    for (int w = w0; w < min(RW, w0 + per); w++) {
-        pre[w] = run;
-        run += __popc(bits[w]);
-    }
-    int total = wsum[32];
-    __syncthreads();
-    return total;
-}
-
-// The same scan with one barrier: pre[] is complete for every thread only
-// after the caller's next barrier, and wsum must not be written again before
-// that barrier.
+// Exclusive scan of popc(bits[w]) over n words by the whole CTA: writes
+// pre[0..n) and returns the total to every thread.  One barrier: pre[] is
+// complete for every thread only after the caller's next barrier, and wsum must
+// not be written again before that barrier.
 __device__ __forceinline__ int cta_scan_popc1(const uint32_t *bits, int *pre, int n, int *wsum) {
     const int nt = blockDim.x, tid = threadIdx.x;
     const int per = (n + nt - 1) / nt;
@@ -70,38 +32,6 @@ __device__ __forceinline__ int cta_scan_popc1(const uint32_t *bits, int *pre, in
     for (int w = w0; w < min(n, w0 + per); w++) {
         pre[w] = run;
         run += __popc(bits[w]);
-    }
-    return total;
-}
-
-// The same scan over packed (word, prefix) pairs: fills bp[w].y and returns
-// the total to every thread.  One barrier: every warp then reads all warp
-// totals and takes its own offset, so the y fields are complete for every
-// thread only after the caller's next barrier, and wsum must not be written
-// again before that barrier.
-__device__ __forceinline__ int cta_scan_popc_packed(uint2 *bp, int n, int *wsum) {
-    const int nt = blockDim.x, tid = threadIdx.x;
-    const int per = (n + nt - 1) / nt;
-    const int w0 = tid * per;
-    int local = 0;
-    for (int w = w0; w < min(n, w0 + per); w++) local += __popc(bp[w].x);
-    const int lane = tid & 31, wid = tid >> 5, nw = nt >> 5;
-    int incl = local;
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-        int t = __shfl_up_sync(kFull, incl, o);
-        if (lane >= o) incl += t;
-    }
-    if (lane == 31) wsum[wid] = incl;
-    __syncthreads();
-    // lane l < nw holds warp l's total; the warps before this one give its offset
-    const int wt = lane < nw ? wsum[lane] : 0;
-    const int before = __reduce_add_sync(kFull, lane < wid ? wt : 0);
-    const int total = __reduce_add_sync(kFull, wt);
-    int run = before + incl - local;
-    for (int w = w0; w < min(n, w0 + per); w++) {
-        bp[w].y = (uint32_t)run;
-        run += __popc(bp[w].x);
     }
     return total;
 }

@@ -39,7 +39,6 @@ namespace {
 // Table classes: 2^8 slots per warp and 32 warps per CTA (column bounds up to
 // 128), or 2^10 slots and 8 warps (bounds up to 512); one CTA per SM.
 constexpr int kSmallClassLog[2] = {8, 10};
-constexpr int kSmallClassWarps[2] = {32, 8};
 constexpr int kNumBarriers = 2;
 
 // result block (device int64, caller-owned)

@@ -415,10 +415,6 @@ constexpr int kLongSeg = 32;
 constexpr int mid_seg(int threads) { return threads <= 256 ? 256 : 65536 / threads; }
 constexpr int short_windows(int threads) { return (threads * (kLongSeg - 1) + 31) / 32; }
 
-__device__ __forceinline__ unsigned hash_row(int r, int shift) {
-    return ((unsigned)r * 0x9E3779B1u) >> shift;
-}
-
 __device__ __forceinline__ int warp_sum_i(int v) {
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(kFull, v, o);
