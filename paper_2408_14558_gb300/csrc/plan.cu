@@ -516,7 +516,10 @@ __global__ void k_gather_copy(const int64_t *__restrict__ At_colptr, const int32
     int64_t s0 = lo, bk = 0, shk = 0, lim = -1;
     for (int64_t f = e0; f < e1; f += 32) {
         if (f + 32 > lim) {
-            if (lim >= 0) s0 += __popc(__ballot_sync(kFull, bk <= f)) - 1;  // the column holding entry f
+            // the column holding entry f: one of the 32, or the next where f
+            // begins it (from a column earlier, 31 columns of one entry behind
+            // f's would not fit the 32 that the lanes hold)
+            if (lim >= 0) s0 += f == lim ? 32 : __popc(__ballot_sync(kFull, bk <= f)) - 1;
             const int64_t sk = s0 + lane;
             bk = sk < ndt ? At_colptr[sk] : INT64_MAX;
             shk = sk < ndt ? ld_ptr(Acolptr, p64, dtilde[sk]) - bk : 0;

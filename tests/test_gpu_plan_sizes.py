@@ -82,6 +82,22 @@ def test_validation_finds_a_bad_row_at_every_alignment(offset, at):
     assert_full_parity(g.multiply(M, M, 2, 16), oracle.spgemm(A, A), "restored")
 
 
+@pytest.mark.parametrize("lens", [[1], [1] * 31 + [2], [2] + [1] * 31, [1, 1, 40], [32], [1, 2]])
+@pytest.mark.parametrize("P", [1, 5])
+def test_gather_of_scattered_short_columns(lens, P):
+    """A~'s columns of one entry or little more, picked from A with gaps: a
+    32-entry step meets up to 32 columns, wherever the 32 that the lanes hold end."""
+    rng = np.random.default_rng(len(lens) + P)
+    n = 6000
+    cols = np.repeat(np.arange(n), np.resize(lens, n))
+    rows = np.concatenate([np.sort(rng.choice(n, k, replace=False)) for k in np.resize(lens, n)])
+    A = synth._csc_from_sorted(n, n, cols, rows, rng.uniform(-1, 1, rows.size))
+    for per in (3, 40):   # B's columns need some of A's only
+        picks = np.concatenate([np.sort(rng.choice(n, per, replace=False)) for _ in range(60)])
+        B = synth._csc_from_sorted(n, 60, np.repeat(np.arange(60), per), picks, rng.uniform(-1, 1, picks.size))
+        assert_full_parity(run_gpu(A, B, P, 64), oracle.spgemm(A, B), f"per={per}")
+
+
 @pytest.mark.parametrize("lens", [[520] * 30, [700, 0, 4000, 1, 513] * 4])
 def test_long_columns_of_B(lens):
     """A mean above 512 entries per column of B: one CTA per column in the statistics."""
