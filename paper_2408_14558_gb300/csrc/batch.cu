@@ -217,7 +217,7 @@ __global__ void k_batch_persistent(const BatchInst *__restrict__ insts, const Ba
                 bool full = false;
                 warp_walk<false, 4, Acc>(
                     p0, p1, lane, ws, in.Arow, seg, [](long long) { return Acc(0); },
-                    [&](int r, Acc, Acc, bool ok) {
+                    [&](int r, Acc, Acc, bool ok, auto) {
                         if (warp_hash_slot(skeys, logS, r, ok) < 0 && ok) full = true;
                     });
                 const int cnt = warp_count_keys(skeys, logS, lane);
@@ -252,11 +252,11 @@ __global__ void k_batch_persistent(const BatchInst *__restrict__ insts, const Ba
                 tab.clear(lane);
                 bool full = false;
                 // A's values may be stored as double, int32 or int64
-                warp_walk<true, 4, Acc>(
+                warp_walk<true, 4, Acc, HeavyAcc<Acc>::crowds>(
                     p0, p1, lane, ws, in.Arow, seg,
                     [&](long long e) { return bval_load<Acc>(in.Aval, in.vt, e); },
-                    [&](int r, Acc a, Acc b, bool ok) {
-                        if (!tab.add(acc, r, a, b, ok)) full = true;
+                    [&](int r, Acc a, Acc b, bool ok, auto crowded) {
+                        if (!tab.template add<decltype(crowded)::value>(acc, r, a, b, ok)) full = true;
                     });
                 __syncwarp();
                 const int nout = tab.compact(acc, lane);

@@ -51,6 +51,16 @@ __device__ __forceinline__ int cta_scan_popc1(const uint32_t *bits, int *pre, in
 // their instructions.  The marker is a signalling NaN: no arithmetic
 // instruction returns one, so no sum is taken for it.
 //
+// Where products crowd on few slots, that is slow: k lanes that want one slot
+// cost k rounds, and a 64-bit exchange of k lanes on a slot takes k passes, which
+// the holder's store waits for.  There add_crowded sums a warp's products of one
+// slot in registers first and adds the sum once (the walks find out by sampling a
+// window, see window_crowds).  100,000 products a column, 99% of them on one row:
+// exchanges alone 14.7 ms, DMUL + atomicAdd 10.0, combined 1.2; all of a light
+// column's products on four rows 0.76, 0.37 and 0.31 ms.  Combining inside
+// add_products (after a few tries, without sampling) made squaring an R-MAT graph
+// 12% slower: its registers and votes count in every step.
+//
 // Wrapping int64 sums are kept as two 32-bit halves in separate arrays: a
 // 64-bit add is a 32-bit atomic add on the low half that returns the old low
 // word, from which the carry out of the low half follows exactly; the high
@@ -79,10 +89,31 @@ __device__ __forceinline__ void shared_red32(uint32_t addr, uint32_t v) {
     asm volatile("red.shared.add.u32 [%0], %1;" ::"r"(addr), "r"(v));
 }
 
+
+// The sum of v over the lanes of `peers` (a group of lanes that this one belongs
+// to; the whole warp calls it), in the lowest lane of the group.  In every step
+// the group's lanes of odd rank hand their sums to the lane before them and drop
+// out, and the ranks of the others halve.
+__device__ __forceinline__ double warp_sum_peers(unsigned peers, int lane, double v) {
+    unsigned rank = __popc(peers & ((1u << lane) - 1u));
+    unsigned above = peers & (~1u << lane);  // lanes of the group above this one that still hold a sum
+    bool live = true;
+    while (__any_sync(kFull, above != 0u)) {
+        const double t = __shfl_sync(kFull, v, above ? __ffs((int)above) - 1 : 0);
+        live = live && !(rank & 1u);
+        const unsigned hold = __ballot_sync(kFull, live);
+        if (live && above) v += t;
+        above = live ? above & hold : 0u;
+        rank >>= 1;
+    }
+    return v;
+}
+
 template <typename Acc>
 struct HeavyAcc;
 template <>
 struct HeavyAcc<double> {
+    static constexpr bool crowds = true;  // many products on one slot want add_crowded
     double *a;
     uint32_t sa;  // its shared-memory address
     static constexpr size_t bytes_per_slot = 8;
@@ -130,9 +161,21 @@ struct HeavyAcc<double> {
         }
         return true;
     }
+    // slot at address ad += x * y wherever ok, one product a lane (the whole warp
+    // calls it); false as above
+    __device__ __forceinline__ bool add_crowded(uint32_t ad, double x, double y, bool ok) const {
+        const int lane = threadIdx.x & 31;
+        const unsigned peers = __match_any_sync(kFull, ok ? ad : ~(uint32_t)lane);
+        const double v = warp_sum_peers(peers, lane, x * y);
+        if (!ok || lane != __ffs((int)peers) - 1) return true;
+        for (int t = 0; t < kSlotTries; t++)
+            if (try_add(ad, v, 1.0)) return true;
+        return false;
+    }
 };
 template <>
 struct HeavyAcc<long long> {
+    static constexpr bool crowds = false;
     uint32_t *lo, *hi;
     uint32_t sa, hoff;  // address of lo, distance of hi from lo in bytes
     static constexpr size_t bytes_per_slot = 8;
@@ -178,6 +221,18 @@ struct HeavyAcc<long long> {
         return true;
     }
 };
+
+// The products of a walk's step into their slots, in the walk's form.
+template <bool CROWDED, typename Acc, int N>
+__device__ __forceinline__ bool add_to(const HeavyAcc<Acc> &acc, const uint32_t (&ad)[N], const Acc (&x)[N],
+                                       const Acc (&y)[N], const bool (&ok)[N]) {
+    if constexpr (CROWDED) {
+        static_assert(N == 1, "a crowded walk takes one window at a time");
+        return acc.add_crowded(ad[0], x[0], y[0], ok[0]);
+    } else {
+        return acc.add_products(ad, x, y, ok);
+    }
+}
 
 // Rank table of a heavy item: one 32-bit entry per 16 rows, the rows' bits in
 // the low half, the number of set bits before them (at most 65,535) in the

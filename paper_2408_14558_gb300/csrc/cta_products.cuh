@@ -32,6 +32,7 @@ struct CtaBatch {
     uint2 win[kShortWindows];
     int cut[2];  // window segments and products of the middle class, if not all of it fits
     int next;    // next window to claim
+    bool crowded;  // the products of the last sampled batch crowd on few rows
     // all threads, once, before the first cta_products (which leaves the bits
     // clear again); a barrier must follow
     __device__ __forceinline__ void clear() {
@@ -92,9 +93,9 @@ __device__ __forceinline__ SegReg<Acc> cta_first_seg(int64_t p0, int64_t p1, Seg
 template <typename F>
 struct EachProduct {
     F f;
-    template <int N, typename Acc>
+    template <int N, typename Acc, typename Crowded>
     __device__ __forceinline__ void operator()(const int (&r)[N], const Acc (&a)[N], const Acc (&b)[N],
-                                               const bool (&ok)[N]) const {
+                                               const bool (&ok)[N], Crowded) const {
 #pragma unroll
         for (int u = 0; u < N; u++)
             if (ok[u]) f(r[u], mul_acc<Acc>(a[u], b[u]));
@@ -109,9 +110,9 @@ __device__ __forceinline__ EachProduct<F> each_product(F f) {
 // whole CTA (all threads must call it; blockDim.x == NT); `first` is
 // cta_first_seg(p0, p1, seg), and sb.clear() must have run once.
 // seg(p, start, len, bv) gives the A~ positions [start, start+len) that B'
-// entry p multiplies and its value; body(r, a, b, ok) takes this lane's next
-// N products: rows r[u], the factors a[u] (from A~) and b[u] (from B'), and
-// whether each exists.  The segments of the next batch are fetched before the
+// entry p multiplies and its value; body(r, a, b, ok, crowded) takes this lane's
+// next N products: rows r[u], the factors a[u] (from A~) and b[u] (from B'), and
+// whether each exists; the whole warp calls it.  The segments of the next batch are fetched before the
 // current batch is walked.
 // Long segments (>= kMidSeg entries): a warp takes steps of 32 x U products,
 // lanes reading consecutive entries, U loads per lane in flight.  A step inside
@@ -124,9 +125,13 @@ __device__ __forceinline__ EachProduct<F> each_product(F f) {
 // from one window to the next.
 // The long steps are shared evenly by the warps, the windows are claimed (few of
 // them: shared by number).
+// CROWD: body has a form for products that crowd on few rows (crowded is a true
+// type, N is 1).  Warp 0 looks at the first window of every eighth batch that
+// has a next one, and the batches after it take that form where it crowds
+// (segments of 32 entries or more cannot: their rows are distinct).
 // One batch must hold < 2^31 products (heavy items bound their segments to the
 // item's row range).  Ends with a barrier.
-template <bool NEED_VAL, int U, typename Acc, int NT, typename SegFn, typename Body>
+template <bool NEED_VAL, int U, typename Acc, bool CROWD = false, int NT, typename SegFn, typename Body>
 __device__ __forceinline__ void cta_products(int64_t p0, int64_t p1, CtaBatch<Acc, NT> &sb,
                                              const int32_t *__restrict__ At_row, const Acc *__restrict__ At_val,
                                              SegReg<Acc> first, SegFn seg, Body body) {
@@ -138,6 +143,7 @@ __device__ __forceinline__ void cta_products(int64_t p0, int64_t p1, CtaBatch<Ac
         const long long st = cur.st;
         const int len = cur.len;
         const Acc bv = cur.bv;
+        const bool crowd = CROWD && b0 > p0 && sb.crowded;  // (written between the barriers below)
         // the shortest class numbers its products from 0 (windows), the middle
         // one from there on (windows, as far as they go), the longest after
         // the middle class's own products (long part); counts packed in one
@@ -173,6 +179,21 @@ __device__ __forceinline__ void cta_products(int64_t p0, int64_t p1, CtaBatch<Ac
             if (NEED_VAL) sb.bv[i] = bv;
         }
         __syncthreads();
+        if constexpr (CROWD) {
+            if (wid == 0 && b0 + NT < p1 && ((b0 - p0) / NT & 7) == 0) {
+                // the first window is made of this warp's own short segments:
+                // lane l's product belongs to the last one that begins by then
+                const bool mine = cls == 2 && len > 0;
+                const int e2 = (int)((uint32_t)ex[2] >> 16);
+                const uint32_t M = __reduce_or_sync(kFull, mine && e2 < 32 ? 1u << e2 : 0u);
+                const uint32_t segs = __ballot_sync(kFull, mine);
+                const bool ok = lane < __shfl_sync(kFull, mine ? e2 + len : e2, 31);
+                const int src = ok ? (int)__fns(segs, 0, __popc(M & (kFull >> (31 - lane)))) : 0;
+                const long long at = __shfl_sync(kFull, st - e2, src) + lane;
+                const bool crowds = window_crowds(ok ? __ldg(At_row + at) : ~lane);
+                if (lane == 0) sb.crowded = crowds;
+            }
+        }
         if (b0 + NT < p1) cur = cta_first_seg<Acc>(b0 + NT, p1, seg);
         // window segments [0, ns) with products [0, nsp), long segments
         // [ns, n) with products [lp0, lp1)
@@ -215,7 +236,7 @@ __device__ __forceinline__ void cta_products(int64_t p0, int64_t p1, CtaBatch<Ac
                 };
                 // one step of N windows over segment boundaries: located and
                 // loaded, then used
-                auto step = [&](const int f, auto windows, auto full) {
+                auto step = [&](const int f, auto windows, auto full, auto crowded) {
                     constexpr int N = decltype(windows)::value;
                     constexpr bool FULL = decltype(full)::value;  // no lane past the warp's range
                     int r[N];
@@ -237,11 +258,15 @@ __device__ __forceinline__ void cta_products(int64_t p0, int64_t p1, CtaBatch<Ac
                             if (NEED_VAL) a[u] = __ldg(At_val + e);
                         }
                     }
-                    body(r, a, bu, ok);
+                    body(r, a, bu, ok, crowded);
                 };
                 using One = std::integral_constant<int, 1>;
                 using All = std::integral_constant<int, U>;
                 int f = f0;
+                if constexpr (CROWD) {
+                    if (crowd)
+                        for (; f < f1; f += 32) step(f, One{}, std::false_type{}, std::true_type{});
+                }
                 while (f < f1) {
                     if (f >= nB) advance();
                     const int lim = min(nB, f1);
@@ -259,16 +284,16 @@ __device__ __forceinline__ void cta_products(int64_t p0, int64_t p1, CtaBatch<Ac
                                 bu[u] = bvA;
                                 ok[u] = true;
                             }
-                            body(r, a, bu, ok);
+                            body(r, a, bu, ok, std::false_type{});
                             f += 32 * U;
                             rp += 32 * U;
                             if (NEED_VAL) vp += 32 * U;
                         } while (f + 32 * U <= lim);
                     } else if (f + 32 * U <= f1) {
-                        step(f, All{}, std::true_type{});
+                        step(f, All{}, std::true_type{}, std::false_type{});
                         f += 32 * U;
                     } else {
-                        step(f, One{}, std::false_type{});
+                        step(f, One{}, std::false_type{}, std::false_type{});
                         f += 32;
                     }
                 }
@@ -285,7 +310,7 @@ __device__ __forceinline__ void cta_products(int64_t p0, int64_t p1, CtaBatch<Ac
         // claims are the better share: the betweenness batch 43.5 ms, 44.4 by number)
         {
             const uint32_t upto = kFull >> (31 - lane);
-            auto step = [&](const int w, auto windows, auto full) {
+            auto step = [&](const int w, auto windows, auto full, auto crowded) {
                 constexpr int N = decltype(windows)::value;
                 constexpr bool FULL = decltype(full)::value;
                 int r[N];
@@ -311,7 +336,7 @@ __device__ __forceinline__ void cta_products(int64_t p0, int64_t p1, CtaBatch<Ac
                 }
                 __syncwarp();
                 if (lane < N) sb.win[w + lane].x = 0u;
-                body(r, a, bu, ok);
+                body(r, a, bu, ok, crowded);
             };
             auto claim = [&]() {
                 int c = 0;
@@ -319,16 +344,19 @@ __device__ __forceinline__ void cta_products(int64_t p0, int64_t p1, CtaBatch<Ac
                 return __shfl_sync(kFull, c, 0);
             };
             using One = std::integral_constant<int, 1>;
-            if (nwin <= nw) {
-                if (wid < nwin) step(wid, One{}, std::false_type{});
+            if (CROWD && crowd) {
+                if constexpr (CROWD)
+                    for (int w = wid; w < nwin; w += nw) step(w, One{}, std::false_type{}, std::true_type{});
+            } else if (nwin <= nw) {
+                if (wid < nwin) step(wid, One{}, std::false_type{}, std::false_type{});
             } else {
                 const bool few = nsteps == 0 && nwin <= nw * U;  // one claim a warp: its own number
                 for (int w = few ? wid * U : claim(); w < nwin;) {
                     const int wnext = few ? nwin : claim();
                     if ((w + U) * 32 <= nsp) {
-                        step(w, std::integral_constant<int, U>{}, std::true_type{});
+                        step(w, std::integral_constant<int, U>{}, std::true_type{}, std::false_type{});
                     } else {
-                        for (; w < nwin; w++) step(w, One{}, std::false_type{});
+                        for (; w < nwin; w++) step(w, One{}, std::false_type{}, std::false_type{});
                     }
                     w = wnext;
                 }

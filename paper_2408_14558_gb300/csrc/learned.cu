@@ -246,7 +246,7 @@ __global__ void __launch_bounds__(WARPS * 32)
         const int64_t p0 = ld_ptr(Bcolptr, p64, j), p1 = ld_ptr(Bcolptr, p64, j + 1);
         tab.clear(lane);
         bool full = false;
-        warp_walk<true, 4, Acc>(
+        warp_walk<true, 4, Acc, HeavyAcc<Acc>::crowds>(
             p0, p1, lane, segs[wid], At_row,
             [&](int64_t p, long long &st, int &len, Acc &bv) {
                 int q = Bq[p];
@@ -257,8 +257,8 @@ __global__ void __launch_bounds__(WARPS * 32)
                 }
             },
             [&](long long e) { return __ldg(At_val + e); },
-            [&](int r, Acc a, Acc b, bool ok) {
-                if (!tab.add(acc, r, a, b, ok)) full = true;
+            [&](int r, Acc a, Acc b, bool ok, auto crowded) {
+                if (!tab.template add<decltype(crowded)::value>(acc, r, a, b, ok)) full = true;
             });
         __syncwarp();
         const int nout = tab.compact(acc, lane);
@@ -336,8 +336,9 @@ __global__ void __launch_bounds__(kBatch)
         const uint32_t abase = acc.addr(0) - ((uint32_t)rbase << HeavyAcc<Acc>::slot_shift);
         unsigned char *sbase = seen - rbase;
         bool stuck = false;
-        cta_products<true, SPG_NUM_UNROLL, Acc>(
-            p0, p1, sb, At_row, At_val, first, seg, [&](const auto &r, const auto &a, const auto &b, const auto &ok) {
+        cta_products<true, SPG_NUM_UNROLL, Acc, HeavyAcc<Acc>::crowds>(
+            p0, p1, sb, At_row, At_val, first, seg,
+            [&](const auto &r, const auto &a, const auto &b, const auto &ok, auto crowded) {
                 constexpr int N = sizeof(r) / sizeof(r[0]);
                 uint32_t ad[N];
 #pragma unroll
@@ -345,7 +346,7 @@ __global__ void __launch_bounds__(kBatch)
                     ad[u] = abase + ((uint32_t)r[u] << HeavyAcc<Acc>::slot_shift);
                     if (ok[u]) sbase[r[u]] = 1;
                 }
-                if (!acc.add_products(ad, a, b, ok)) stuck = true;
+                if (!add_to<decltype(crowded)::value>(acc, ad, a, b, ok)) stuck = true;
             });
         if (stuck) atomicOr(err, kDevErrInternal);
         // thread w puts word w together (and clears its bytes); the scan then

@@ -39,7 +39,7 @@ __global__ void __launch_bounds__(WARPS * 32, LOGS <= 8 ? 8 : 1)
         const int64_t base = Ccolptr[j], want = Ccolptr[j + 1] - base;
         tab.clear(lane);
         bool full = false;
-        warp_walk<true, (LOGS <= 8 ? 2 : 4), Acc>(
+        warp_walk<true, (LOGS <= 8 ? 2 : 4), Acc, HeavyAcc<Acc>::crowds>(
             p0, p1, lane, segs[wid], At_row,
             [&](int64_t p, long long &st, int &len, Acc &bv) {
                 int q = Bq[p];
@@ -50,9 +50,9 @@ __global__ void __launch_bounds__(WARPS * 32, LOGS <= 8 ? 8 : 1)
                 }
             },
             [&](long long e) { return __ldg(At_val + e); },
-            [&](int r, Acc a, Acc b, bool ok) {
+            [&](int r, Acc a, Acc b, bool ok, auto crowded) {
                 if (mask.bits && ok && !mask_keeps(mask, j, r)) ok = false;
-                if (!tab.add(acc, r, a, b, ok)) full = true;
+                if (!tab.template add<decltype(crowded)::value>(acc, r, a, b, ok)) full = true;
             });
         __syncwarp();
         const int nout = tab.compact(acc, lane);
@@ -192,9 +192,9 @@ __global__ void __launch_bounds__(NT, SPG_NUM_MINB * kBatch / NT)
             bool miss = false;
             if (direct) {
                 const uint32_t base = slot0 - ((uint32_t)rbase << kSlotShift);
-                cta_products<true, SPG_NUM_UNROLL, Acc>(
+                cta_products<true, SPG_NUM_UNROLL, Acc, HeavyAcc<Acc>::crowds>(
                     h.p0, h.p1, sb, At_row, At_val, first, seg,
-                    [&](const auto &r, const auto &a, const auto &b, const auto &ok) {
+                    [&](const auto &r, const auto &a, const auto &b, const auto &ok, auto crowded) {
                         constexpr int N = sizeof(r) / sizeof(r[0]);
                         uint32_t ad[N];
 #pragma unroll
@@ -204,13 +204,13 @@ __global__ void __launch_bounds__(NT, SPG_NUM_MINB * kBatch / NT)
                             if (ok[u]) miss |= !MASKED && !((rank_word(tab[(r[u] - (int)rbase) >> 5]) >> (r[u] & 31)) & 1u);
 #endif
                         }
-                        if (!acc.add_products(ad, a, b, ok)) miss = true;
+                        if (!add_to<decltype(crowded)::value>(acc, ad, a, b, ok)) miss = true;
                     });
             } else {
                 const uint32_t *ranks = (const uint32_t *)tab - 2 * t0 * RW;
-                cta_products<true, SPG_NUM_UNROLL, Acc>(
+                cta_products<true, SPG_NUM_UNROLL, Acc, HeavyAcc<Acc>::crowds>(
                     h.p0, h.p1, sb, At_row, At_val, first, seg,
-                    [&](const auto &r, const auto &a, const auto &b, const auto &ok) {
+                    [&](const auto &r, const auto &a, const auto &b, const auto &ok, auto crowded) {
                         constexpr int N = sizeof(r) / sizeof(r[0]);
                         uint32_t ad[N];
                         bool keep[N];
@@ -236,7 +236,7 @@ __global__ void __launch_bounds__(NT, SPG_NUM_MINB * kBatch / NT)
                                 }
                             }
                         }
-                        if (!acc.add_products(ad, a, b, keep)) miss = true;
+                        if (!add_to<decltype(crowded)::value>(acc, ad, a, b, keep)) miss = true;
                     });
             }
             if (miss) bad_sh = 1;

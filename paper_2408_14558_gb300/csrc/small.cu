@@ -205,7 +205,7 @@ __global__ void __launch_bounds__(WARPS * 32) k_small_multiply(SmallArgs a) {
                     }
                 },
                 [](long long) { return Acc(0); },
-                [&](int r, Acc, Acc, bool ok) {
+                [&](int r, Acc, Acc, bool ok, auto) {
                     if (warp_hash_slot(keys, lg, r, ok) < 0 && ok) full = true;
                 });
             c = warp_count_keys(keys, lg, lane);
@@ -331,7 +331,7 @@ __global__ void __launch_bounds__(WARPS * 32) k_small_multiply(SmallArgs a) {
         tab.clear(lane);
         const int64_t p0 = ld_ptr(a.Bcp, a.bp64, j), p1 = ld_ptr(a.Bcp, a.bp64, j + 1);
         bool full = false;
-        warp_walk<true, 4, Acc>(
+        warp_walk<true, 4, Acc, HeavyAcc<Acc>::crowds>(
             p0, p1, lane, segs[wid], a.Arow,
             [&](int64_t p, long long &st, int &len, Acc &bv) {
                 const int64_t kk = ld_ptr(a.Brow, a.bi64, p);
@@ -342,8 +342,8 @@ __global__ void __launch_bounds__(WARPS * 32) k_small_multiply(SmallArgs a) {
                 }
             },
             [&](long long e) { return ld_val<Acc>(a.Aval, a.avt, e); },
-            [&](int r, Acc x, Acc y, bool ok) {
-                if (!tab.add(acc, r, x, y, ok)) full = true;
+            [&](int r, Acc x, Acc y, bool ok, auto crowded) {
+                if (!tab.template add<decltype(crowded)::value>(acc, r, x, y, ok)) full = true;
             });
         __syncwarp();
         const int nout = tab.compact(acc, lane);

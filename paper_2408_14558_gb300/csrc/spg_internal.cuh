@@ -307,6 +307,16 @@ __device__ __forceinline__ long long mul_acc<long long>(long long a, long long b
     return (long long)((unsigned long long)a * (unsigned long long)b);
 }
 
+// Whether the products of a window crowd on few rows (row: this lane's, a number
+// of its own where it has none; the whole warp calls it): at least kCrowdLanes of
+// them share a row with kCrowdGroup others.  Graphs whose hub rows meet three or
+// four products of a window stay below (their walk is better off uncombined).
+constexpr int kCrowdGroup = 4, kCrowdLanes = 12;
+__device__ __forceinline__ bool window_crowds(int row) {
+    const unsigned peers = __match_any_sync(kFull, row);
+    return __popc(__ballot_sync(kFull, __popc(peers) > kCrowdGroup)) >= kCrowdLanes;
+}
+
 // Heavy items: the rows of a symbolic item have their bitmap in shared memory
 // (at most kSymMaxWords words = 262,144 rows), those of a numeric item their
 // packed (bitmap word, prefix) pairs (at most kNumMaxWords words = 65,536

@@ -39,7 +39,7 @@ __global__ void __launch_bounds__(WARPS * 32)
                 }
             },
             [&](long long) { return 0ll; },
-            [&](int r, long long, long long, bool ok) {
+            [&](int r, long long, long long, bool ok, auto) {
                 if (mask.bits && ok && !mask_keeps(mask, j, r)) ok = false;
                 if (warp_hash_slot(tab, LOGS, r, ok) < 0 && ok) full = true;
             });

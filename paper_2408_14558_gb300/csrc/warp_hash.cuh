@@ -16,71 +16,105 @@ struct WarpSeg {
     Acc bv[32];
 };
 
+// Stage the segments of the B' entries p0 + at .. p0 + at + 31 (below p0 + n): the
+// number of their products; `first` is this lane's first one (INT32_MAX for an
+// empty one).
+template <bool NEED_VAL, typename Acc, typename SegFn>
+__device__ __forceinline__ int warp_stage(int64_t p0, int at, int n, int lane, WarpSeg<Acc> &ws, SegFn &seg,
+                                          int &first) {
+    long long st = 0;
+    int len = 0;
+    Acc bv = Acc(0);
+    if (at + lane < n) seg(p0 + at + lane, st, len, bv);
+    int incl = len;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const int t = __shfl_up_sync(kFull, incl, o);
+        if (lane >= o) incl += t;
+    }
+    const int total = __shfl_sync(kFull, incl, 31);
+    first = len > 0 ? incl - len : INT32_MAX;
+    const uint32_t some = __ballot_sync(kFull, len > 0);
+    if (len > 0) {
+        const int i = __popc(some & ((1u << lane) - 1u));
+        ws.start[i] = st - first;
+        if (NEED_VAL) ws.bv[i] = bv;
+    }
+    __syncwarp();
+    return total;
+}
+
+// The windows of a staged batch.
+template <bool NEED_VAL, int U, bool CROWDED, typename Acc, typename ValFn, typename Body>
+__device__ __forceinline__ void warp_windows(int total, int first, int lane, const WarpSeg<Acc> &ws,
+                                             const int32_t *__restrict__ At_row, ValFn &aval, Body &body) {
+    const uint32_t upto = kFull >> (31 - lane);
+    int begun = -1;  // last segment begun before the window
+    for (int f0 = 0; f0 < total; f0 += 32 * U) {
+        int r[U];
+        Acc a[U], b[U];
+        bool ok[U];
+#pragma unroll
+        for (int u = 0; u < U; u++) {
+            const int f = f0 + 32 * u;
+            ok[u] = f + lane < total;
+            r[u] = 0;
+            a[u] = Acc(0);
+            b[u] = Acc(0);
+            if (f < total) {
+                const uint32_t d = (uint32_t)(first - f);
+                const uint32_t M = __reduce_or_sync(kFull, d < 32u ? 1u << d : 0u);
+                const int k = begun + __popc(M & upto);
+                begun += __popc(M);
+                if (ok[u]) {
+                    const long long e = ws.start[k] + (f + lane);
+                    r[u] = __ldg(At_row + e);
+                    if (NEED_VAL) {
+                        a[u] = aval(e);
+                        b[u] = ws.bv[k];
+                    }
+                }
+            }
+        }
+#pragma unroll
+        for (int u = 0; u < U; u++)
+            if (f0 + 32 * u < total) body(r[u], a[u], b[u], ok[u], std::integral_constant<bool, CROWDED>{});
+    }
+    __syncwarp();
+}
+
 // Walk every product of the B' entries [p0, p1) of one output column with a
 // whole warp.  seg(p, start, len, bv) gives the A~ positions [start, start+len)
 // that B' entry p multiplies and its value; aval(e) loads A~'s value e.  The
 // products of 32 consecutive entries are numbered consecutively; a window of 32
 // products finds its segments from one bit per segment start (an OR over the
 // lanes), so all 32 lanes stay busy however short the segments are.  U windows
-// are located and loaded before any of them is used.  body(r, a, b, ok) is
-// called by the whole warp, one product per lane where ok.
-template <bool NEED_VAL, int U, typename Acc, typename SegFn, typename ValFn, typename Body>
+// are located and loaded before any of them is used.  body(r, a, b, ok, crowded)
+// is called by the whole warp, one product per lane where ok.
+// CROWD: the body has a form for products that crowd on few rows (crowded is a
+// true type); a column of more than 32 entries takes it for 256 entries at a time
+// whose first window of products crowds (fewer entries bring at most as many
+// products of one row: not worth the look).
+template <bool NEED_VAL, int U, typename Acc, bool CROWD = false, typename SegFn, typename ValFn, typename Body>
 __device__ __forceinline__ void warp_walk(int64_t p0, int64_t p1, int lane, WarpSeg<Acc> &ws,
                                           const int32_t *__restrict__ At_row, SegFn seg, ValFn aval, Body body) {
-    const uint32_t upto = kFull >> (31 - lane);
-    for (int64_t base = p0; base < p1; base += 32) {
-        const int64_t p = base + lane;
-        long long st = 0;
-        int len = 0;
-        Acc bv = Acc(0);
-        if (p < p1) seg(p, st, len, bv);
-        int incl = len;
-#pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-            const int t = __shfl_up_sync(kFull, incl, o);
-            if (lane >= o) incl += t;
-        }
-        const int total = __shfl_sync(kFull, incl, 31);
-        const int first = len > 0 ? incl - len : INT32_MAX;
-        const uint32_t some = __ballot_sync(kFull, len > 0);
-        if (len > 0) {
-            const int at = __popc(some & (upto >> 1));
-            ws.start[at] = st - first;
-            if (NEED_VAL) ws.bv[at] = bv;
-        }
-        __syncwarp();
-        int begun = -1;  // last segment begun before the window
-        for (int f0 = 0; f0 < total; f0 += 32 * U) {
-            int r[U];
-            Acc a[U], b[U];
-            bool ok[U];
-#pragma unroll
-            for (int u = 0; u < U; u++) {
-                const int f = f0 + 32 * u;
-                ok[u] = f + lane < total;
-                r[u] = 0;
-                a[u] = Acc(0);
-                b[u] = Acc(0);
-                if (f < total) {
-                    const uint32_t d = (uint32_t)(first - f);
-                    const uint32_t M = __reduce_or_sync(kFull, d < 32u ? 1u << d : 0u);
-                    const int k = begun + __popc(M & upto);
-                    begun += __popc(M);
-                    if (ok[u]) {
-                        const long long e = ws.start[k] + (f + lane);
-                        r[u] = __ldg(At_row + e);
-                        if (NEED_VAL) {
-                            a[u] = aval(e);
-                            b[u] = ws.bv[k];
-                        }
-                    }
-                }
+    const int n = (int)(p1 - p0);  // (at most k < 2^31 - 1)
+    bool crowds = false;
+    for (int at = 0; at < n; at += 32) {
+        int first;
+        const int total = warp_stage<NEED_VAL>(p0, at, n, lane, ws, seg, first);
+        if constexpr (CROWD) {
+            if (n > 32 && (at & 255) == 0) {
+                const uint32_t M = __reduce_or_sync(kFull, first < 32 ? 1u << first : 0u);
+                const int k = __popc(M & (kFull >> (31 - lane))) - 1;
+                crowds = window_crowds(lane < total ? __ldg(At_row + ws.start[k] + lane) : ~lane);
             }
-#pragma unroll
-            for (int u = 0; u < U; u++)
-                if (f0 + 32 * u < total) body(r[u], a[u], b[u], ok[u]);
+            if (crowds) {
+                warp_windows<NEED_VAL, 1, true>(total, first, lane, ws, At_row, aval, body);
+                continue;
+            }
         }
-        __syncwarp();
+        warp_windows<NEED_VAL, U, false>(total, first, lane, ws, At_row, aval, body);
     }
 }
 
@@ -230,12 +264,13 @@ struct WarpTable {
         __syncwarp();
     }
     // body of warp_walk: a product of row r into its slot; false if the table is full
+    template <bool CROWDED>
     __device__ __forceinline__ bool add(const HeavyAcc<Acc> &acc, int r, Acc a, Acc b, bool ok) const {
         const int slot = warp_hash_slot(keys(), logS, r, ok);
         const uint32_t ad[1] = {acc.addr(max(slot, 0))};
         const Acc x[1] = {a}, y[1] = {b};
         const bool o[1] = {ok && slot >= 0};
-        return acc.add_products(ad, x, y, o) && (slot >= 0 || !ok);
+        return add_to<CROWDED>(acc, ad, x, y, o) && (slot >= 0 || !ok);
     }
     // Move the occupied slots' rows and values to the front; returns their
     // number.  (A write never reaches a slot of a later, still unread chunk.)
