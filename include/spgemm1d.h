@@ -165,6 +165,11 @@ void spgemm_default_options(spg_options *opt);
  * SPG_UNSUPPORTED (a semiring other than SPG_SEMIRING_PLUS_TIMES),
  * SPG_UNSUPPORTED (m, k, n or the gathered column count >= 2^31),
  * SPG_OUT_OF_MEMORY, SPG_CUDA_ERROR.  On error *out is NULL.
+ * The library keeps the page-locked words and events of destroyed plans for
+ * later ones: at most 16 sets of about 9 KB of host memory and 18 events, for
+ * the life of the process, each used by one plan at a time.  They belong to the
+ * CUDA context they were made in: after a cudaDeviceReset new ones are made (a
+ * plan itself does not outlive the reset).
  */
 spg_status spgemm_plan(const spg_csc *A, const spg_csc *B, const spg_options *opt, spg_plan **out);
 

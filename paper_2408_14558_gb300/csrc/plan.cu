@@ -18,7 +18,6 @@
 #include <algorithm>
 #include <cstdarg>
 #include <cstring>
-#include <mutex>
 #include <new>
 
 #include "spg_internal.cuh"
@@ -920,91 +919,24 @@ __global__ void k_split(const int64_t *At_colptr, const int32_t *At_row, int64_t
 
 // ------------------------------------------------------------------ host
 
-// A plan's page-locked words and its 18 events, kept for the next plan:
-// creating and destroying them took about 80 us a plan, a fifth of a small
-// multiply.  A kit is handed out to one plan at a time, under a lock, and comes
-// back once that plan's stream is idle; at most kMaxKits wait (about 9 KB each),
-// the others are destroyed.  Plans of more than kKitBlocks blocks get page-locked
-// words of their own size.
+// The plans' page-locked words and events (plan_kits.cuh): words for
+// kKitBlocks blocks are kept, plans of more get words of their own size.
 namespace {
-struct Kit {
-    int dev;
-    int64_t *pinned;
-    size_t words;
-    cudaEvent_t ev[8], kev[10];
-};
-constexpr size_t kMaxKits = 16;
 constexpr int kKitBlocks = 1024;
-std::mutex g_kits_lock;
-std::vector<Kit> &kits() {
-    static std::vector<Kit> *v = new std::vector<Kit>();  // (never destroyed: the driver may be gone by then)
+PlanKits &kits() {
+    // (never destroyed: the driver may be gone by then)
+    static PlanKits *v = new PlanKits(kPinnedBlocks + (size_t)kKitBlocks + 1);
     return *v;
 }
 
-void destroy_kit(Kit &k) {
-    for (cudaEvent_t e : k.ev)
-        if (e) cudaEventDestroy(e);
-    for (cudaEvent_t e : k.kev)
-        if (e) cudaEventDestroy(e);
-    if (k.pinned) cudaFreeHost(k.pinned);
-}
-
 spg_status take_kit(spg_plan *p) {
-    const size_t words = kPinnedBlocks + (size_t)std::max(p->P, kKitBlocks) + 1;
-    Kit k{};
-    bool found = false;
-    {
-        std::lock_guard<std::mutex> hold(g_kits_lock);
-        for (size_t i = 0; i < kits().size() && !found; i++)
-            if (kits()[i].dev == p->dev && kits()[i].words >= words) {
-                k = kits()[i];
-                kits()[i] = kits().back();
-                kits().pop_back();
-                found = true;
-            }
-    }
-    spg_status s = SPG_OK;
-    if (!found) {
-        k.dev = p->dev;
-        k.words = words;
-        s = cuda_check(cudaMallocHost(&k.pinned, sizeof(int64_t) * words), "cudaMallocHost");
-        for (auto &e : k.ev)
-            if (!s) s = cuda_check(cudaEventCreate(&e), "event");
-        for (auto &e : k.kev)
-            if (!s) s = cuda_check(cudaEventCreate(&e), "event");
-        if (s) {
-            const std::string keep = g_last_error;
-            destroy_kit(k);
-            g_last_error = keep;
-            return s;
-        }
-    }
-    p->h_pinned = k.pinned;
-    p->pinned_words = k.words;
-    std::copy(k.ev, k.ev + 8, p->ev);
-    std::copy(k.kev, k.kev + 10, p->kev);
+    p->ctx = context_id();
+    const spg_status s = cuda_check(kits().take(p->ctx, kPinnedBlocks + (size_t)p->P + 1, &p->kit), "plan words and events");
+    if (s) return s;
+    p->h_pinned = p->kit.pinned;
+    std::copy(p->kit.ev, p->kit.ev + 8, p->ev);
+    std::copy(p->kit.kev, p->kit.kev + 10, p->kev);
     return SPG_OK;
-}
-
-// The plan's stream must be idle.
-void give_kit(spg_plan *p) {
-    if (!p->h_pinned) return;
-    Kit k{};
-    k.dev = p->dev;
-    k.pinned = p->h_pinned;
-    k.words = p->pinned_words;
-    std::copy(p->ev, p->ev + 8, k.ev);
-    std::copy(p->kev, p->kev + 10, k.kev);
-    p->h_pinned = nullptr;
-    bool kept = false;
-    if (k.words == kPinnedBlocks + (size_t)kKitBlocks + 1) {
-        std::lock_guard<std::mutex> hold(g_kits_lock);
-        if (kits().size() < kMaxKits) {
-            kits().push_back(k);
-            kept = true;
-        }
-    }
-    if (!kept) destroy_kit(k);
 }
 }  // namespace
 
@@ -1462,11 +1394,11 @@ extern "C" spg_status spgemm_plan(const spg_csc *A, const spg_csc *B, const spg_
 
 extern "C" spg_status spgemm_plan_destroy(spg_plan *p) {
     if (!p) return SPG_OK;
-    cudaStreamSynchronize(p->st);
+    const bool idle = cudaStreamSynchronize(p->st) == cudaSuccess;
     if (p->graph_exec) cudaGraphExecDestroy(p->graph_exec);
     if (p->graph) cudaGraphDestroy(p->graph);
     ws_free_all(p);
-    give_kit(p);
+    kits().give(p->kit, idle, context_id());
     delete p;
     return SPG_OK;
 }

@@ -27,6 +27,7 @@
 
 #include <nvtx3/nvToolsExt.h>
 
+#include "plan_kits.cuh"
 #include "spgemm1d.h"
 
 namespace spg {
@@ -160,14 +161,15 @@ struct spg_plan {
 
     spg_stats stats{};
     // ev[0..1] plan, ev[2..3] symbolic, ev[4..5] numeric; kev[2g], kev[2g+1]
-    // bracket kernel group g (see KernelGroup).  They and h_pinned come from a
-    // pool (plan.cu, take_kit) and may hold an earlier plan's records:
+    // bracket kernel group g (see KernelGroup).  They and h_pinned belong to the
+    // plan's kit (plan_kits.cuh) and may hold an earlier plan's records:
     // kev_used and ev_numeric tell which this plan has made.
     cudaEvent_t ev[8] = {nullptr};
     cudaEvent_t kev[10] = {nullptr};
     bool kev_used[5] = {false, false, false, false, false};
     bool ev_numeric = false;
-    size_t pinned_words = 0;
+    spg::PlanKit kit;
+    unsigned long long ctx = 0;  // the context that the plan was made in
     int dev = -1;
     int64_t launches = 0;
 };
@@ -175,18 +177,20 @@ struct spg_plan {
 namespace spg {
 
 // Resident CTAs per SM of a kernel whose shared memory never changes, asked
-// once per device (the two calls take 3 us, a plan has up to twelve such
-// launches); `tag` makes one cache per kernel.
+// once per context (the two calls take 3 us, a plan has up to twelve such
+// launches; a context that a cudaDeviceReset has made anew has lost the
+// attribute); `tag` makes one cache per kernel.
 template <typename Tag, typename Kern>
 inline int resident_ctas(spg_plan *p, Kern kern, int threads, size_t smem) {
-    static std::atomic<int> cached[16];
-    std::atomic<int> *slot = p->dev >= 0 && p->dev < 16 ? cached + p->dev : nullptr;
-    int occ = slot ? slot->load(std::memory_order_relaxed) : 0;
-    if (occ > 0) return occ;
+    static std::atomic<unsigned long long> cached[16];  // per device: context id * 64 + CTAs
+    std::atomic<unsigned long long> *slot = p->ctx && p->dev >= 0 && p->dev < 16 ? cached + p->dev : nullptr;
+    const unsigned long long have = slot ? slot->load(std::memory_order_relaxed) : 0;
+    if (have && have / 64 == p->ctx) return (int)(have % 64);
+    int occ = 0;
     cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kern, threads, smem);
     if (occ < 1) return 1;
-    if (slot) slot->store(occ, std::memory_order_relaxed);
+    if (slot && occ < 64) slot->store(p->ctx * 64 + (unsigned long long)occ, std::memory_order_relaxed);
     return occ;
 }
 
