@@ -374,21 +374,19 @@ static spg_status numeric_typed(spg_plan *p, spg_csc *C) {
     return s;
 }
 
-// The light columns' numeric bins (by their exact counts), once per plan:
-// launched by the symbolic pass, whose read-back brings their sizes.
+// The light columns' numeric bins (by their exact counts): launched by the
+// symbolic pass, whose read-back brings their sizes; a symbolic pass that is
+// called again after a failed one makes them anew.
 spg_status queue_numeric_bins(spg_plan *p) {
     const int64_t n = p->n;
-    if (p->nbinlist || n == 0) return SPG_OK;
+    if (n == 0) return SPG_OK;
     int8_t *bn = (int8_t *)ws_alloc(p, (size_t)(n + 1));
-    p->nbinlist = (int32_t *)ws_alloc(p, sizeof(int32_t) * (size_t)(n + 1));
+    if (!p->nbinlist) p->nbinlist = (int32_t *)ws_alloc(p, sizeof(int32_t) * (size_t)(n + 1));
     if (!bn || !p->nbinlist) return SPG_OUT_OF_MEMORY;
-    const spg_status s = bin_columns_queue(p, bn, p->nbinlist, 2);
-    p->nbins_queued = s == SPG_OK;
-    return s;
+    return bin_columns_queue(p, bn, p->nbinlist, 2);
 }
 void read_numeric_bins(spg_plan *p) {
-    if (p->nbins_queued) bin_offsets(p, p->nbin_off);
-    p->nbins_queued = false;
+    if (p->n > 0) bin_offsets(p, p->nbin_off);
 }
 
 spg_status run_numeric(spg_plan *p, spg_csc *C) {

@@ -157,7 +157,6 @@ struct spg_plan {
     cudaGraph_t graph = nullptr;     // captured refresh + numeric (spgemm_plan_capture)
     cudaGraphExec_t graph_exec = nullptr;
     int64_t nbin_off[spg::kNumBins + 1] = {0};
-    bool nbins_queued = false;       // their read-back is on the stream
 
     spg_stats stats{};
     // ev[0..1] plan, ev[2..3] symbolic, ev[4..5] numeric; kev[2g], kev[2g+1]
