@@ -74,19 +74,19 @@ constexpr int kSlotTries = 1 << 22;  // bound of one lane's retries
 __device__ __forceinline__ uint32_t shared_addr(const void *p) { return (uint32_t)__cvta_generic_to_shared(p); }
 __device__ __forceinline__ unsigned long long shared_exch64(uint32_t addr, unsigned long long v) {
     unsigned long long o;
-    asm volatile("atom.shared.exch.b64 %0, [%1], %2;" : "=l"(o) : "r"(addr), "l"(v));
+    asm volatile("atom.shared.exch.b64 %0, [%1], %2;" : "=l"(o) : "r"(addr), "l"(v) : "memory");
     return o;
 }
 __device__ __forceinline__ void shared_st64(uint32_t addr, double v) {
-    asm volatile("st.volatile.shared.f64 [%0], %1;" ::"r"(addr), "d"(v));
+    asm volatile("st.volatile.shared.f64 [%0], %1;" ::"r"(addr), "d"(v) : "memory");
 }
 __device__ __forceinline__ uint32_t shared_add32(uint32_t addr, uint32_t v) {
     uint32_t o;
-    asm volatile("atom.shared.add.u32 %0, [%1], %2;" : "=r"(o) : "r"(addr), "r"(v));
+    asm volatile("atom.shared.add.u32 %0, [%1], %2;" : "=r"(o) : "r"(addr), "r"(v) : "memory");
     return o;
 }
 __device__ __forceinline__ void shared_red32(uint32_t addr, uint32_t v) {
-    asm volatile("red.shared.add.u32 [%0], %1;" ::"r"(addr), "r"(v));
+    asm volatile("red.shared.add.u32 [%0], %1;" ::"r"(addr), "r"(v) : "memory");
 }
 
 
