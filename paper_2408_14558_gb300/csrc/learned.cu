@@ -857,10 +857,10 @@ static spg_status launch_light_learned(spg_plan *p, const int32_t *list, int64_t
     return cuda_check(cudaGetLastError(), "learned light");
 }
 
-// Groups of heavy columns in the pipelined assembly (pinned read-back slots
-// 24 .. 24 + 2 * (groups + 1) of the plan hold their boundaries).
+// Groups of heavy columns in the pipelined assembly (their boundaries are read
+// into the plan's page-locked slots from kPinnedHist on).
 constexpr int64_t kLearnedGroups = 8;
-static_assert(24 + 2 * (kLearnedGroups + 1) <= 63, "pinned slots");
+static_assert(kPinnedHist + 2 * (kLearnedGroups + 1) <= kPinnedBins, "the boundaries end before the bins' slots");
 
 struct LearnedState {
     int64_t *cap = nullptr, *capoff = nullptr, *nnz_light = nullptr, *nnz = nullptr;
@@ -1058,7 +1058,7 @@ static spg_status learned_run(spg_plan *p, const spg_options *opt, spg_csc *C, i
     LTRY(cuda_check(cudaStreamSynchronize(st), "cap"));
     const int64_t totcap = p->h_pinned[16];
     p->stats.learned_capacity = totcap;
-    if (n > 0) LTRY(bin_columns(p, L.lbin, L.llist, L.loff));  // uses pinned slots 0..8
+    if (n > 0) LTRY(bin_columns(p, L.lbin, L.llist, L.loff));  // (through the bins' own slots)
     const size_t idxsz = p->out_idx64 ? 8 : 4;
     L.trow = ws_alloc(p, idxsz * (size_t)(totcap + 1));
     L.tval = ws_alloc(p, 8 * (size_t)(totcap + 1));
@@ -1133,13 +1133,13 @@ static spg_status learned_run(spg_plan *p, const spg_options *opt, spg_csc *C, i
         if (!s) {
             launch(p, k_group_bounds, 1, 64, 0, (const int64_t *)hb_d, G, p->nheavy,
                    (const int32_t *)(p->binlist + p->bin_off[kBinHeavy]), (const int64_t *)L.it_first, n, bnd);
-            s = cuda_check(cudaMemcpyAsync(p->h_pinned + 24, bnd, sizeof(int64_t) * 2 * (size_t)(G + 1),
+            s = cuda_check(cudaMemcpyAsync(p->h_pinned + kPinnedHist, bnd, sizeof(int64_t) * 2 * (size_t)(G + 1),
                                            cudaMemcpyDeviceToHost, st), "groups");
         }
         if (!s) s = cuda_check(cudaStreamSynchronize(st), "groups");
         for (int64_t g = 0; g <= G && !s; g++) {
-            ib[g] = p->h_pinned[24 + 2 * g];
-            cb[g] = p->h_pinned[24 + 2 * g + 1];
+            ib[g] = p->h_pinned[kPinnedHist + 2 * g];
+            cb[g] = p->h_pinned[kPinnedHist + 2 * g + 1];
         }
     } else {
         cb[0] = 0;

@@ -128,7 +128,7 @@ static spg_status dev_err_status(int e, const char *phase) {
     return SPG_OK;
 }
 
-// The error word lands in the last pinned slot, so that it can ride along with
+// The error word has a page-locked slot of its own, so that it can ride along with
 // other read-backs: dev_err_queue, then (once the stream is synchronised)
 // dev_err_read.
 spg_status dev_err_queue(spg_plan *p, const char *phase) {

@@ -244,9 +244,9 @@ spg_status dev_err_read(spg_plan *p, const char *phase);
 void collect_stats(spg_plan *p, spg_stats *st);
 // Slots of plan->h_pinned: the device counters or single sizes from 0, the
 // counts of heavy records and items, the hub histogram, bin offsets, the error
-// word, and from kPinnedBlocks on one value per column block.  (The learned
-// path keeps its own sizes in the histogram's slots, which are read in the
-// plan.)
+// word, and from kPinnedBlocks on one value per column block.  (Once the plan
+// has read them, the learned path reads its sizes into the counters' slots 16 to
+// 21 and its groups' boundaries into the histogram's.)
 constexpr int kPinnedHist = 24, kPinnedBins = 56, kPinnedErr = 66, kPinnedRec = 68, kPinnedBlocks = 72;
 int grid_for(int64_t work, int per_block, int max_blocks);
 
