@@ -1211,11 +1211,12 @@ static spg_status plan_build(spg_plan *p) {
                p->nnzb, p->R, p->sym_max_recs, nslab, nsym, (long long *)(p->d_cnt + kCntNnzBHeavy));
         TRY(scan_exclusive_i64(p, nslab, p->rec_first, p->nheavy));
         TRY(scan_exclusive_i64(p, nsym, sym_first, p->nheavy));
-        TRY(hub_histogram_queue(p));
+        const bool hubs = p->opt.sizing != SPG_SIZING_LEARNED;
+        if (hubs) TRY(hub_histogram_queue(p));
         TRY(cuda_check(cudaMemcpyAsync(p->h_pinned + kPinnedRec, p->rec_first + p->nheavy, sizeof(int64_t), cudaMemcpyDeviceToHost, st), "records"));
         TRY(cuda_check(cudaMemcpyAsync(p->h_pinned + kPinnedRec + 1, sym_first + p->nheavy, sizeof(int64_t), cudaMemcpyDeviceToHost, st), "items"));
         TRY(read_counters());
-        hub_histogram_read(p);
+        if (hubs) hub_histogram_read(p);
         // few products per B entry and slab under a mask: wide items
         p->num_wide = p->omask.bits && p->R <= kNumWideCap &&
                       p->h_pinned[kCntProducts] / p->T < kWideProducts * p->h_pinned[kCntNnzBHeavy];

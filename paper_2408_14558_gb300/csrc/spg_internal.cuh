@@ -119,7 +119,8 @@ struct spg_plan {
     int32_t *binlist = nullptr;
     int64_t bin_off[spg::kNumBins + 1] = {0};
 
-    int64_t hub_hist[32] = {0};  // columns of A by floor(log2(length)) (heavy plans)
+    int64_t hub_hist[32] = {0};  // columns of A by floor(log2(length)) (heavy plans), once hub_known
+    bool hub_known = false;
 
     // heavy bins.  A record is one (heavy column, base slab of R rows) inside
     // the column's row window; the records of a column are consecutive.

@@ -290,7 +290,9 @@ constexpr size_t kHubMaxSmem = size_t(192) << 10;  // bitmap words of one hub (r
 // words of a hub bitmap: every base slab of the heavy items (a multiple of 4)
 static int64_t hub_words(const spg_plan *p) { return (int64_t)p->T * (p->R / 32); }
 
-// Launches only: the histogram rides on the plan's read-back.
+// Launches only: the histogram rides on the plan's read-back (learned sizing has
+// no symbolic pass: its plans leave the histogram to build_hubs, should a caller
+// run one after all).
 spg_status hub_histogram_queue(spg_plan *p) {
     // a hub's bitmap is built in one CTA's shared memory
     if (p->k == 0 || (size_t)hub_words(p) * sizeof(uint32_t) > kHubMaxSmem) return SPG_OK;
@@ -307,6 +309,7 @@ spg_status hub_histogram_queue(spg_plan *p) {
 void hub_histogram_read(spg_plan *p) {
     if (p->k == 0 || (size_t)hub_words(p) * sizeof(uint32_t) > kHubMaxSmem) return;
     for (int b = 0; b < 32; b++) p->hub_hist[b] = p->h_pinned[kPinnedHist + b];
+    p->hub_known = true;
 }
 
 static spg_status build_hubs(spg_plan *p, int32_t **hubidx, uint4 **hubbits, int64_t *Wa4) {
@@ -317,7 +320,13 @@ static spg_status build_hubs(spg_plan *p, int32_t **hubidx, uint4 **hubbits, int
     if (k == 0 || (size_t)Wa * sizeof(uint32_t) > kHubMaxSmem) return SPG_OK;
     cudaStream_t st = p->st;
     const int ap64 = p->A.ptr_type == SPG_IDX_I64;
-    spg_status s;
+    spg_status s = SPG_OK;
+    if (!p->hub_known) {
+        s = hub_histogram_queue(p);
+        if (!s) s = cuda_check(cudaStreamSynchronize(st), "hub histogram");
+        if (s) return s;
+        hub_histogram_read(p);
+    }
     int lg = 0;
     while ((int64_t(1) << lg) < kHubMinDeg) lg++;
     int64_t nh = 0;
