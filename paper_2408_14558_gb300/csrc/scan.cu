@@ -134,40 +134,36 @@ __global__ void __launch_bounds__(kScanThreads)
     }
 }
 
-// The whole scan by one CTA, 8192 elements at a time (7 us each: one such tile
-// costs as much as two launches).
+// The whole scan, of up to kScanOne elements, by one CTA (7 us: as much as two
+// launches, so that a second pass would not pay).
 template <typename T>
 __global__ void __launch_bounds__(1024) k_scan_one(const T in, int64_t n, int64_t *__restrict__ out) {
-    __shared__ long long wsum[2][32];
+    __shared__ long long wsum[32];
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-    long long carry = 0;
-    int flip = 0;
-    for (int64_t base = 0; base < n; base += 1024 * kScanPer, flip ^= 1) {
-        const int64_t my = base + (int64_t)threadIdx.x * kScanPer;
-        long long v[kScanPer], run = 0;
+    const int64_t my = (int64_t)threadIdx.x * kScanPer;
+    long long v[kScanPer], run = 0;
 #pragma unroll
-        for (int i = 0; i < kScanPer; i++) {
-            v[i] = my + i < n ? in(my + i) : 0;
-            run += v[i];
-        }
-        long long incl = run;
-#pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-            const long long t = __shfl_up_sync(kFull, incl, o);
-            if (lane >= o) incl += t;
-        }
-        if (lane == 31) wsum[flip][wid] = incl;
-        __syncthreads();  // (the other half of wsum is free again: every thread has passed this barrier since)
-        const long long w = wsum[flip][lane];
-        long long acc = carry + warp_sum_ll(lane < wid ? w : 0) + incl - run;
-        carry += warp_sum_ll(w);
-#pragma unroll
-        for (int i = 0; i < kScanPer; i++) {
-            if (my + i < n) out[my + i] = acc;
-            acc += v[i];
-        }
+    for (int i = 0; i < kScanPer; i++) {
+        v[i] = my + i < n ? in(my + i) : 0;
+        run += v[i];
     }
-    if (threadIdx.x == 0) out[n] = carry;
+    long long incl = run;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const long long t = __shfl_up_sync(kFull, incl, o);
+        if (lane >= o) incl += t;
+    }
+    if (lane == 31) wsum[wid] = incl;
+    __syncthreads();
+    const long long w = wsum[lane];
+    long long acc = warp_sum_ll(lane < wid ? w : 0) + incl - run;
+    const long long total = warp_sum_ll(w);
+#pragma unroll
+    for (int i = 0; i < kScanPer; i++) {
+        if (my + i < n) out[my + i] = acc;
+        acc += v[i];
+    }
+    if (threadIdx.x == 0) out[n] = total;
 }
 
 template <typename T>
