@@ -271,7 +271,8 @@ spg_status spgemm_plan_export(const spg_plan *plan, int32_t block, void *H_bits,
  * ------------------------------------------------------------------------ */
 typedef struct {
     int32_t task_cols;      /* columns per queue task (>= 1; default 64) */
-    int32_t warps_per_cta;  /* 4 or 8 (default 8) */
+    int32_t warps_per_cta;  /* 4 or 8 (default 8): at most; each table class takes the number from half of it up
+                               that keeps most warps on an SM */
     int64_t timeout_ns;     /* bound of a numeric task's wait (default 2 s) */
     int32_t stall_instance; /* failure test: numeric tasks of this instance wait on a flag nothing sets (-1 = off) */
     int32_t reserved;
@@ -306,7 +307,8 @@ spg_status spgemm_batch_destroy(spg_batch *batch);
  * created or updated) the result is stored under the device name and a
  * signature of the workload and reused without timing next time.
  *   spgemm_batch_autotune: task_cols in {16, 64, 256} x warps_per_cta in
- *     {4, 8}, timed on the first `sample` instances (0 = all).
+ *     {4, 8} (upper bounds, as the option), timed on the first `sample`
+ *     instances (0 = all).
  *   spgemm_autotune: light_max in {256, 512, 1024} x slab_rows in
  *     {2048, 4096, 8192} for the plain path (other fields from `base`).
  * Both synchronise; best_ms (may be NULL) receives the winner's time.

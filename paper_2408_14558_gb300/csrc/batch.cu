@@ -36,6 +36,7 @@
 
 #include "block_ops.cuh"
 #include "cta_products.cuh"
+#include "resident_warps.cuh"
 #include "spg_internal.cuh"
 #include "warp_hash.cuh"
 
@@ -480,28 +481,31 @@ static spg_status batch_launch_class(spg_batch *b, int c, cudaStream_t st) {
     if (nt == 0) return SPG_OK;
     auto kern = k_batch_persistent<LOGS_MAX, Acc, OutIdx>;
     // tables of 6, 12 and 24 KB a warp: from half the asked warps per CTA up, the
-    // number that brings most warps onto an SM (what bounds the kernel: 8
-    // resident warps issue in 20% of the cycles)
+    // number that keeps most warps on an SM, by shared memory and registers (what
+    // bounds the kernel: 8 resident warps issue in 20% of the cycles).  The smallest
+    // class, doubles: 24 warps as CTAs of 8, 25 as CTAs of 5
     constexpr size_t per_warp = sizeof(WarpSeg<Acc>) + WarpTable<Acc>::bytes(LOGS_MAX);
-    int warps = 0, resident = 0;
-    for (int w = b->warps; w >= b->warps / 2; w--) {
-        const size_t cta = per_warp * (size_t)w;
-        const int r = cta > (size_t(227) << 10) ? 0 : w * (int)((size_t(228) << 10) / (cta + 1024));
-        if (r > resident) {
-            resident = r;
-            warps = w;
-        }
-    }
-    const size_t smem = per_warp * (size_t)warps;
-    spg_status s = cuda_check(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem),
+    constexpr size_t kMostShared = size_t(227) << 10;
+    const int fit = (int)std::min<size_t>((size_t)b->warps, kMostShared / per_warp);
+    spg_status s = cuda_check(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                                   (int)(per_warp * (size_t)fit)),
                               "batch smem");
     if (s) return s;
-    int occ = 0;
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kern, warps * 32, smem);
-    if (occ < 1) {
-        set_error("batch kernel does not fit on an SM with %d warps", warps);
+    auto ctas = [&](int w) {
+        int n = 0;
+        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, kern, w * 32, per_warp * (size_t)w) != cudaSuccess) {
+            cudaGetLastError();
+            n = 0;
+        }
+        return n;
+    };
+    const int warps = most_resident_warps(b->warps / 2, fit, ctas);
+    if (warps == 0) {
+        set_error("batch kernel does not fit on an SM with %d warps", b->warps);
         return SPG_UNSUPPORTED;
     }
+    const int occ = ctas(warps);
+    const size_t smem = per_warp * (size_t)warps;
     const int grid = b->sm_count * occ;
     b->grid = std::max(b->grid, grid);
     b->smem = std::max(b->smem, smem);

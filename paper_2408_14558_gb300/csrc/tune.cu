@@ -1,7 +1,8 @@
 // Autotuner: times candidate configurations on the caller's own inputs and
 // keeps the fastest, cached in a small JSON file keyed by the device name and
 // a signature of the workload (log2 buckets of its sizes).
-//   batched path: task size (columns per queue task) and CTA shape (warps)
+//   batched path: task size (columns per queue task) and CTA shape (the upper
+//                 bound of its warps)
 //   plain path:   light-bin threshold (largest per-column bound handled by the
 //                 warp hash bins) and heavy base-slab rows
 // The cache file is a flat JSON object of objects with numeric fields; the
