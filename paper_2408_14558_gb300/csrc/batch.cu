@@ -218,8 +218,8 @@ __global__ void k_batch_persistent(const BatchInst *__restrict__ insts, const Ba
                 bool full = false;
                 warp_walk<false, 4, Acc>(
                     p0, p1, lane, ws, in.Arow, seg, [](long long) { return Acc(0); },
-                    [&](int r, Acc, Acc, bool ok, auto) {
-                        if (warp_hash_slot(skeys, logS, r, ok) < 0 && ok) full = true;
+                    [&](const auto &r, const auto &, const auto &, const auto &ok, int windows, auto) {
+                        if (!warp_hash_rows(skeys, logS, r, ok, windows)) full = true;
                     });
                 const int cnt = warp_count_keys(skeys, logS, lane);
                 if (__any_sync(kFull, full) && lane == 0) atomicOr(err, kDevErrInternal);
@@ -256,8 +256,8 @@ __global__ void k_batch_persistent(const BatchInst *__restrict__ insts, const Ba
                 warp_walk<true, 4, Acc, HeavyAcc<Acc>::crowds>(
                     p0, p1, lane, ws, in.Arow, seg,
                     [&](long long e) { return bval_load<Acc>(in.Aval, in.vt, e); },
-                    [&](int r, Acc a, Acc b, bool ok, auto crowded) {
-                        if (!tab.template add<decltype(crowded)::value>(acc, r, a, b, ok)) full = true;
+                    [&](const auto &r, const auto &a, const auto &b, auto &ok, int windows, auto crowded) {
+                        if (!tab.template add<decltype(crowded)::value>(acc, r, a, b, ok, windows)) full = true;
                     });
                 __syncwarp();
                 const int nout = tab.compact(acc, lane);

@@ -50,9 +50,9 @@ __global__ void __launch_bounds__(WARPS * 32, LOGS <= 8 ? 8 : 1)
                 }
             },
             [&](long long e) { return __ldg(At_val + e); },
-            [&](int r, Acc a, Acc b, bool ok, auto crowded) {
-                if (mask.bits && ok && !mask_keeps(mask, j, r)) ok = false;
-                if (!tab.template add<decltype(crowded)::value>(acc, r, a, b, ok)) full = true;
+            [&](const auto &r, const auto &a, const auto &b, auto &ok, int windows, auto crowded) {
+                mask_products(mask, j, r, ok);
+                if (!tab.template add<decltype(crowded)::value>(acc, r, a, b, ok, windows)) full = true;
             });
         __syncwarp();
         const int nout = tab.compact(acc, lane);

@@ -205,8 +205,8 @@ __global__ void __launch_bounds__(WARPS * 32) k_small_multiply(SmallArgs a) {
                     }
                 },
                 [](long long) { return Acc(0); },
-                [&](int r, Acc, Acc, bool ok, auto) {
-                    if (warp_hash_slot(keys, lg, r, ok) < 0 && ok) full = true;
+                [&](const auto &r, const auto &, const auto &, const auto &ok, int windows, auto) {
+                    if (!warp_hash_rows(keys, lg, r, ok, windows)) full = true;
                 });
             c = warp_count_keys(keys, lg, lane);
             if (__any_sync(kFull, full) && lane == 0) fail(a.res, SPG_CUDA_ERROR);
@@ -342,8 +342,8 @@ __global__ void __launch_bounds__(WARPS * 32) k_small_multiply(SmallArgs a) {
                 }
             },
             [&](long long e) { return ld_val<Acc>(a.Aval, a.avt, e); },
-            [&](int r, Acc x, Acc y, bool ok, auto crowded) {
-                if (!tab.template add<decltype(crowded)::value>(acc, r, x, y, ok)) full = true;
+            [&](const auto &r, const auto &x, const auto &y, auto &ok, int windows, auto crowded) {
+                if (!tab.template add<decltype(crowded)::value>(acc, r, x, y, ok, windows)) full = true;
             });
         __syncwarp();
         const int nout = tab.compact(acc, lane);

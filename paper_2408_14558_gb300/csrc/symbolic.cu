@@ -39,9 +39,9 @@ __global__ void __launch_bounds__(WARPS * 32)
                 }
             },
             [&](long long) { return 0ll; },
-            [&](int r, long long, long long, bool ok, auto) {
-                if (mask.bits && ok && !mask_keeps(mask, j, r)) ok = false;
-                if (warp_hash_slot(tab, LOGS, r, ok) < 0 && ok) full = true;
+            [&](const auto &r, const auto &, const auto &, auto &ok, int windows, auto) {
+                mask_products(mask, j, r, ok);
+                if (!warp_hash_rows(tab, LOGS, r, ok, windows)) full = true;
             });
         const int cnt = warp_count_keys(tab, LOGS, lane);
         if (__any_sync(kFull, full) && lane == 0) atomicOr(err, kDevErrInternal);

@@ -76,9 +76,7 @@ __device__ __forceinline__ void warp_windows(int total, int first, int lane, con
                 }
             }
         }
-#pragma unroll
-        for (int u = 0; u < U; u++)
-            if (f0 + 32 * u < total) body(r[u], a[u], b[u], ok[u], std::integral_constant<bool, CROWDED>{});
+        body(r, a, b, ok, min(U, (total - f0 + 31) >> 5), std::integral_constant<bool, CROWDED>{});
     }
     __syncwarp();
 }
@@ -89,8 +87,11 @@ __device__ __forceinline__ void warp_windows(int total, int first, int lane, con
 // products of 32 consecutive entries are numbered consecutively; a window of 32
 // products finds its segments from one bit per segment start (an OR over the
 // lanes), so all 32 lanes stay busy however short the segments are.  U windows
-// are located and loaded before any of them is used.  body(r, a, b, ok, crowded)
-// is called by the whole warp, one product per lane where ok.
+// are located and loaded before any of them is used.  body(r, a, b, ok, windows,
+// crowded) is called by the whole warp for a step's windows at once: `windows` of
+// them hold products, one per lane where ok[u].  (Called for every window by
+// itself: 32,000 products of 1000 rows a column 1.05 ms in doubles and 0.95 in int64,
+// 0.95 and 0.83 so; the refresh on a 128^3 grid 0.349 and 0.342 ms.)
 // CROWD: the body has a form for products that crowd on few rows (crowded is a
 // true type); a column of more than 32 entries takes it for 256 entries at a time
 // whose first window of products crowds (fewer entries bring at most as many
@@ -148,7 +149,28 @@ __device__ __forceinline__ int warp_hash_slot(int *keys, int logS, int r, bool o
     return pend ? -1 : (int)h;
 }
 
-// Fill the 2^logS (>= 64) entries of a table, 16-byte aligned, with empty keys.
+// Rows of a step's windows into a table, without values; false if it is full.
+template <int N>
+__device__ __forceinline__ bool warp_hash_rows(int *keys, int logS, const int (&r)[N], const bool (&ok)[N],
+                                               int windows) {
+    bool there = true;
+#pragma unroll
+    for (int u = 0; u < N; u++)
+        if (u < windows && warp_hash_slot(keys, logS, r[u], ok[u]) < 0 && ok[u]) there = false;
+    return there;
+}
+
+// Clear `ok` where an output mask drops the product.
+template <int N>
+__device__ __forceinline__ void mask_products(const OutMask &mask, int j, const int (&r)[N], bool (&ok)[N]) {
+    if (mask.bits) {
+#pragma unroll
+        for (int u = 0; u < N; u++)
+            if (ok[u] && !mask_keeps(mask, j, r[u])) ok[u] = false;
+    }
+}
+
+// Fill the 2^logS (>= 32) entries of a table, 16-byte aligned, with empty keys.
 __device__ __forceinline__ void warp_clear_keys(int *keys, int logS, int lane) {
     int4 *k4 = (int4 *)keys;
     for (int s = lane; s < (1 << logS) / 4; s += 32) k4[s] = make_int4(kEmptyKey, kEmptyKey, kEmptyKey, kEmptyKey);
@@ -263,14 +285,22 @@ struct WarpTable {
         warp_clear_keys(keys(), logS, lane);
         __syncwarp();
     }
-    // body of warp_walk: a product of row r into its slot; false if the table is full
-    template <bool CROWDED>
-    __device__ __forceinline__ bool add(const HeavyAcc<Acc> &acc, int r, Acc a, Acc b, bool ok) const {
-        const int slot = warp_hash_slot(keys(), logS, r, ok);
-        const uint32_t ad[1] = {acc.addr(max(slot, 0))};
-        const Acc x[1] = {a}, y[1] = {b};
-        const bool o[1] = {ok && slot >= 0};
-        return add_to<CROWDED>(acc, ad, x, y, o) && (slot >= 0 || !ok);
+    // body of warp_walk: the products of a step's windows into their slots; false if
+    // the table is full
+    template <bool CROWDED, int N>
+    __device__ __forceinline__ bool add(const HeavyAcc<Acc> &acc, const int (&r)[N], const Acc (&a)[N],
+                                        const Acc (&b)[N], const bool (&ok)[N], int windows) const {
+        bool good = true;
+#pragma unroll
+        for (int u = 0; u < N; u++)
+            if (u < windows) {
+                const int slot = warp_hash_slot(keys(), logS, r[u], ok[u]);
+                const uint32_t ad[1] = {acc.addr(max(slot, 0))};
+                const Acc x[1] = {a[u]}, y[1] = {b[u]};
+                const bool o[1] = {ok[u] && slot >= 0};
+                if (!(add_to<CROWDED>(acc, ad, x, y, o) && (slot >= 0 || !ok[u]))) good = false;
+            }
+        return good;
     }
     // Move the occupied slots' rows and values to the front; returns their
     // number.  (A write never reaches a slot of a later, still unread chunk.)
