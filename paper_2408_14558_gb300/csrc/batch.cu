@@ -210,7 +210,8 @@ __global__ void k_batch_persistent(const BatchInst *__restrict__ insts, const Ba
                 if (heavy_col[colb + j]) continue;  // counted by the heavy kernel
                 const int64_t p0 = ld_ptr(in.Bcp, in.bcp64, j), p1 = ld_ptr(in.Bcp, in.bcp64, j + 1);
                 // twice the class's table, over its values: every column's bound
-                // min(flops, m) is at most a quarter of it
+                // min(flops, m) is at most a quarter of it (measured with
+                // compare-and-swap inserts)
                 constexpr int logS = LOGS_MAX + 1;
                 int *skeys = (int *)area;
                 warp_clear_keys(skeys, logS, lane);
@@ -248,6 +249,7 @@ __global__ void k_batch_persistent(const BatchInst *__restrict__ insts, const Ba
                 const int64_t p0 = ld_ptr(in.Bcp, in.bcp64, j), p1 = ld_ptr(in.Bcp, in.bcp64, j + 1);
                 // >= 4 x the column's count (at most the class's table): a
                 // sparser table probes less, which outweighs clearing more
+                // (measured with compare-and-swap inserts)
                 const WarpTable<Acc> tab(area, min(LOGS_MAX, log_table(want > 0 ? want : 1) + 1));
                 const HeavyAcc<Acc> acc = tab.acc();
                 tab.clear(lane);
@@ -483,7 +485,8 @@ static spg_status batch_launch_class(spg_batch *b, int c, cudaStream_t st) {
     // tables of 6, 12 and 24 KB a warp: from half the asked warps per CTA up, the
     // number that keeps most warps on an SM, by shared memory and registers (what
     // bounds the kernel: 8 resident warps issue in 20% of the cycles).  The smallest
-    // class, doubles: 24 warps as CTAs of 8, 25 as CTAs of 5
+    // class is limited by registers: at 72 a thread 28 warps as CTAs of 7 or 4 but 24
+    // as CTAs of 8, at the 79 of this build 24 either way
     constexpr size_t per_warp = sizeof(WarpSeg<Acc>) + WarpTable<Acc>::bytes(LOGS_MAX);
     constexpr size_t kMostShared = size_t(227) << 10;
     const int fit = (int)std::min<size_t>((size_t)b->warps, kMostShared / per_warp);

@@ -18,9 +18,12 @@
 namespace spg {
 
 // Small tables (up to 256 slots): 32 registers a thread and two windows in
-// flight keep 64 warps on an SM (refresh of A * P_agg on a 128^3 grid: 0.44 ms
-// at 62 registers and four windows, 0.35 so; tables of four times the entries
-// instead of two made no difference).
+// flight keep up to 64 warps on an SM.  Kernel time for 200,003 columns of doubles,
+// so | without the bound and with four windows: 36 products a column (128 slots)
+// 253 | 286 us, 64 products 323 | 356, 100 products (256 slots, of which shared
+// memory holds seven CTAs) 686 | 746; int64 the same within 2%.  Six CTAs of
+// 256-slot tables instead were 4% faster for int64 and 8% slower for doubles.
+// Tables of four times the entries instead of two made no difference.
 template <int LOGS, int WARPS, typename Acc, typename OutIdx>
 __global__ void __launch_bounds__(WARPS * 32, LOGS <= 8 ? 8 : 1)
     k_num_light(const int32_t *__restrict__ list, int64_t ncols, const void *Bcolptr, int p64,
@@ -123,11 +126,11 @@ __global__ void k_num_headers(int64_t nitems, const int32_t *__restrict__ num_re
 // header while the current one is written out.  MASKED: the bitmaps hold only
 // the rows an output mask admits, and a product whose row is absent is dropped
 // (rank items) or accumulated into a slot that is not written (direct items).
-// What bounds it: the shared-memory pipe in the walk (l1tex wavefronts 67% of
-// the whole kernel for int64, 74% for doubles on a 50,000-vertex R-MAT graph,
+// What bounds it: the shared-memory pipe in the walk (l1tex wavefronts 66% of
+// the whole kernel for int64, 73% for doubles on a 50,000-vertex R-MAT graph,
 // of which 8 + 9 a window are the doubles' exchange and store) and, on sparse
 // items, the barriers and latencies between an item's phases (about half of its
-// time; issue slots 52-63% busy).  Measured against the walk that placed every
+// time; issue slots 53-63% busy).  Measured against the walk that placed every
 // window across segments, with 8-byte look-ups and atomicAdd(double): squaring
 // an R-MAT graph of 262,144 vertices in doubles 65.6 -> 49.3 ms, of 100,003 in
 // int64 5.4 -> 4.4 ms, one 25,000-column chunk of the similarity product (dense
@@ -352,7 +355,11 @@ static spg_status numeric_typed(spg_plan *p, spg_csc *C) {
         // per four products of an entry of C); more of them write over a wider
         // range at once, which the link answers with less bandwidth (40,009
         // vertices, 1.6 GB of C, four groups: 15.4 ms at four CTAs per SM,
-        // 14.6 at two, 14.3 at one, 14.8 at 3/4)
+        // 14.6 at two, 14.3 at one, 14.8 at 3/4).  Over eleven products of 5,003
+        // to 100,003 columns with 1 to 4 products an entry, all the CTAs that fit
+        // were 0 to 9% slower (12,011 vertices, four groups: 4.42 -> 4.84 ms), one
+        // per two or eight products the same; at 8.6 products an entry one per
+        // eight was 8% faster (8.54 -> 7.84 ms)
         if (p->c_on_host)
             occ = (int)std::max<int64_t>(1, std::min<int64_t>(occ, p->stats.products / 4 / std::max<int64_t>(p->nnzC, 1)));
         int g = grid_for(p->nnum, 1, p->sm_count * occ);

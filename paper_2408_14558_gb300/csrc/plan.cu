@@ -511,8 +511,9 @@ __global__ void k_gather_copy(const int64_t *__restrict__ At_colptr, const int32
     // lane k holds column s0 + k: its start, and how far A's column begins from
     // there; they serve every step up to entry `lim`, where column s0 + 32
     // begins.  (Loading them anew for every 32 entries, each load waiting for the
-    // step before, took 98 us for 14.6M entries in columns of 7; the refresh that
-    // the copy is part of went from 0.355 to 0.347 ms.)
+    // step before, took 98 us for 14.6M entries in columns of 7; four replays of the
+    // refresh that the copy is part of, with the wait behind them, went from 0.355 to
+    // 0.347 ms each.)
     int64_t s0 = lo, bk = 0, shk = 0, lim = -1;
     for (int64_t f = e0; f < e1; f += 32) {
         if (f + 32 > lim) {

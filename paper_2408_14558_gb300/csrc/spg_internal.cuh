@@ -352,9 +352,13 @@ constexpr int kNumCapMin = SPG_NUM_CAP_MIN;
 // Every item stages all of its column's B' entries, and where an entry brings
 // few products per slab of rows (A's columns are short and the output mask
 // leaves long columns: the betweenness products) that staging is the work.
-// Measured on the betweenness batch of 1024 sources on 65,536 vertices (about 2
-// products per entry and slab): 45.6 ms with 4096-entry items, 42.7 with these;
-// on the squaring of R-MAT graphs (about 20): 60.0 and 63.1 ms.
+// Measured, 4096-entry items | by this rule | always these: betweenness batches of
+// 1024 sources on 65,536 vertices, 32 neighbours 41.7 | 39.6 | 36.2 ms, 8 neighbours
+// 19.6 | 18.6 | 18.7, of 16 sources 16.3 | 15.6 | 14.6; 4096 masked columns of 4000
+// entries that keep 90% of 65,536 rows 4.19 | 3.18 | 3.18, that keep 10% of them 1.66 |
+// 1.81 | 1.81 (a column then fits one 4096-entry item: the rule does not know how many
+// entries the mask leaves).  Without a mask (squaring R-MAT graphs, about 20 products
+// per entry and slab): 60.0 and 63.1 ms.
 constexpr int kNumWideCap = 10240, kWideProducts = 6;
 // C and the heavy bitmaps pass through L2 once; storing (and reading the
 // bitmaps) with the evict-first hint keeps A~, which the products re-read,

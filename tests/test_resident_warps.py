@@ -14,11 +14,11 @@ SOURCE = r"""
 #include <cstdio>
 #include "resident_warps.cuh"
 using spg::most_resident_warps;
-// CTAs of w warps on an SM: 65,536 registers in units of 256 a warp, 228 KB with 1 KB kept per CTA
+// CTAs of w warps on an SM: four partitions of 16,384 registers, 228 KB with 1 KB kept per CTA
 static int sm(int w, int regs, long table) {
     const long smem = table * w;
     if (smem > 227 * 1024) return 0;
-    return (int)std::min<long>(65536 / (((regs + 7) / 8 * 8) * 32 * w), 228 * 1024 / (smem + 1024));
+    return (int)std::min<long>(4 * (16384 / ((regs + 7) / 8 * 8 * 32)) / w, 228 * 1024 / (smem + 1024));
 }
 int main() {
     auto pick = [](int least, int most, int regs, long table) {
@@ -26,7 +26,7 @@ int main() {
     };
     // shared memory alone would keep 32 warps either way: registers decide
     assert(sm(8, 72, 6656) == 3 && sm(4, 72, 6656) == 7 && pick(4, 8, 72, 6656) == 7);
-    assert(sm(8, 80, 6656) == 3 && sm(5, 80, 6656) == 5 && pick(4, 8, 80, 6656) == 5);
+    assert(sm(8, 80, 6656) == 3 && sm(4, 80, 6656) == 6 && pick(4, 8, 80, 6656) == 8);
     assert(pick(2, 4, 72, 6656) == 4);
     // few registers: shared memory decides, and of equal numbers the largest CTA
     assert(pick(4, 8, 32, 6656) == 8 && pick(4, 8, 32, 25088) == 8 && pick(2, 4, 32, 25088) == 3);
