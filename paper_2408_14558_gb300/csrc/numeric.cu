@@ -9,6 +9,7 @@
 //               acc[rank] in shared memory, and the slab is written out in row
 //               order with no sort
 #include <algorithm>
+#include <type_traits>
 
 #include "block_ops.cuh"
 #include "cta_products.cuh"
@@ -18,12 +19,18 @@
 namespace spg {
 
 // Small tables (up to 256 slots): 32 registers a thread and two windows in
-// flight keep up to 64 warps on an SM.  Kernel time for 200,003 columns of doubles,
+// flight (one, see below) keep up to 64 warps on an SM.  Kernel time for 200,003 columns of doubles,
 // so | without the bound and with four windows: 36 products a column (128 slots)
 // 253 | 286 us, 64 products 323 | 356, 100 products (256 slots, of which shared
 // memory holds seven CTAs) 686 | 746; int64 the same within 2%.  Six CTAs of
 // 256-slot tables instead were 4% faster for int64 and 8% slower for doubles.
+// Doubles in 64-slot tables take one window at a time (what two keep in registers
+// spills): 9 products a column 151 -> 142 us, 25 products 189 -> 179, the refresh of
+// A * P_agg on a 128^3 grid 342 -> 332 us; in int64 25 products would take 175 ->
+// 178 us, in 128 slots both are the same, in 256 slots one is 5% slower.
 // Tables of four times the entries instead of two made no difference.
+template <int LOGS, typename Acc>
+constexpr int kLightWindows = LOGS <= 6 && std::is_same<Acc, double>::value ? 1 : LOGS <= 8 ? 2 : 4;
 template <int LOGS, int WARPS, typename Acc, typename OutIdx>
 __global__ void __launch_bounds__(WARPS * 32, LOGS <= 8 ? 8 : 1)
     k_num_light(const int32_t *__restrict__ list, int64_t ncols, const void *Bcolptr, int p64,
@@ -42,7 +49,7 @@ __global__ void __launch_bounds__(WARPS * 32, LOGS <= 8 ? 8 : 1)
         const int64_t base = Ccolptr[j], want = Ccolptr[j + 1] - base;
         tab.clear(lane);
         bool full = false;
-        warp_walk<true, (LOGS <= 8 ? 2 : 4), Acc, HeavyAcc<Acc>::crowds>(
+        warp_walk<true, kLightWindows<LOGS, Acc>, Acc, HeavyAcc<Acc>::crowds>(
             p0, p1, lane, segs[wid], At_row,
             [&](int64_t p, long long &st, int &len, Acc &bv) {
                 int q = Bq[p];

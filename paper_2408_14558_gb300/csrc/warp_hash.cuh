@@ -91,8 +91,7 @@ __device__ __forceinline__ void warp_windows(int total, int first, int lane, con
 // crowded) is called by the whole warp for a step's windows at once: `windows` of
 // them hold products, one per lane where ok[u].  (Called for every window by
 // itself: 32,000 products of 1000 rows a column 1.05 ms in doubles and 0.95 in int64,
-// 0.95 and 0.83 so; four replays of the refresh on a 128^3 grid, with the wait behind
-// them, 0.349 and 0.342 ms each, replays queued one behind the other 0.289 and 0.294.)
+// 0.95 and 0.83 so; columns of few products take the same time.)
 // CROWD: the body has a form for products that crowd on few rows (crowded is a
 // true type); a column of more than 32 entries takes it for 256 entries at a time
 // whose first window of products crowds (fewer entries bring at most as many
